@@ -96,7 +96,7 @@ struct Rows {
 };
 static_assert(kPipeAlignRows % kTileRows == 0, "row chunks must be whole tiles");
 
-int grid_for(const ens_matrix *A, int64_t rows, const void *kernel, int64_t rows_per_block = kTileRows) {
+int grid_for(const ens_matrix *A, int64_t rows, const void *kernel, int64_t rows_per_block) {
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreads, 0);
   if (per_sm < 1) per_sm = 1;
@@ -123,10 +123,10 @@ cudaError_t run(const ens_matrix *A, int m, const void *X, void *Y, uint32_t mas
   }
   if constexpr (capped) {
     auto k = gspmv_kernel_capped<Arith, VEC, LANES>;
-    k<<<grid_for(A, v.n, (const void *)k), kThreads, 0, s>>>(v, m, (const T *)X, y, mask);
+    k<<<grid_for(A, v.n, (const void *)k, tile_rows_for(v.n, LANES)), kThreads, 0, s>>>(v, m, (const T *)X, y, mask);
   } else {
     auto k = gspmv_kernel<Arith, VEC, LANES>;
-    k<<<grid_for(A, v.n, (const void *)k), kThreads, 0, s>>>(v, m, (const T *)X, y, mask);
+    k<<<grid_for(A, v.n, (const void *)k, tile_rows_for(v.n, LANES)), kThreads, 0, s>>>(v, m, (const T *)X, y, mask);
   }
   return cudaGetLastError();
 }

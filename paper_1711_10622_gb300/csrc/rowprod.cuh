@@ -514,6 +514,15 @@ __device__ __forceinline__ void row_split_pairs(int32_t j0, int32_t j1, const in
 // ------------------------------------------------------------------ row tiles (shared memory)
 constexpr int kTileRows = 256;
 constexpr int kTileNnz = 2048;
+// Rows of one tile for a product of n rows with `lanes` threads per row: kTileRows, halved while the
+// tiles are fewer than two per SM (152 SMs) and a tile still holds one row per row group. 32^3 rows in
+// tiles of 256 rows are 128 blocks and leave SMs idle (with the grids of the solver limited to the tiles and its
+// per-column scalars formed once, a plain 32^3, m = 4 solve takes 7.4 ms against 12.4).
+__host__ __device__ constexpr int tile_rows_for(int64_t n, int lanes) {
+  int r = kTileRows;
+  while (r > 256 / lanes && (n + r - 1) / r < 304) r >>= 1;
+  return r;
+}
 constexpr int kCsrPad = 4;  // extra elements allocated after row_ptr, col_idx and every value array
 
 template <typename V>
@@ -718,7 +727,7 @@ struct ArithF64Hybrid {
   __device__ __forceinline__ static double dinv(const MatView &A, int64_t i) { return __ldg(A.dinv + i); }
 };
 
-// A block walks tiles of kTileRows consecutive rows (grid-stride). For each tile it stages the
+// A block walks tiles of tile_rows_for() consecutive rows (grid-stride). For each tile it stages the
 // row pointers and the tile's contiguous CSR segment (column indices and values) in shared
 // memory with 16-byte coalesced loads (the arrays are padded so the rounded-out segment stays
 // inside them), then each row group of LANES threads computes rows g, g + G, g + 2G, ... of the
@@ -733,10 +742,10 @@ struct ArithF64Hybrid {
 template <int VEC, int LANES, typename Fn>
 __device__ __forceinline__ void tile_order_rows(int64_t n, int32_t m, Fn &&fn) {
   constexpr int G = 256 / LANES;
-  constexpr int RPG = kTileRows / G;
+  const int R = tile_rows_for(n, LANES), RPG = R / G;
   const int lane = threadIdx.x % LANES, grp = threadIdx.x / LANES;
-  for (int64_t r0 = (int64_t)blockIdx.x * kTileRows; r0 < n; r0 += (int64_t)gridDim.x * kTileRows) {
-    const int rows = (int)min((int64_t)kTileRows, n - r0);
+  for (int64_t r0 = (int64_t)blockIdx.x * R; r0 < n; r0 += (int64_t)gridDim.x * R) {
+    const int rows = (int)min((int64_t)R, n - r0);
     for (int rr = 0; rr < RPG; ++rr) {
       const int lr = rr * G + grp;
       if (lr >= rows) break;
@@ -751,7 +760,7 @@ __device__ __forceinline__ void tile_rows(const MatView &A, int32_t m, const typ
   using T = typename Arith::T;
   constexpr int kThr = 256;
   constexpr int G = kThr / LANES;
-  constexpr int RPG = kTileRows / G;
+  const int R = tile_rows_for(A.n, LANES), RPG = R / G;
   // Row pointers of the current tile and of the next one: the next tile's are copied asynchronously
   // while the current tile is computed, so each tile waits for one memory round trip (its CSR
   // segment) instead of two (row pointers, then the segment they delimit). Measured on GB300:
@@ -762,13 +771,13 @@ __device__ __forceinline__ void tile_rows(const MatView &A, int32_t m, const typ
   __shared__ __align__(16) typename Arith::Tile sm;
   __shared__ __align__(16) int32_t rpb[kPrefetch ? 2 : 1][kTileRows + 4];
   const int lane = threadIdx.x % LANES, grp = threadIdx.x / LANES;
-  int64_t r0 = (int64_t)blockIdx.x * kTileRows;
+  int64_t r0 = (int64_t)blockIdx.x * R;
   if constexpr (kPrefetch) {
-    if (r0 < A.n) stage16<int32_t>(rpb[0], A.rp + r0, ((int)min((int64_t)kTileRows, (int64_t)A.n - r0) + 1 + 3) & ~3);
+    if (r0 < A.n) stage16<int32_t>(rpb[0], A.rp + r0, ((int)min((int64_t)R, (int64_t)A.n - r0) + 1 + 3) & ~3);
     __syncthreads();
   }
-  for (int cur = 0; r0 < A.n; r0 += (int64_t)gridDim.x * kTileRows, cur ^= kPrefetch ? 1 : 0) {
-    const int rows = (int)min((int64_t)kTileRows, (int64_t)A.n - r0);
+  for (int cur = 0; r0 < A.n; r0 += (int64_t)gridDim.x * R, cur ^= kPrefetch ? 1 : 0) {
+    const int rows = (int)min((int64_t)R, (int64_t)A.n - r0);
     const int32_t *rp = rpb[cur];
     if constexpr (!kPrefetch) {
       stage16<int32_t>(rpb[0], A.rp + r0, (rows + 1 + 3) & ~3);
@@ -778,9 +787,9 @@ __device__ __forceinline__ void tile_rows(const MatView &A, int32_t m, const typ
     const bool staged = ae - ab <= kTileNnz;
     if (staged) Arith::stage(sm, A, ab, ae);
     if constexpr (kPrefetch) {
-      const int64_t r1 = r0 + (int64_t)gridDim.x * kTileRows;
+      const int64_t r1 = r0 + (int64_t)gridDim.x * R;
       if (r1 < A.n) {
-        stage16_async<int32_t>(rpb[cur ^ 1], A.rp + r1, ((int)min((int64_t)kTileRows, (int64_t)A.n - r1) + 1 + 3) & ~3);
+        stage16_async<int32_t>(rpb[cur ^ 1], A.rp + r1, ((int)min((int64_t)R, (int64_t)A.n - r1) + 1 + 3) & ~3);
         cp_async_commit();
       }
     }
@@ -788,7 +797,7 @@ __device__ __forceinline__ void tile_rows(const MatView &A, int32_t m, const typ
     // sweep counter: spreads native_mask over tiles; the per-warp rotation keeps warps of one SM in
     // different phases so the FP64 pipe (native sweeps) and the FP32/integer pipes (split sweeps)
     // work at the same time
-    const uint32_t sweep0 = (uint32_t)(r0 / kTileRows) * RPG + (threadIdx.x >> 5) * 5u + blockIdx.x;
+    const uint32_t sweep0 = (uint32_t)(r0 / R) * RPG + (threadIdx.x >> 5) * 5u + blockIdx.x;
     if (staged) {
 #pragma unroll 1
       for (int rr = 0; rr < RPG; ++rr) {

@@ -45,7 +45,11 @@ enum : int32_t { FL_EARLY = 1, FL_ZERO_B = 2, FL_NOSTEP = 4 };
 
 template <typename T>
 struct Cols {
-  T *rho, *rho_old, *alpha, *omega, *bn2, *thr2, *rh2, *rn2, *tol, *mean;
+  // beta = (rho / rho_old) (alpha / omega) of the iteration that begins; rn, rn_inv = ||r|| and 1 / ||r|| of
+  // the refinement loop. The last block of a reduction forms them once per column: a division or root in
+  // every thread of the kernels that use them cost more FP64 pipe time than their updates (k_p on 32^3
+  // rows, m = 4: 12.8 us before).
+  T *rho, *beta, *alpha, *omega, *bn2, *thr2, *rh2, *rn2, *rn, *rn_inv, *tol, *mean;
   int32_t *state, *iters, *status, *flags;
   double *relres;
   int32_t *it;  // [2]: iterations completed, "go" flag (some column active and it < max_iter)
@@ -158,9 +162,11 @@ __global__ void ENS_TILE_BOUNDS(Arith)
     cs.rn2[l] = rn2;
     cs.rh2[l] = rn2;
     cs.rho[l] = rn2;  // rhat = r0, so rho_1 = (rhat, r0) = ||r0||^2
-    cs.rho_old[l] = T(1);
+    cs.beta[l] = rn2;  // rho / 1 * (1 / 1); p = v = 0 here
     cs.alpha[l] = T(1);
     cs.omega[l] = T(1);
+    cs.rn[l] = sqrt(rn2);
+    cs.rn_inv[l] = rsqrt(rn2);
     cs.state[l] = st;
     cs.status[l] = status;
     cs.flags[l] = fl;
@@ -190,7 +196,7 @@ __global__ void __launch_bounds__(kThreads)
   for (int q = 0; q < VEC; ++q) {
     const int l = c + q;
     act[q] = cs.state[l] == ST_ACTIVE;
-    beta[q] = act[q] ? (cs.rho[l] / cs.rho_old[l]) * (cs.alpha[l] / cs.omega[l]) : T(0);
+    beta[q] = act[q] ? cs.beta[l] : T(0);
     om[q] = act[q] ? cs.omega[l] : T(0);
   }
   ENS_ROWS(i) {
@@ -368,13 +374,20 @@ __global__ void ENS_TILE_BOUNDS(Arith)
 }
 
 // ----------------------------------------------------------------------------- x, r update
+// Condition of the device-driven iteration loop (a conditional WHILE graph node): k_xr, which ends an
+// iteration, sets it with the "go" flag (a kernel of its own for it cost a launch per iteration). set = false
+// in the host-driven loop.
+struct LoopCond {
+  cudaGraphConditionalHandle h;
+  bool set;
+};
 template <typename Arith, int VEC, int LANES>
 __global__ void __launch_bounds__(kThreads)
     k_xr(MatView A, int32_t m, typename Arith::T *x, const typename Arith::T *__restrict__ ph,
          const typename Arith::T *__restrict__ sh, const typename Arith::T *__restrict__ s,
          const typename Arith::T *__restrict__ t, typename Arith::T *__restrict__ r,
          const typename Arith::T *__restrict__ rh, int32_t max_iter, Cols<typename Arith::T> cs,
-         typename Arith::T *partials, unsigned *counter) {
+         typename Arith::T *partials, unsigned *counter, LoopCond loop) {
   using T = typename Arith::T;
   const int32_t c = (threadIdx.x % LANES) * VEC;
   T acc[2][VEC], al[VEC], om[VEC];
@@ -418,7 +431,6 @@ __global__ void __launch_bounds__(kThreads)
     }
     if (st != ST_ACTIVE) return;
     const T rn2 = tt.v[0][l], rr = tt.v[1][l];
-    cs.rho_old[l] = cs.rho[l];
     cs.rn2[l] = rn2;
     if (!isfinite(rn2)) {
       cs.state[l] = ST_DONE;
@@ -439,6 +451,7 @@ __global__ void __launch_bounds__(kThreads)
         cs.status[l] = ENS_COL_BREAKDOWN;
         cs.iters[l] = it + 1;
       } else {
+        cs.beta[l] = (rr / cs.rho[l]) * (cs.alpha[l] / cs.omega[l]);
         cs.rho[l] = rr;
       }
     }
@@ -446,13 +459,10 @@ __global__ void __launch_bounds__(kThreads)
     int32_t any = 0;
     for (int l = 0; l < m; ++l) any |= cs.state[l] != ST_DONE;
     cs.it[0] = it;
-    cs.it[1] = any && it < max_iter;
+    const bool go = any && it < max_iter;
+    cs.it[1] = go;
+    if (loop.set) cudaGraphSetConditional(loop.h, go ? 1u : 0u);
   });
-}
-
-// Loop condition of the device-driven iteration graph (a conditional WHILE node).
-static __global__ void k_loop_cond(cudaGraphConditionalHandle h, const int32_t *__restrict__ it) {
-  if (threadIdx.x == 0) cudaGraphSetConditional(h, it[1] ? 1u : 0u);
 }
 
 // ----------------------------------------------------------------------------- finishing
@@ -528,6 +538,8 @@ __global__ void ENS_TILE_BOUNDS(Arith)
     if (outer) {
       if (cs.state[l] != ST_ACTIVE) return;
       cs.rn2[l] = rr;
+      cs.rn[l] = sqrt(rr);
+      cs.rn_inv[l] = rsqrt(rr);
       if (!isfinite(rr)) {
         cs.state[l] = ST_DONE;
         cs.status[l] = ENS_COL_NONFINITE;
@@ -552,7 +564,7 @@ __global__ void __launch_bounds__(kThreads)
   if (c >= m) return;
   double sc[VEC];
 #pragma unroll
-  for (int q = 0; q < VEC; ++q) sc[q] = cs.state[c + q] == ST_ACTIVE ? rsqrt(cs.rn2[c + q]) : 0.0;
+  for (int q = 0; q < VEC; ++q) sc[q] = cs.state[c + q] == ST_ACTIVE ? cs.rn_inv[c + q] : 0.0;
   for (int64_t i = (int64_t)blockIdx.x * (kThreads / LANES) + threadIdx.x / LANES; i < n;
        i += (int64_t)gridDim.x * (kThreads / LANES)) {
     double rv[VEC];
@@ -587,7 +599,7 @@ __global__ void __launch_bounds__(kThreads)
   double sc[VEC];
 #pragma unroll
   for (int q = 0; q < VEC; ++q)  // an inner solve that met a non-finite value contributes nothing
-    sc[q] = cs.state[c + q] == ST_ACTIVE && inner_status[c + q] != ENS_COL_NONFINITE ? sqrt(cs.rn2[c + q]) : 0.0;
+    sc[q] = cs.state[c + q] == ST_ACTIVE && inner_status[c + q] != ENS_COL_NONFINITE ? cs.rn[c + q] : 0.0;
   for (int64_t i = (int64_t)blockIdx.x * (kThreads / LANES) + threadIdx.x / LANES; i < n;
        i += (int64_t)gridDim.x * (kThreads / LANES)) {
     double xv[VEC];
@@ -685,6 +697,9 @@ struct Scratch {
   }
 };
 
+// Tiles of a product of n rows with `lanes` threads per row.
+inline int64_t tile_count(int64_t n, int lanes) { return (n + tile_rows_for(n, lanes) - 1) / tile_rows_for(n, lanes); }
+
 inline MatView view_of(const ens_matrix *A) {
   return MatView{(int32_t)A->n, A->row, A->col, A->val, A->val32, A->valsplit, A->dinv, A->dinv32};
 }
@@ -692,7 +707,7 @@ inline MatView view_of(const ens_matrix *A) {
 template <typename T>
 cudaError_t alloc_cols(Scratch &sc, int m, Cols<T> &cs) {
   cudaError_t e = cudaSuccess;
-  T **tp[] = {&cs.rho, &cs.rho_old, &cs.alpha, &cs.omega, &cs.bn2, &cs.thr2, &cs.rh2, &cs.rn2, &cs.tol, &cs.mean};
+  T **tp[] = {&cs.rho, &cs.beta, &cs.alpha, &cs.omega, &cs.bn2, &cs.thr2, &cs.rh2, &cs.rn2, &cs.rn, &cs.rn_inv, &cs.tol, &cs.mean};
   for (T **p : tp)
     if (e == cudaSuccess) e = sc.get(p, m);
   int32_t **ip[] = {&cs.state, &cs.iters, &cs.status, &cs.flags};
@@ -938,7 +953,7 @@ struct AmgCycle {
       }
       const int64_t rows_per_block = kThreads / lanes;
       const int64_t sms = h.A->num_sms;
-      L.grid = (int)std::max<int64_t>(1, std::min<int64_t>((L.n + kTileRows - 1) / kTileRows, sms * LightBlocks<Arith>::value));
+      L.grid = (int)std::max<int64_t>(1, std::min<int64_t>(tile_count(L.n, lanes), sms * LightBlocks<Arith>::value));
       L.sms = (int)sms;
       L.egrid = (int)std::max<int64_t>(1, std::min<int64_t>((L.n + rows_per_block - 1) / rows_per_block, sms * 8));
       L.cgrid = (int)std::max<int64_t>(1, std::min<int64_t>((L.nc + rows_per_block - 1) / rows_per_block, sms * 8));
@@ -973,7 +988,7 @@ struct AmgCycle {
       }
       if constexpr (std::is_same<Ar, ArithF64Split>::value && V == 2 && Ln >= 2) {
         if (mp % 4 == 0 && launch_amg_smooth2_4_split(Ln / 2, add, L.As, L.A, mp, src, z, it, c1, c2, L.as_mask, L.sms,
-                                                      (L.n + kTileRows - 1) / kTileRows, st))
+                                                      tile_count(L.n, Ln / 2), st))
           return;
       }
       if (add)
@@ -997,7 +1012,7 @@ struct AmgCycle {
       if constexpr (std::is_same<Ar, ArithF64Split>::value && V == 2 && Ln >= 2) {
         if (mp % 4 == 0)
           done = launch_cheb4_split(Ln / 2, first, last, L.A, mp, din, dout, src, L.cres, z, c1, c2, L.mask, L.sms,
-                                    (L.n + kTileRows - 1) / kTileRows, st);
+                                    tile_count(L.n, Ln / 2), st);
       }
       if (done)
         ;
@@ -1019,7 +1034,7 @@ struct AmgCycle {
   void resid(const Level &L, const T *z, const T *r, cudaStream_t st) {
     if constexpr (std::is_same<Ar, ArithF64Split>::value && V == 2 && Ln >= 2) {
       if (mp % 4 == 0 &&
-          launch_amg_resid4_split(Ln / 2, L.A, mp, z, r, L.res, L.mask, L.sms, (L.n + kTileRows - 1) / kTileRows, st))
+          launch_amg_resid4_split(Ln / 2, L.A, mp, z, r, L.res, L.mask, L.sms, tile_count(L.n, Ln / 2), st))
         return;
     }
     k_amg_resid<Ar, V, Ln><<<L.grid, kThreads, 0, st>>>(L.A, mp, z, r, L.res, L.mask);
@@ -1113,9 +1128,11 @@ struct Bicg {
     lanes = 1;
     while (lanes * vec < mp) lanes <<= 1;
     num_sms = M->num_sms;
-    grid = M->num_sms * 4;
-    tgrid = M->num_sms * TileBlocks<Arith>::value;
-    lgrid = M->num_sms * LightBlocks<Arith>::value;
+    // no more blocks than the rows fill: an idle block of a reduction still adds its zeros and its partial
+    const int64_t tiles = tile_count(n, lanes), need = (n * lanes + kThreads - 1) / kThreads;
+    grid = (int)std::min<int64_t>((int64_t)M->num_sms * 4, need);
+    tgrid = (int)std::min<int64_t>((int64_t)M->num_sms * TileBlocks<Arith>::value, tiles);
+    lgrid = (int)std::min<int64_t>((int64_t)M->num_sms * LightBlocks<Arith>::value, tiles);
     prec = o.precond == ENS_PRECOND_CHEBYSHEV;
     cheb_steps = o.cheb_steps;
     theta = 0.5 * (o.cheb_hi + o.cheb_lo);
@@ -1193,7 +1210,7 @@ struct Bicg {
       if constexpr (std::is_same<Arith, ArithF64Split>::value && V == 2 && L >= 2) {
         if (mp % 4 == 0)
           done = launch_cheb4_split(L / 2, first, last, A, mp, din, dout, src, res, z, c1, c2, mask, num_sms,
-                                    INT64_MAX, st);
+                                    tile_count(n, L / 2), st);
       }
       if (done)
         ;
@@ -1212,7 +1229,7 @@ struct Bicg {
 
   // One BiCGStab iteration for every column (frozen columns are no-ops); the iteration number
   // lives on the device, so the same launches can be captured once and replayed.
-  cudaError_t iteration(T *x, int max_iter, cudaStream_t st) {
+  cudaError_t iteration(T *x, int max_iter, cudaStream_t st, LoopCond lc = LoopCond{}) {
     const T inv_theta = (T)(1.0 / theta);
     return with_vl<kVec4>(vec, lanes, [&](auto Vc, auto Lc) {
       constexpr int V = decltype(Vc)::value, L = decltype(Lc)::value;
@@ -1232,7 +1249,7 @@ struct Bicg {
         if (use_amg) amg.template cycle<V, L>(0, s_, sh, st);
       }
       k_t<Arith, V, L><<<tgrid, kThreads, 0, st>>>(A, mp, sh, t, s_, cs, partials, counter, mask);
-      k_xr<Arith, V, L><<<grid, kThreads, 0, st>>>(A, mp, x, ph, sh, s_, t, r, rh, max_iter, cs, partials, counter);
+      k_xr<Arith, V, L><<<grid, kThreads, 0, st>>>(A, mp, x, ph, sh, s_, t, r, rh, max_iter, cs, partials, counter, lc);
       return cudaGetLastError();
     });
   }
@@ -1278,7 +1295,7 @@ struct Bicg {
 
   // Device-driven loop: one iteration is captured as the body of a conditional WHILE graph node
   // whose condition (some column active and fewer than max_iter iterations) is set on the device
-  // by k_loop_cond; one graph launch runs the whole solve with no host round trip. The loop ends
+  // by k_xr (LoopCond); one graph launch runs the whole solve with no host round trip. The loop ends
   // after at most max_iter iterations.
   //
   // The instantiated loop is kept and replayed by later calls on the same x and max_iter (the mixed
@@ -1325,11 +1342,7 @@ struct Bicg {
     if (e == cudaSuccess)
       e = cudaStreamBeginCaptureToGraph(loop.cap, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-      cudaError_t ek = iteration(x, max_iter, loop.cap);
-      if (ek == cudaSuccess) {
-        k_loop_cond<<<1, 32, 0, loop.cap>>>(h, cs.it);
-        ek = cudaGetLastError();
-      }
+      cudaError_t ek = iteration(x, max_iter, loop.cap, LoopCond{h, true});
       cudaGraph_t captured = nullptr;
       e = cudaStreamEndCapture(loop.cap, &captured);
       if (e == cudaSuccess) e = ek;
@@ -1638,12 +1651,7 @@ struct SysImpl : SysBase {
         e = capture_while(cap, &h, &body);
         if (e == cudaSuccess)
           e = capture_into(body, [&](cudaStream_t c) {
-            cudaError_t ek = S.iteration(x, o.max_iter, c);
-            if (ek == cudaSuccess) {
-              k_loop_cond<<<1, 32, 0, c>>>(h, S.cs.it);
-              ek = cudaGetLastError();
-            }
-            return ek;
+            return S.iteration(x, o.max_iter, c, LoopCond{h, true});
           });
       }
     } else {
@@ -1664,12 +1672,7 @@ struct SysImpl : SysBase {
             ek = capture_while(c, &hi, &ibody);
             if (ek == cudaSuccess)
               ek = capture_into(ibody, [&](cudaStream_t c2) {
-                cudaError_t ei = I.iteration(d32, o.inner_max_iter, c2);
-                if (ei == cudaSuccess) {
-                  k_loop_cond<<<1, 32, 0, c2>>>(hi, I.cs.it);
-                  ei = cudaGetLastError();
-                }
-                return ei;
+                return I.iteration(d32, o.inner_max_iter, c2, LoopCond{hi, true});
               });
             // the inner loop's condition starts at 1 when the graph is launched; re-arm it after the
             // loop ends so that the next outer step runs its inner solve again

@@ -1,0 +1,50 @@
+"""Products and solves at the row counts where the tile height changes (tile_rows_for): the last size of
+one height and the first of the next, with a ragged last tile, against the CPU oracle.
+
+Tolerances as in test_gpu_gspmv.py: float64 1e-12 of |A||X| per element, float32 (row length + 2) 2^-24.
+"""
+
+import numpy as np
+import pytest
+
+import gen
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def ens():
+    from paper_1711_10622_gb300 import build
+
+    build.build()
+    import paper_1711_10622_gb300 as ens
+
+    return ens
+
+
+def _banded(n, seed):
+    rng = np.random.default_rng(seed)
+    i = np.arange(n, dtype=np.int64)
+    cols = np.stack([np.maximum(i - 100, 0), i, np.minimum(i + 37, n - 1)], axis=1)
+    rp = (3 * np.arange(n + 1)).astype(np.int32)
+    return gen.Operator("banded", (n, 1, 1), ("x",) * 3, rp, cols.reshape(-1).astype(np.int32), rng.standard_normal(3 * n), False)
+
+
+@pytest.mark.parametrize("n", [303 * 64 + 1, 304 * 64 - 63, 303 * 128 + 1, 303 * 256, 303 * 256 + 1])
+@pytest.mark.parametrize("m,dtype", [(1, "f64"), (2, "f64"), (8, "f64"), (4, "f32"), (32, "f32")])
+def test_product_at_tile_height_edges(ens, n, m, dtype):
+    op = _banded(n, n)
+    X = gen.rhs_normal(n, m, m)
+    if dtype == "f32":
+        op = gen.Operator(op.name, op.shape, op.bcs, op.row_ptr, op.col_idx, op.val.astype(np.float32).astype(np.float64), False)
+        X = X.astype(np.float32)
+    with ens.Matrix.from_operator(op) as A:
+        Y = ens.gspmv(A, torch.from_numpy(X).cuda()).cpu().numpy().astype(np.float64)
+    X = X.astype(np.float64)
+    ref = oracle.gspmv(op, X)
+    scale = np.abs(op.val).reshape(n, 3, 1) * np.abs(X)[op.col_idx.reshape(n, 3)]
+    tol = 1e-12 if dtype == "f64" else 5 * 2.0**-24
+    assert np.all(np.abs(Y - ref) <= tol * scale.sum(axis=1))
