@@ -29,6 +29,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "amg_small.cuh"
 #include "ens_internal.cuh"
 #include "reduce.cuh"
 #include "rowprod.cuh"
@@ -749,86 +750,6 @@ __global__ void __launch_bounds__(kThreads)
   }
 }
 
-// The coarsest level's whole smoothing z = S_steps(src) in one block (levels of at most
-// kCoarseBlockRows rows): the first term of k_amg_first and then every step of k_cheb, with a block
-// barrier where the separate launches had a kernel boundary. A step's product reads the previous
-// step's d, written in this launch, so X is loaded with plain (coherent) loads and multiplied with
-// native FMA (float values for the float32 solver): a few thousand products per step, where one
-// launch per step cost more than its work.
-constexpr int kCoarseBlockRows = 2048;
-constexpr int kMaxCoarseSteps = 64;
-template <typename T>
-struct CoarseCoefs {
-  T c1[kMaxCoarseSteps], c2[kMaxCoarseSteps];  // step k >= 1
-};
-
-template <typename Arith, int VEC, int LANES>
-__global__ void __launch_bounds__(kThreads)
-    k_amg_coarse(MatView A, int32_t m, const typename Arith::T *__restrict__ src, typename Arith::T *da,
-                 typename Arith::T *db, typename Arith::T *res, typename Arith::T *z, typename Arith::T inv_theta,
-                 CoarseCoefs<typename Arith::T> cf, int32_t steps) {
-  using T = typename Arith::T;
-  constexpr int G = kThreads / LANES;
-  const int32_t c = (threadIdx.x % LANES) * VEC;
-  const bool act = c < m;
-  if (act)
-    for (int64_t i = threadIdx.x / LANES; i < A.n; i += G) {
-      T sv[VEC];
-      load_vec<T, VEC>(src + i * m + c, sv);
-      const T sc = Arith::dinv(A, i) * inv_theta;
-#pragma unroll
-      for (int q = 0; q < VEC; ++q) sv[q] *= sc;
-      store_vec<T, VEC>(da + i * m + c, sv);
-      store_vec<T, VEC>(z + i * m + c, sv);
-    }
-  __syncthreads();
-  T *din = da, *dout = db;
-  for (int k = 1; k < steps; ++k) {
-    const bool first = k == 1, last = k == steps - 1;
-    const T c1 = cf.c1[k], c2 = cf.c2[k];
-    if (act)
-      for (int64_t i = threadIdx.x / LANES; i < A.n; i += G) {
-        T w[VEC];
-#pragma unroll
-        for (int q = 0; q < VEC; ++q) w[q] = T(0);
-        for (int32_t j = A.rp[i]; j < A.rp[i + 1]; ++j) {
-          T a;
-          if constexpr (std::is_same<T, float>::value)
-            a = A.val32[j];
-          else
-            a = A.val[j];
-          T x[VEC];
-          load_vec_rw<T, VEC>(din + (int64_t)A.ci[j] * m + c, x);
-#pragma unroll
-          for (int q = 0; q < VEC; ++q) w[q] = fma(a, x[q], w[q]);
-        }
-        T di[VEC], rs[VEC], zv[VEC], dn[VEC];
-        load_vec_rw<T, VEC>(din + i * m + c, di);
-        if (first)
-          load_vec<T, VEC>(src + i * m + c, rs);
-        else
-          load_vec_rw<T, VEC>(res + i * m + c, rs);
-        load_vec_rw<T, VEC>(z + i * m + c, zv);
-        const T dv = Arith::dinv(A, i);
-#pragma unroll
-        for (int q = 0; q < VEC; ++q) {
-          rs[q] -= w[q];
-          dn[q] = c1 * di[q] + c2 * (dv * rs[q]);
-          zv[q] += dn[q];
-        }
-        store_vec<T, VEC>(z + i * m + c, zv);
-        if (!last) {
-          store_vec<T, VEC>(res + i * m + c, rs);
-          store_vec<T, VEC>(dout + i * m + c, dn);
-        }
-      }
-    __syncthreads();
-    T *t = din;
-    din = dout;
-    dout = t;
-  }
-}
-
 // res = r - A z
 template <typename Arith, int VEC, int LANES>
 __global__ void __launch_bounds__(kThreads, ChebBlocks<Arith, VEC>::value)
@@ -926,6 +847,78 @@ struct AmgCycle {
   std::vector<Level> lev;
   ens_amg_opts o;
   int mp = 0, vec = 2, lanes = 1;
+  // Levels from tail_at down run in one launch of one cluster (amg_small.cuh); lev.size(): none.
+  size_t tail_at = 0;
+  TailArgs<T> tail;
+
+  // Values of a level's matrix in the type of the cycle.
+  static const T *values(const MatView &A) {
+    if constexpr (std::is_same<T, float>::value)
+      return A.val32;
+    else
+      return A.val;
+  }
+  static const T *inv_diag(const MatView &A) {
+    if constexpr (std::is_same<T, float>::value)
+      return A.dinv32;
+    else
+      return A.dinv;
+  }
+  // Levels that share a row's nonzeros between threads: few enough rows that one thread group per row
+  // leaves SMs idle or waiting. In float64 the sums are native, so only while the FP64 pipe needs a few
+  // microseconds for them.
+  bool small(const Level &L) const { return L.n * mp <= (std::is_same<T, float>::value ? 1 << 21 : 1 << 18); }
+  bool fused_smoothing(const Level &L) const { return o.smooth_steps == 2 && L.has_as; }
+
+  // The descriptors of the tail: the coarsest level and, going up, the levels small enough for one cluster.
+  void setup_tail() {
+    const size_t nl = lev.size();
+    tail_at = nl;
+    if (o.coarse_steps > kMaxCoarseSteps || lev[nl - 1].n > kTailCoarseRows) return;
+    tail_at = nl - 1;
+    const int64_t rows = std::is_same<T, float>::value ? kTailRows : kTailRowsF64;
+    while (tail_at > 0 && nl - tail_at < kMaxTailLevels && lev[tail_at - 1].n <= rows && fused_smoothing(lev[tail_at - 1])) --tail_at;
+    const double theta = 0.5 * (o.cheb_hi + o.cheb_lo), delta = 0.5 * (o.cheb_hi - o.cheb_lo), sigma = theta / delta;
+    TailArgs<T> &a = tail;
+    a = TailArgs<T>{};
+    a.nl = (int32_t)(nl - tail_at);
+    a.m = mp;
+    a.lanes = lanes;
+    a.steps = o.coarse_steps;
+    a.inv_theta = (T)(1.0 / theta);
+    double rho_prev = 1.0 / sigma;
+    for (int k = 1; k < kMaxCoarseSteps; ++k) {
+      const double rho = 1.0 / (2.0 * sigma - rho_prev);
+      a.k1[k] = (T)(rho * rho_prev);
+      a.k2[k] = (T)(2.0 * rho / delta);
+      rho_prev = rho;
+    }
+    a.c1 = a.k1[1];
+    a.c2 = a.k2[1];
+    const Level &C = lev[nl - 1];
+    a.da = C.da;
+    a.db = C.db;
+    a.res = C.cres;
+    for (size_t l = tail_at; l < nl; ++l) {
+      const Level &L = lev[l];
+      TailLevel<T> &t = a.lev[l - tail_at];
+      t.rp = L.A.rp;
+      t.ci = L.A.ci;
+      t.va = values(L.A);
+      t.srp = L.As.rp;
+      t.sci = L.As.ci;
+      t.sva = L.has_as ? values(L.As) : nullptr;
+      t.dinv = inv_diag(L.A);
+      t.agg = L.agg;
+      t.ptr = L.ptr;
+      t.mem = L.mem;
+      t.r = L.r;
+      t.z = L.z;
+      t.res = L.res;
+      t.n = (int32_t)L.n;
+      t.nc = (int32_t)L.nc;
+    }
+  }
 
   cudaError_t setup(Scratch &sc, const ens_amg *H, int mp_, int vec_, int lanes_) {
     o = H->opts;
@@ -962,11 +955,16 @@ struct AmgCycle {
         if (e == cudaSuccess) e = sc.get(&L.r, blk);
         if (e == cudaSuccess) e = sc.get(&L.z, blk);
       }
-      T **bufs[] = {&L.res, &L.cres, &L.da, &L.db};
-      for (T **b : bufs)
-        if (e == cudaSuccess) e = sc.get(b, blk);
+      const bool coarsest = l + 1 == H->lev.size();
+      if (!coarsest && e == cudaSuccess) e = sc.get(&L.res, blk);
+      if (coarsest || !fused_smoothing(L)) {  // blocks of the update-by-update smoothing
+        T **bufs[] = {&L.cres, &L.da, &L.db};
+        for (T **b : bufs)
+          if (e == cudaSuccess) e = sc.get(b, blk);
+      }
       lev.push_back(L);
     }
+    if (e == cudaSuccess) setup_tail();
     return e;
   }
 
@@ -977,6 +975,11 @@ struct AmgCycle {
     if (steps == 2 && L.has_as) {  // both updates in one pass over the scaled copy
       const double sigma = theta / delta, rho_prev = 1.0 / sigma, rho = 1.0 / (2.0 * sigma - rho_prev);
       const T c1 = (T)(rho * rho_prev), c2 = (T)(2.0 * rho / delta), it = (T)(1.0 / theta);
+      if (small(L)) {
+        launch_small_smooth2(SmallLevel<T>{L.As.rp, L.As.ci, values(L.As), inv_diag(L.A), (int32_t)L.n, mp, Ln}, V, add, src, z, it, c1,
+                             c2, st);
+        return;
+      }
       if constexpr (std::is_same<Ar, ArithF64Split>::value || std::is_same<Ar, ArithF64Hybrid>::value) {
         if (!L.as_split) {  // the scaled copy's values leave the split range: native products
           if (add)
@@ -1032,6 +1035,10 @@ struct AmgCycle {
   // L.res = r - A z on level L
   template <typename Ar, int V, int Ln>
   void resid(const Level &L, const T *z, const T *r, cudaStream_t st) {
+    if (small(L)) {
+      launch_small_resid(SmallLevel<T>{L.A.rp, L.A.ci, values(L.A), inv_diag(L.A), (int32_t)L.n, mp, Ln}, V, z, r, L.res, st);
+      return;
+    }
     if constexpr (std::is_same<Ar, ArithF64Split>::value && V == 2 && Ln >= 2) {
       if (mp % 4 == 0 &&
           launch_amg_resid4_split(Ln / 2, L.A, mp, z, r, L.res, L.mask, L.sms, tile_count(L.n, Ln / 2), st))
@@ -1044,21 +1051,6 @@ struct AmgCycle {
   void level_cycle(size_t l, const T *r, T *z, cudaStream_t st) {
     const Level &L = lev[l];
     if (l + 1 == lev.size()) {
-      if (L.n <= kCoarseBlockRows && o.coarse_steps <= kMaxCoarseSteps) {  // one block, one launch
-        const double theta = 0.5 * (o.cheb_hi + o.cheb_lo), delta = 0.5 * (o.cheb_hi - o.cheb_lo);
-        const double sigma = theta / delta;
-        double rho_prev = 1.0 / sigma;
-        CoarseCoefs<T> cf{};
-        for (int k = 1; k < o.coarse_steps; ++k) {
-          const double rho = 1.0 / (2.0 * sigma - rho_prev);
-          cf.c1[k] = (T)(rho * rho_prev);
-          cf.c2[k] = (T)(2.0 * rho / delta);
-          rho_prev = rho;
-        }
-        k_amg_coarse<Ar, V, Ln><<<1, kThreads, 0, st>>>(L.A, mp, r, L.da, L.db, L.cres, z, (T)(1.0 / theta), cf,
-                                                        o.coarse_steps);
-        return;
-      }
       this->template smooth<Ar, V, Ln>(L, r, z, false, o.coarse_steps, st);
       return;
     }
@@ -1075,6 +1067,13 @@ struct AmgCycle {
   // Levels where the split arithmetic cannot run (value range) use native DFMA.
   template <int V, int Ln>
   void cycle(size_t l, const T *r, T *z, cudaStream_t st) {
+    if (l >= tail_at) {
+      TailArgs<T> a = tail;
+      a.lev[0].r = const_cast<T *>(r);  // read only
+      a.lev[0].z = z;
+      launch_amg_tail(a, V, st);
+      return;
+    }
     if constexpr (std::is_same<Arith, ArithF64Split>::value || std::is_same<Arith, ArithF64Hybrid>::value) {
       if (!lev[l].split) {
         this->template level_cycle<ArithF64Native, V, Ln>(l, r, z, st);
