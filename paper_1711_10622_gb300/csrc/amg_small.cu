@@ -22,7 +22,7 @@ namespace ens {
 namespace solver {
 namespace {
 
-constexpr int kTailBlocks = 8;  // portable cluster size
+constexpr int kTailBlocks = 8;  // portable cluster size; 16 gave 3 % on the mixed solve and lost 1 % on the batch
 constexpr int kTailThreads = 1024;
 constexpr size_t kTailSmem = 96 * 1024;
 
@@ -141,6 +141,43 @@ __device__ __forceinline__ void smooth2_rows(const Place &p, const int32_t *rp, 
   }
 }
 
+// rc_I = sum of res over the rows of aggregate I, the rows dealt to the S threads of the aggregate.
+template <typename T, int VEC>
+__device__ __forceinline__ void restrict_rows(const Place &p, const int32_t *__restrict__ ptr, const int32_t *__restrict__ mem, int32_t nc,
+                                              int32_t m, int32_t lanes, int32_t S, const T *res, T *rc) {
+  for (int32_t i0 = 0; i0 < nc; i0 += p.groups) {
+    const int32_t I = i0 + p.grp;
+    const bool ok = I < nc && p.col;
+    T acc[VEC];
+#pragma unroll
+    for (int q = 0; q < VEC; ++q) acc[q] = T(0);
+    if (ok) {
+      const int32_t t1 = __ldg(ptr + I + 1);
+      for (int32_t t = __ldg(ptr + I) + p.sub; t < t1; t += 4 * S) {
+        T v[4][VEC];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (t + u * S < t1) load_cg<T, VEC>(res + (int64_t)__ldg(mem + t + u * S) * m + p.c, v[u]);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (t + u * S < t1)
+#pragma unroll
+            for (int q = 0; q < VEC; ++q) acc[q] += v[u][q];
+      }
+    }
+    for (int32_t off = lanes; off < lanes * S; off <<= 1)
+#pragma unroll
+      for (int q = 0; q < VEC; ++q) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], off);
+    if (ok && p.sub == 0) store_vec<T, VEC>(rc + (int64_t)I * m + p.c, acc);
+  }
+}
+
+template <typename T, int VEC>
+__global__ void __launch_bounds__(256)
+    k_small_restrict(const int32_t *ptr, const int32_t *mem, int32_t nc, int32_t m, int32_t lanes, int32_t S, const T *res, T *rc) {
+  const Place p = place<VEC>((int32_t)(blockIdx.x * 256 + threadIdx.x), (int32_t)gridDim.x * 256, m, lanes, S);
+  restrict_rows<T, VEC>(p, ptr, mem, nc, m, lanes, S, res, rc);
+}
 template <typename T, int VEC>
 __global__ void __launch_bounds__(256)
     k_small_resid(SmallLevel<T> A, int32_t S, const T *z, const T *r, T *res) {
@@ -209,7 +246,7 @@ __device__ __forceinline__ void coarse_updates(const TailArgs<T> &a, const TailL
 }
 
 template <typename T, int VEC>
-__global__ void __launch_bounds__(kTailThreads) k_amg_tail(const __grid_constant__ TailArgs<T> a, int32_t S, int32_t Sc, int in_smem) {
+__global__ void __launch_bounds__(kTailThreads) k_amg_tail(const __grid_constant__ TailArgs<T> a, int32_t S, int in_smem) {
   extern __shared__ __align__(16) unsigned char raw[];
   const int32_t rank = (int32_t)blockIdx.x, m = a.m;
   const Place p = place<VEC>(rank * kTailThreads + (int32_t)threadIdx.x, kTailBlocks * kTailThreads, m, a.lanes, S);
@@ -221,24 +258,7 @@ __global__ void __launch_bounds__(kTailThreads) k_amg_tail(const __grid_constant
     cluster_barrier();
     resid_rows<T, VEC>(p, L.rp, L.ci, L.va, L.n, m, a.lanes, S, L.z, L.r, L.res);
     cluster_barrier();
-    for (int32_t I = e.grp; I < L.nc && e.col; I += e.groups) {  // rows of an aggregate in ascending order
-      T acc[VEC];
-#pragma unroll
-      for (int q = 0; q < VEC; ++q) acc[q] = T(0);
-      const int32_t t1 = __ldg(L.ptr + I + 1);
-      for (int32_t t = __ldg(L.ptr + I); t < t1; t += 4) {
-        T v[4][VEC];
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (t + u < t1) load_cg<T, VEC>(L.res + (int64_t)__ldg(L.mem + t + u) * m + e.c, v[u]);
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (t + u < t1)
-#pragma unroll
-            for (int q = 0; q < VEC; ++q) acc[q] += v[u][q];
-      }
-      store_vec<T, VEC>(C.r + (int64_t)I * m + e.c, acc);
-    }
+    restrict_rows<T, VEC>(p, L.ptr, L.mem, L.nc, m, a.lanes, S, L.res, C.r);
     cluster_barrier();
   }
   if (rank == 0) {
@@ -246,7 +266,7 @@ __global__ void __launch_bounds__(kTailThreads) k_amg_tail(const __grid_constant
     if (in_smem) {
       const int64_t blk = (int64_t)L.n * m;
       T *d0 = reinterpret_cast<T *>(raw), *d1 = d0 + blk, *res = d1 + blk, *z = res + blk;
-      coarse_updates<T, VEC, true>(a, L, d0, d1, res, z, Sc);
+      coarse_updates<T, VEC, true>(a, L, d0, d1, res, z, S);
       const Place g = place<VEC>((int32_t)threadIdx.x, kTailThreads, m, a.lanes, 1);
       for (int32_t i = g.grp; i < L.n && g.col; i += g.groups) {
         T zv[VEC];
@@ -254,7 +274,7 @@ __global__ void __launch_bounds__(kTailThreads) k_amg_tail(const __grid_constant
         store_vec<T, VEC>(L.z + (int64_t)i * m + g.c, zv);
       }
     } else {
-      coarse_updates<T, VEC, false>(a, L, a.da, a.db, a.res, L.z, Sc);
+      coarse_updates<T, VEC, false>(a, L, a.da, a.db, a.res, L.z, S);
     }
   }
   cluster_barrier();
@@ -295,10 +315,10 @@ cudaError_t run_tail(const TailArgs<T> &a, cudaStream_t st) {
   at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  // four threads per row on the levels above the coarsest (8 blocks hold their rows in one to four sweeps),
-  // eight on the coarsest, whose rows are the longest
-  const int32_t S = std::min(4, 32 / a.lanes), Sc = std::min(8, 32 / a.lanes);
-  return cudaLaunchKernelEx(&cfg, k, a, S, Sc, in_smem ? 1 : 0);
+  // Four threads per row, on the coarsest level too (channel 96^3, m = 8, mixed solve: 59.5 ms; 8 threads
+  // there 63.0, 16: 69.6; 8 or 16 on the other levels as well: 62.0 and 67.8).
+  const int32_t S = std::min(4, 32 / a.lanes);
+  return cudaLaunchKernelEx(&cfg, k, a, S, in_smem ? 1 : 0);
 }
 
 // Threads per row: the rows of the level spread over the GPU's resident threads (152 SMs x 2048), at most 16
@@ -337,8 +357,26 @@ cudaError_t small_smooth2(const SmallLevel<T> &A, int vec, bool add, const T *sr
   });
 }
 
+template <typename T>
+cudaError_t small_restrict(const int32_t *ptr, const int32_t *mem, int32_t nc, int32_t m, int32_t lanes, int vec, const T *res, T *rc,
+                           cudaStream_t st) {
+  const int32_t S = parts(nc, lanes);
+  return with_vec<T>(vec, [&](auto V) {
+    k_small_restrict<T, decltype(V)::value><<<blocks_for(nc, lanes, S), 256, 0, st>>>(ptr, mem, nc, m, lanes, S, res, rc);
+    return cudaGetLastError();
+  });
+}
+
 }  // namespace
 
+cudaError_t launch_small_restrict(const int32_t *ptr, const int32_t *mem, int32_t nc, int32_t m, int32_t lanes, int vec, const float *res,
+                                  float *rc, cudaStream_t st) {
+  return small_restrict<float>(ptr, mem, nc, m, lanes, vec, res, rc, st);
+}
+cudaError_t launch_small_restrict(const int32_t *ptr, const int32_t *mem, int32_t nc, int32_t m, int32_t lanes, int vec, const double *res,
+                                  double *rc, cudaStream_t st) {
+  return small_restrict<double>(ptr, mem, nc, m, lanes, vec, res, rc, st);
+}
 cudaError_t launch_amg_tail(const TailArgs<float> &a, int vec, cudaStream_t st) {
   return with_vec<float>(vec, [&](auto V) { return run_tail<float, decltype(V)::value>(a, st); });
 }

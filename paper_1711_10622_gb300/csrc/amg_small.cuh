@@ -61,5 +61,11 @@ cudaError_t launch_small_smooth2(const SmallLevel<float> &As, int vec, bool add,
 cudaError_t launch_small_smooth2(const SmallLevel<double> &As, int vec, bool add, const double *src, double *z, double inv_theta,
                                  double c1, double c2, cudaStream_t st);
 
+// rc_I = sum of res over the rows of aggregate I (members mem[ptr[I]..ptr[I+1])).
+cudaError_t launch_small_restrict(const int32_t *ptr, const int32_t *mem, int32_t nc, int32_t m, int32_t lanes, int vec, const float *res,
+                                  float *rc, cudaStream_t st);
+cudaError_t launch_small_restrict(const int32_t *ptr, const int32_t *mem, int32_t nc, int32_t m, int32_t lanes, int vec, const double *res,
+                                  double *rc, cudaStream_t st);
+
 }  // namespace solver
 }  // namespace ens

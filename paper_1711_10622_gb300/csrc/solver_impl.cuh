@@ -1057,7 +1057,10 @@ struct AmgCycle {
     const Level &C = lev[l + 1];
     this->template smooth<Ar, V, Ln>(L, r, z, false, o.smooth_steps, st);
     this->template resid<Ar, V, Ln>(L, z, r, st);
-    k_amg_restrict<T, V, Ln><<<L.cgrid, kThreads, 0, st>>>(L.nc, mp, L.ptr, L.mem, L.res, C.r);
+    if (small(C))
+      launch_small_restrict(L.ptr, L.mem, (int32_t)L.nc, mp, Ln, V, L.res, C.r, st);
+    else
+      k_amg_restrict<T, V, Ln><<<L.cgrid, kThreads, 0, st>>>(L.nc, mp, L.ptr, L.mem, L.res, C.r);
     this->template cycle<V, Ln>(l + 1, C.r, C.z, st);
     k_amg_prolong<T, V, Ln><<<L.egrid, kThreads, 0, st>>>(L.n, mp, L.agg, C.z, z);
     this->template resid<Ar, V, Ln>(L, z, r, st);
