@@ -1165,7 +1165,8 @@ struct Bicg {
       sh = s_;
       da = db = res = nullptr;
     }
-    if (e == cudaSuccess) e = sc.get(&partials, (size_t)std::max(grid, tgrid) * 3 * kMaxSolveM);
+    // the same for every width (not the grids of this one): a server fits the workspace as beta + gamma m
+    if (e == cudaSuccess) e = sc.get(&partials, (size_t)num_sms * std::max(4, TileBlocks<Arith>::value) * 3 * kMaxSolveM);
     if (e == cudaSuccess) e = sc.get(&counter, 1);
     if (e == cudaSuccess) e = cudaMemsetAsync(counter, 0, sizeof(unsigned), s);
     if (e == cudaSuccess) e = alloc_cols(sc, mp, cs);
