@@ -1,0 +1,293 @@
+// Row boxes of a sparse matrix (see boxprod.cuh for the product that uses them): built on the host when
+// the matrix is created, by several threads, and uploaded; the values are laid out on the device.
+//
+// A box is up to kBoxRows rows whose columns overlap as much as possible. For the stencils of grid
+// operators these are bricks of grid cells, found from the matrix alone: `short_step` and `long_step` are
+// the two commonest distances between a row and a later column (one line and one plane of the grid), and a
+// brick starts at the first free row and follows, line by line, the actual columns nearest to those
+// distances, so removed cells that shift the numbering do not matter. A box ends early when its columns
+// would exceed kBoxCols. Any matrix gets a correct plan; it is kept only where the columns are read few
+// enough times to pay (columns of all boxes <= 0.45 nnz) and the boxes are mostly full.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cmath>
+#include <cstdint>
+#include <cstring>
+#include <new>
+#include <thread>
+#include <unordered_map>
+#include <vector>
+
+#include "boxprod.cuh"
+#include "ens_internal.cuh"
+
+namespace ens {
+namespace {
+
+// The two commonest distances d = col - row > 1 over a sample of rows: the commonest, and the commonest of
+// those at least twice as far or half as near. 0 where there is none.
+void common_steps(int64_t n, const int32_t *rp, const int32_t *ci, int64_t &short_step, int64_t &long_step) {
+  std::unordered_map<int64_t, int64_t> count;
+  const int64_t samples = std::min<int64_t>(n, 4096);
+  for (int64_t s = 0; s < samples; ++s) {
+    const int64_t i = (int64_t)((uint64_t)s * 2654435761u % (uint64_t)n);  // not in step with the grid's lines
+    for (int32_t j = rp[i]; j < rp[i + 1]; ++j)
+      if ((int64_t)ci[j] - i > 1) ++count[(int64_t)ci[j] - i];
+  }
+  int64_t a = 0, na = 0, b = 0, nb = 0;
+  for (auto &e : count)
+    if (e.second > na || (e.second == na && e.first < a)) a = e.first, na = e.second;
+  for (auto &e : count)
+    if ((e.first >= 2 * a || 2 * e.first <= a) && (e.second > nb || (e.second == nb && e.first < b))) b = e.first, nb = e.second;
+  if (nb * 8 < na) b = 0;
+  short_step = b == 0 ? a : std::min(a, b);
+  long_step = b == 0 ? 0 : std::max(a, b);
+}
+
+struct Part {  // boxes of one range of rows
+  std::vector<int32_t> rows, cols;        // concatenated
+  std::vector<uint16_t> loc;              // kBoxRows * K per box, slot-major
+  std::vector<int32_t> nrows, ncols;
+  int64_t ucols = 0;
+};
+
+// Columns of the box that is being filled -> position, by open addressing; cleared by a new stamp.
+struct ColumnSet {
+  static constexpr int kSize = 4096;
+  std::vector<int32_t> key, pos, stamp;
+  int32_t now = 0, count = 0;
+  ColumnSet() : key(kSize), pos(kSize), stamp(kSize, 0) {}
+  void clear() { ++now, count = 0; }
+  // Position of c, or -1 if it is not there; `at` is where it goes.
+  int32_t find(int32_t c, uint32_t &at) const {
+    at = ((uint32_t)c * 2654435761u) >> 20;
+    while (stamp[at] == now) {
+      if (key[at] == c) return pos[at];
+      at = (at + 1) & (kSize - 1);
+    }
+    return -1;
+  }
+};
+
+void build_part(int64_t r0, int64_t r1, const int32_t *rp, const int32_t *ci, int32_t K, int64_t s1, int64_t s2, Part &P) {
+  const int64_t n = r1 - r0;
+  std::vector<uint8_t> used(n, 0);
+  ColumnSet cs;
+  const int lines = s2 ? kBoxLinesY : s1 ? kBoxLinesY * kBoxLinesZ : 1, planes = s2 ? kBoxLinesZ : 1;
+  const int len = s1 ? kBoxLineX : kBoxRows;
+  // the row in [r0, r1) that row i's columns name at about distance d, or -1
+  auto step = [&](int64_t i, int64_t d) -> int64_t {
+    int64_t best = -1, off = d / 2 + 1;
+    for (int32_t j = rp[i]; j < rp[i + 1]; ++j) {
+      const int64_t e = (int64_t)ci[j] - i, t = e > d ? e - d : d - e;
+      if (e > 1 && t < off) off = t, best = ci[j];
+    }
+    return best < r1 ? best : -1;
+  };
+  auto from = [&](int64_t base, int64_t d) -> int64_t {  // the second row of a line decides: the first may wrap
+    if (base + 1 < r1) {
+      const int64_t t = step(base + 1, d);
+      if (t > 0) return t - 1;
+    }
+    return step(base, d);
+  };
+  std::vector<int32_t> rows;
+  int64_t next = r0;
+  while (next < r1) {
+    if (used[next - r0]) {
+      ++next;
+      continue;
+    }
+    rows.clear();
+    cs.clear();
+    const size_t col0 = P.cols.size();
+    // a row joins when the box has room for it and for its new columns
+    auto take = [&](int64_t i) -> bool {
+      if ((int)rows.size() == kBoxRows) return false;
+      int32_t fresh = 0;
+      uint32_t at;
+      for (int32_t j = rp[i]; j < rp[i + 1]; ++j) fresh += cs.find(ci[j], at) < 0;
+      if (cs.count + fresh > kBoxCols) return false;
+      for (int32_t j = rp[i]; j < rp[i + 1]; ++j)
+        if (cs.find(ci[j], at) < 0) {
+          cs.stamp[at] = cs.now;
+          cs.key[at] = ci[j];
+          cs.pos[at] = cs.count++;
+          P.cols.push_back(ci[j]);
+        }
+      rows.push_back((int32_t)i);
+      used[i - r0] = 1;
+      return true;
+    };
+    bool full = false;
+    int64_t plane = next;
+    for (int z = 0; z < planes && plane >= 0 && !full; ++z) {
+      int64_t line = plane;
+      for (int y = 0; y < lines && line >= 0 && !full; ++y) {
+        for (int x = 0; x < len && line + x < r1 && !used[line + x - r0]; ++x)
+          if (!take(line + x)) {
+            full = true;
+            break;
+          }
+        line = s1 ? from(line, s1) : -1;
+        if (line >= 0 && (line < r0 || line >= r1)) line = -1;
+      }
+      plane = s2 ? from(plane, s2) : -1;
+      if (plane >= 0 && (plane < r0 || plane >= r1)) plane = -1;
+    }
+    if (rows.empty()) {  // one row with more columns than a box holds: no plan
+      P.ucols = INT64_MAX / 4;
+      return;
+    }
+    // Columns in ascending order: neighbouring rows of the box then read neighbouring X rows, staged from
+    // whole lines of memory and read from shared memory without bank conflicts.
+    std::sort(P.cols.begin() + col0, P.cols.end());
+    cs.clear();
+    for (size_t q = col0; q < P.cols.size(); ++q) {
+      uint32_t at;
+      cs.find(P.cols[q], at);
+      cs.stamp[at] = cs.now;
+      cs.key[at] = P.cols[q];
+      cs.pos[at] = cs.count++;
+    }
+    const size_t l0 = P.loc.size();
+    P.loc.resize(l0 + (size_t)kBoxRows * K, (uint16_t)kBoxCols);  // missing entries: the row of zeros
+    for (size_t r = 0; r < rows.size(); ++r) {
+      const int64_t i = rows[r];
+      uint32_t at;
+      for (int32_t j = rp[i]; j < rp[i + 1]; ++j) P.loc[l0 + (size_t)(j - rp[i]) * kBoxRows + r] = (uint16_t)cs.find(ci[j], at);
+    }
+    P.rows.insert(P.rows.end(), rows.begin(), rows.end());
+    P.nrows.push_back((int32_t)rows.size());
+    P.ncols.push_back((int32_t)(P.cols.size() - col0));
+    P.ucols += cs.count;
+  }
+}
+
+// Values of every box slot from the CSR arrays (0 in the padding): split pairs and float32.
+__global__ void k_box_values(int32_t boxes, int32_t K, const int32_t *__restrict__ brow, const int2 *__restrict__ bcnt,
+                             const int32_t *__restrict__ rp, const float2 *__restrict__ vs, const float *__restrict__ v32,
+                             float2 *__restrict__ bvs, float *__restrict__ bv32) {
+  const int64_t total = (int64_t)boxes * K * kBoxRows;
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t r = (int32_t)(e % kBoxRows);
+    const int64_t q = e / kBoxRows;
+    const int32_t k = (int32_t)(q % K), b = (int32_t)(q / K);
+    float2 v = make_float2(0.f, 0.f);
+    float f = 0.f;
+    if (r < bcnt[b].x) {
+      const int32_t i = brow[(int64_t)b * kBoxRows + r], j = rp[i] + k;
+      if (j < rp[i + 1]) {
+        v = vs[j];
+        f = v32[j];
+      }
+    }
+    bvs[e] = v;
+    bv32[e] = f;
+  }
+}
+
+template <typename T>
+cudaError_t upload(T **dst, const std::vector<T> &src, cudaStream_t s) {
+  cudaError_t e = cudaMalloc(reinterpret_cast<void **>(dst), std::max<size_t>(src.size(), 1) * sizeof(T));
+  if (e == cudaSuccess && !src.empty()) e = cudaMemcpyAsync(*dst, src.data(), src.size() * sizeof(T), cudaMemcpyHostToDevice, s);
+  return e;
+}
+
+}  // namespace
+
+void free_box(BoxPlan &B) {
+  cudaFree(B.row);
+  cudaFree(B.cnt);
+  cudaFree(B.col);
+  cudaFree(B.loc);
+  cudaFree(B.vs);
+  cudaFree(B.v32);
+  B = BoxPlan{};
+}
+
+cudaError_t build_box(ens_matrix *A, const int32_t *rp, const int32_t *ci, cudaStream_t s) {
+  const int64_t n = A->n, nnz = A->nnz;
+  const int32_t K = A->max_row_len;
+  if (n < kBoxMinRows || K < 1 || K > kBoxMaxLen || (double)nnz < 0.75 * (double)K * (double)n) return cudaSuccess;
+  int64_t s1 = 0, s2 = 0;
+  common_steps(n, rp, ci, s1, s2);
+  const int64_t per_min = 1 << 16;
+  const int parts = (int)std::max<int64_t>(1, std::min<int64_t>({(int64_t)std::max(1u, std::thread::hardware_concurrency()), 16, n / per_min}));
+  std::vector<Part> part(parts);
+  // ranges end on whole bricks of planes where the planes are known
+  const int64_t unit = s2 ? s2 * kBoxLinesZ : kBoxRows;
+  auto bound = [&](int p) { return p == parts ? n : std::min(n, (n * p / parts + unit / 2) / unit * unit); };
+  bool memory = true;
+  {
+    std::vector<std::thread> th;
+    std::vector<uint8_t> failed(parts, 0);
+    auto work = [&](int p) {
+      try {
+        build_part(bound(p), bound(p + 1), rp, ci, K, s1, s2, part[p]);
+      } catch (const std::bad_alloc &) {
+        failed[p] = 1;
+      }
+    };
+    int started = 1;
+    try {
+      th.reserve(parts);
+      for (; started < parts; ++started) th.emplace_back(work, started);
+    } catch (...) {  // no more threads: the rest runs here
+    }
+    work(0);
+    for (int p = started; p < parts; ++p) work(p);
+    for (auto &t : th) t.join();
+    for (uint8_t f : failed) memory = memory && !f;
+  }
+  if (!memory) return cudaSuccess;  // no plan
+  int64_t boxes = 0, ucols = 0;
+  for (auto &p : part) boxes += (int64_t)p.nrows.size(), ucols += p.ucols;
+  if (ucols > (int64_t)(0.45 * (double)nnz) || boxes * kBoxRows > n + n / 4 * 3 + 64 * kBoxRows) return cudaSuccess;
+  std::vector<int32_t> row, col;
+  std::vector<int2> cnt;
+  std::vector<uint16_t> loc;
+  try {
+    row.assign((size_t)boxes * kBoxRows, -1);
+    col.assign((size_t)boxes * kBoxCols, 0);
+    loc.reserve((size_t)boxes * kBoxRows * K);
+    cnt.reserve(boxes);
+    for (auto &p : part) {
+      size_t r = 0, c = 0;
+      for (size_t b = 0; b < p.nrows.size(); ++b) {
+        std::memcpy(row.data() + cnt.size() * kBoxRows, p.rows.data() + r, p.nrows[b] * sizeof(int32_t));
+        std::memcpy(col.data() + cnt.size() * kBoxCols, p.cols.data() + c, p.ncols[b] * sizeof(int32_t));
+        r += p.nrows[b];
+        c += p.ncols[b];
+        cnt.push_back(make_int2(p.nrows[b], p.ncols[b]));
+      }
+      loc.insert(loc.end(), p.loc.begin(), p.loc.end());
+    }
+  } catch (const std::bad_alloc &) {
+    return cudaSuccess;
+  }
+  BoxPlan &B = A->box;
+  B.boxes = (int32_t)boxes;
+  B.K = K;
+  const size_t slots = (size_t)boxes * K * kBoxRows;
+  cudaError_t e = upload(&B.row, row, s);
+  if (e == cudaSuccess) e = upload(&B.cnt, cnt, s);
+  if (e == cudaSuccess) e = upload(&B.col, col, s);
+  if (e == cudaSuccess) e = upload(&B.loc, loc, s);
+  if (e == cudaSuccess) e = cudaMalloc((void **)&B.vs, slots * sizeof(float2));
+  if (e == cudaSuccess) e = cudaMalloc((void **)&B.v32, slots * sizeof(float));
+  if (e == cudaSuccess) {
+    k_box_values<<<A->num_sms * 8, 256, 0, s>>>(B.boxes, K, B.row, B.cnt, A->row, A->valsplit, A->val32, B.vs, B.v32);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (e != cudaSuccess) free_box(B);
+  if (e == cudaErrorMemoryAllocation) {  // the matrix works without a plan
+    cudaGetLastError();
+    e = cudaSuccess;
+  }
+  return e;
+}
+
+}  // namespace ens

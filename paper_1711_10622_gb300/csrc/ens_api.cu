@@ -88,6 +88,7 @@ void free_matrix(ens_matrix *A) {
   cudaFree(A->valsplit);
   cudaFree(A->dinv);
   cudaFree(A->dinv32);
+  free_box(A->box);
   cudaFree(A->stage_x);
   cudaFree(A->stage_y);
   for (cudaEvent_t ev : A->pipe_ev)
@@ -201,6 +202,11 @@ ens_status ens::create_matrix(int64_t n, int64_t ncols, int64_t nnz, const int32
   }
   A->split_ok = (hflags & 1u) == 0;
   A->full_diag = (hflags & 2u) == 0;
+  e = build_box(A, row_ptr, col_idx, s);
+  if (e != cudaSuccess) {
+    free_matrix(A);
+    return cuda_fail(e, "create_matrix: row boxes");
+  }
   // Row chunks of the pipelined host-buffer product: up to kPipeChunks chunks of whole tiles, each
   // with the set of X row blocks its column indices reach.
   {
@@ -286,7 +292,7 @@ ens_status ens_tuned_variant(const ens_matrix *A, int32_t m, int32_t dtype, int3
   const int di = dtype == ENS_F32 ? 1 : 0;
   if (lanes) *lanes = A->tuned_lanes[di][m];
   if (share) *share = dtype == ENS_F32 ? 0 : A->tuned_share[m];
-  if (untiled) *untiled = A->tuned_direct[di][m];
+  if (untiled) *untiled = A->tuned_direct[di][m];  // of the row-by-row launch (row boxes are neither)
   return ENS_OK;
 }
 

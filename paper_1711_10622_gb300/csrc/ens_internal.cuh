@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "ensemble_solve.h"
+#include "rowprod.cuh"
 
 struct ens_amg;  // aggregation multigrid hierarchy attached to a matrix (amg.cu)
 
@@ -38,7 +39,10 @@ struct ens_matrix {
   int8_t tuned_lanes[2][kTuneMaxM + 1];
   int8_t tuned_share[kTuneMaxM + 1];
   int8_t tuned_direct[2][kTuneMaxM + 1];  // 1: rows straight from global memory (no tile), 0: tiled
+  bool tuned_box[2][kTuneMaxM + 1];       // false: the autotuner found a row-by-row launch faster than row boxes
+  ens::BoxPlan box;                            // row boxes (box.boxes = 0: none)
   ens_matrix() {
+    for (int i = 0; i <= kTuneMaxM; ++i) tuned_box[0][i] = tuned_box[1][i] = true;
     for (int i = 0; i <= kTuneMaxM; ++i)
       tuned_lanes[0][i] = tuned_lanes[1][i] = tuned_share[i] = tuned_direct[0][i] = tuned_direct[1][i] = -1;
   }
@@ -95,6 +99,13 @@ ens_status fail(ens_status st, const char *fmt, ...);
 // Record a CUDA failure (message includes cudaGetErrorString) and return ENS_ERR_CUDA/OOM.
 ens_status cuda_fail(cudaError_t e, const char *what);
 void clear_error();
+
+// Row boxes of A from its host CSR arrays (A->box stays empty where boxes do not pay or memory is short).
+cudaError_t build_box(ens_matrix *A, const int32_t *row_ptr, const int32_t *col_idx, cudaStream_t s);
+void free_box(BoxPlan &B);
+// Whether products of width m use A's row boxes: one exists, the width gains by it and no row-by-row
+// arithmetic or traversal was asked for.
+bool use_box(const ens_matrix *A, int m, int dtype);
 
 // Split-float path usable for this matrix (mode, value range, row lengths).
 bool use_split(const ens_matrix *A);

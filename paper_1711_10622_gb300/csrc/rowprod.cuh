@@ -22,6 +22,18 @@ struct MatView {
   const float *__restrict__ dinv32;
 };
 
+// Row boxes of a matrix (boxplan.cu, boxprod.cuh), on the device; boxes = 0: none. Box b holds rows
+// row[b * kBoxRows + 0 .. cnt[b].x) and columns col[b * kBoxCols + 0 .. cnt[b].y); entry k of its row r is
+// loc (a column position of the box), vs / v32 at index (b * K + k) * kBoxRows + r.
+struct BoxPlan {
+  int32_t boxes = 0, K = 0;
+  int32_t *row = nullptr, *col = nullptr;
+  int2 *cnt = nullptr;
+  uint16_t *loc = nullptr;
+  float2 *vs = nullptr;
+  float *v32 = nullptr;
+};
+
 template <typename T, int VEC>
 struct Vec;
 template <>

@@ -1,0 +1,136 @@
+"""Products by row boxes (operators of 65536 rows and more) against the CPU oracle, element by element:
+ragged boxes (removed cells, odd grids), rows of different lengths, every chunk remainder, misaligned blocks,
+values outside the split range, zeros and non-finite values.
+
+Tolerances as in test_gpu_gspmv.py: float64 1e-12 of |A||X| per element, float32 (row length + 2) 2^-24.
+"""
+
+import numpy as np
+import pytest
+
+import gen
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def ens():
+    from paper_1711_10622_gb300 import build
+
+    build.build()
+    import paper_1711_10622_gb300 as ens
+
+    return ens
+
+
+def _stencil9(nx, ny):
+    """A two-dimensional nine-point operator with missing entries: rows of 4 to 9 nonzeros, some empty."""
+    rng = np.random.default_rng(nx)
+    j, i = np.divmod(np.arange(nx * ny), nx)
+    cols, keep = [], []
+    for dj in (-1, 0, 1):
+        for di in (-1, 0, 1):
+            a, b = i + di, j + dj
+            cols.append(b * nx + a)
+            keep.append((a >= 0) & (a < nx) & (b >= 0) & (b < ny))
+    cols, keep = np.stack(cols, 1), np.stack(keep, 1)
+    keep &= rng.random(nx * ny)[:, None] > 0.001  # empty rows
+    rp = np.concatenate([[0], np.cumsum(keep.sum(1))]).astype(np.int32)
+    col = cols[keep].astype(np.int32)
+    return gen.Operator("stencil9", (nx, ny, 1), ("x",) * 3, rp, col, rng.standard_normal(col.size), False)
+
+
+OPS = {
+    "cubes97x43x37": lambda: gen.cubes(97, 43, 37, size=6),
+    "channel64x40x32": lambda: gen.channel(64, 40, 32),
+    "dirichlet41": lambda: gen.dirichlet_box(41),
+    "stencil9_301x257": lambda: _stencil9(301, 257),
+}
+_cache = {}
+
+
+def _op(name):
+    if name not in _cache:
+        _cache[name] = OPS[name]()
+    assert _cache[name].n >= 65536
+    return _cache[name]
+
+
+def _check(op, X, Y, tol=1e-12):
+    X = X.astype(np.float64)
+    ref = oracle.gspmv(op, X)
+    S = op.to_scipy().copy()
+    S.data = np.abs(S.data)
+    assert np.all(np.abs(Y.astype(np.float64) - ref) <= tol * np.asarray(S @ np.abs(X)))
+
+
+@pytest.mark.parametrize("name", list(OPS))
+@pytest.mark.parametrize("m", [3, 4, 5, 6, 8, 11, 12, 16, 20, 24, 33])
+def test_product(ens, name, m):
+    op = _op(name)
+    X = gen.rhs_normal(op.n, m, m)
+    X32 = X.astype(np.float32)
+    op32 = gen.Operator(op.name, op.shape, op.bcs, op.row_ptr, op.col_idx, op.val.astype(np.float32).astype(np.float64), False)
+    with ens.Matrix.from_operator(op) as A:
+        _check(op, X, ens.gspmv(A, torch.from_numpy(X).cuda()).cpu().numpy())
+        L = int(np.diff(op.row_ptr).max())
+        _check(op32, X32, ens.gspmv(A, torch.from_numpy(X32).cuda()).cpu().numpy(), (L + 2) * 2.0**-24)
+
+
+@pytest.mark.parametrize("m", [4, 8, 16])
+def test_misaligned_blocks(ens, m):
+    op = _op("cubes97x43x37")
+    with ens.Matrix.from_operator(op) as A:
+        for off in (1, 2):
+            for dt, tol in ((torch.float64, 1e-12), (torch.float32, 9 * 2.0**-24)):
+                X = torch.randn(op.n * m + off, dtype=dt, device="cuda")[off:].view(op.n, m)
+                Y = torch.empty(op.n * m + off, dtype=dt, device="cuda")[off:].view(op.n, m)
+                ens.gspmv(A, X, Y)
+                ref = op if dt == torch.float64 else gen.Operator(op.name, op.shape, op.bcs, op.row_ptr, op.col_idx, op.val.astype(np.float32).astype(np.float64), False)
+                _check(ref, X.cpu().numpy(), Y.cpu().numpy(), tol)
+
+
+@pytest.mark.parametrize("m", [3, 8])
+def test_ranges(ens, m):
+    """Zeros, values below and above the split range, and sums beyond float go to native products."""
+    op = _op("channel64x40x32")
+    X = gen.rhs_normal(op.n, m, 7)
+    X[::97, 0] = 0.0
+    X[::89, 1] = 1e-30
+    X[::83, 2] = 3e27
+    X[::79, 1] = -1e280
+    X[:, m - 1] *= 1e-19
+    big = gen.Operator(op.name, op.shape, op.bcs, op.row_ptr, op.col_idx, op.val * 1e12, op.singular)
+    for o in (op, big):
+        with ens.Matrix.from_operator(o) as A:
+            _check(o, X, ens.gspmv(A, torch.from_numpy(X).cuda()).cpu().numpy())
+            Z = ens.gspmv(A, torch.zeros(op.n, m, dtype=torch.float64, device="cuda"))
+            assert not Z.any()
+            one = torch.ones(op.n, m, dtype=torch.float64, device="cuda")
+            _check(o, one.cpu().numpy(), ens.gspmv(A, one).cpu().numpy())
+
+
+@pytest.mark.parametrize("dtype", [np.float64, np.float32])
+def test_nonfinite(ens, dtype):
+    """Infinities and NaN reach exactly the rows whose entries name them, as in the definition."""
+    op = _op("cubes97x43x37")
+    m = 8
+    X = gen.rhs_normal(op.n, m, 8).astype(dtype)
+    X[1000, 1], X[2000, 2], X[3000, 3] = np.nan, np.inf, -np.inf
+    with ens.Matrix.from_operator(op) as A:
+        Y = ens.gspmv(A, torch.from_numpy(X).cuda()).cpu().numpy().astype(np.float64)
+    ref = oracle.gspmv(op, X.astype(np.float64))
+    assert np.array_equal(np.isnan(Y), np.isnan(ref))
+    assert np.array_equal(Y[np.isinf(ref)], ref[np.isinf(ref)])
+    assert np.array_equal(np.isfinite(Y), np.isfinite(ref))
+
+
+def test_repeatable(ens):
+    op = _op("dirichlet41")
+    X = torch.from_numpy(gen.rhs_normal(op.n, 8, 5)).cuda()
+    with ens.Matrix.from_operator(op) as A:
+        Y = ens.gspmv(A, X)
+        assert all(torch.equal(Y, ens.gspmv(A, X)) for _ in range(3))
