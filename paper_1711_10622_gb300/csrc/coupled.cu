@@ -553,7 +553,7 @@ struct Coupled {
     if (e != cudaSuccess) return e;
     if (o.precond == ENS_PRECOND_AMG) {
       use_pre = true;
-      return pre.setup(sc, M->amg, mp, vec, lanes);
+      return pre.setup(sc, M->amg, mp, vec, lanes, true);
     }
     if (o.precond == ENS_PRECOND_CHEBYSHEV) {
       single.opts.theta = 0.0;
@@ -567,7 +567,7 @@ struct Coupled {
       L.A = const_cast<ens_matrix *>(M);
       single.lev.assign(1, L);
       use_pre = true;
-      return pre.setup(sc, &single, mp, vec, lanes);
+      return pre.setup(sc, &single, mp, vec, lanes, true);
     }
     return cudaSuccess;
   }

@@ -217,6 +217,7 @@ ens_status amg_apply_impl(const ens_matrix *A, int32_t m, const void *R, void *Z
   const int32_t mp = m == 1 ? 1 : (m + 1) & ~1;
   // the solver's column mapping: four float32 columns per lane where the width and (for unpadded
   // blocks, which are used in place) the 16-byte alignment allow, two otherwise
+  const bool al32 = mp != m || ((uintptr_t)R % 32 == 0 && (uintptr_t)Z % 32 == 0);  // for row boxes
   const bool al16 = mp != m || ((uintptr_t)R % 16 == 0 && (uintptr_t)Z % 16 == 0);
   const int vec = mp == 1 ? 1 : (std::is_same<Arith, ArithF32>::value && mp % 4 == 0 && al16) ? 4 : 2;
   int lanes = 1;
@@ -239,7 +240,7 @@ ens_status amg_apply_impl(const ens_matrix *A, int32_t m, const void *R, void *Z
       r = rp;
     }
     solver::AmgCycle<Arith> cyc;
-    if (e == cudaSuccess) e = cyc.setup(sc, A->amg, mp, vec, lanes);
+    if (e == cudaSuccess) e = cyc.setup(sc, A->amg, mp, vec, lanes, al32);
     if (e == cudaSuccess) e = cyc.apply(r, mp != m ? zp : z, s);
     if (e == cudaSuccess && mp != m) {
       k_amg_unpad<T><<<pgrid, 256, 0, s>>>(n, m, mp, zp, z);

@@ -35,6 +35,14 @@ bool launch_cheb4_split(int lanes4, bool first, bool last, const MatView &A, int
 }
 
 namespace {
+template <int L>
+void cheb3_4(const MatView &A, int32_t m, const double *z, const double *zp, const double *src, double *z1, double c1, double c2,
+             uint32_t mask, int grid, cudaStream_t st) {
+  if (!zp)
+    k_cheb3<ArithF64Split, 4, L, true><<<grid, kThreads, 0, st>>>(A, m, z, zp, src, z1, c1, c2, mask);
+  else
+    k_cheb3<ArithF64Split, 4, L, false><<<grid, kThreads, 0, st>>>(A, m, z, zp, src, z1, c1, c2, mask);
+}
 int grid4(int num_sms, int64_t grid_cap) {
   return (int)std::max<int64_t>(1, std::min<int64_t>(grid_cap, (int64_t)num_sms * ChebBlocks<ArithF64Split, 4>::value));
 }
@@ -52,6 +60,17 @@ void smooth4(bool add, const MatView &As, const MatView &A, int32_t m, const dou
     k_amg_smooth2<ArithF64Split, 4, L, false><<<grid, kThreads, 0, st>>>(As, A, m, src, z, it, c1, c2, mask);
 }
 }  // namespace
+
+bool launch_cheb3_4_split(int lanes4, const MatView &A, int32_t m, const double *z, const double *zp, const double *src,
+                          double *z1, double c1, double c2, uint32_t mask, int num_sms, int64_t grid_cap, cudaStream_t st) {
+  const int grid = grid4(num_sms, grid_cap);
+  switch (lanes4) {  // one lane per row (m = 4) spills at 48 registers: the two-column form runs it
+    case 2: cheb3_4<2>(A, m, z, zp, src, z1, c1, c2, mask, grid, st); return true;
+    case 4: cheb3_4<4>(A, m, z, zp, src, z1, c1, c2, mask, grid, st); return true;
+    case 8: cheb3_4<8>(A, m, z, zp, src, z1, c1, c2, mask, grid, st); return true;
+    default: return false;
+  }
+}
 
 bool launch_amg_resid4_split(int lanes4, const MatView &A, int32_t m, const double *z, const double *r, double *res,
                              uint32_t mask, int num_sms, int64_t grid_cap, cudaStream_t st) {

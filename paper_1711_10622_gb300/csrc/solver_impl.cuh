@@ -6,16 +6,18 @@
 // beta); every operator application is one GSpMV over the whole block, so the matrix is read
 // once per product for all m columns. Per iteration (right preconditioning, M^-1 = Chebyshev
 // polynomial or identity):
-//   k_p     p = r + beta (p - omega v)            [+ d0 = D^-1 p / theta, ph = d0]
-//   k_cheb  (cheb_steps - 1) x: GSpMV of d, fused 3-term update of d, z = ph, residual
+//   k_p     p = r + beta (p - omega v)            [+ z_1 = D^-1 p / theta]
+//   k_cheb3 (cheb_steps - 1) x: GSpMV of z_k, fused three-term update of z_k+1, the last into ph
 //   k_v     v = A ph,  (rhat, v)  -> alpha       (dot fused into the GSpMV epilogue)
 //   k_s     s = r - alpha v,  ||s||^2 -> half-step convergence   [+ Chebyshev start for s]
-//   k_cheb  ... z = sh
+//   k_cheb3 ... into sh
 //   k_t     t = A sh, (t, s), (t, t) -> omega     (dots fused into the GSpMV epilogue)
 //   k_xr    x += alpha ph + omega sh, r = s - omega t, ||r||^2, (rhat, r) -> convergence, rho
 // The per-column scalar step runs in the last block of each reduction (reduce.cuh), so the
 // scalars never leave the device; the host only reads the m convergence flags every
 // check_every iterations. Converged columns are frozen (their x is no longer updated).
+//
+// Where the matrix has row boxes (boxprod.cuh) the kernels with a GSpMV run in that form (solver_box.cu).
 //
 // The solver works on internal copies of B and X whose row stride is m rounded up to an even
 // width, so every kernel uses 16-byte row-segment accesses (m = 1 keeps stride 1).
@@ -30,6 +32,7 @@
 #include <vector>
 
 #include "amg_small.cuh"
+#include "boxsolve.cuh"
 #include "ens_internal.cuh"
 #include "reduce.cuh"
 #include "rowprod.cuh"
@@ -66,6 +69,55 @@ template <>
 struct Tiny<float> {
   static constexpr float v = 1e-30f;
 };
+
+// Per-column scalar steps, run by the last block of the reduction that completes their dot products.
+// After (rhat, v): alpha, or breakdown (x keeps its last finite iterate).
+template <typename T>
+__device__ __forceinline__ void step_alpha(const Cols<T> &cs, int l, T rv) {
+  if (cs.state[l] != ST_ACTIVE) return;
+  cs.iters[l] = cs.it[0] + 1;
+  const T al = cs.rho[l] / rv;
+  if (rv == T(0) || !isfinite(al)) {
+    cs.state[l] = ST_DONE;
+    cs.status[l] = ENS_COL_BREAKDOWN;
+    if (cs.it[0] == 0) cs.flags[l] |= FL_NOSTEP;
+    return;
+  }
+  cs.alpha[l] = al;
+}
+// After (t, s) and (t, t): omega, or breakdown before x is updated with a non-finite step.
+template <typename T>
+__device__ __forceinline__ void step_omega(const Cols<T> &cs, int l, T ts, T t2) {
+  if (cs.state[l] != ST_ACTIVE) return;
+  const T om = ts / t2;
+  if (t2 == T(0) || !isfinite(om)) {
+    cs.state[l] = ST_DONE;
+    cs.status[l] = ENS_COL_BREAKDOWN;
+    if (cs.it[0] == 0) cs.flags[l] |= FL_NOSTEP;
+    return;
+  }
+  cs.omega[l] = om;
+}
+// After ||b - A x||^2: the reported residual, or (outer) the convergence test of the refinement loop.
+template <typename T>
+__device__ __forceinline__ void residual_norm(const Cols<T> &cs, int l, T rr, int outer) {
+  if (outer) {
+    if (cs.state[l] != ST_ACTIVE) return;
+    cs.rn2[l] = rr;
+    cs.rn[l] = sqrt(rr);
+    cs.rn_inv[l] = rsqrt(rr);
+    if (!isfinite(rr)) {
+      cs.state[l] = ST_DONE;
+      cs.status[l] = ENS_COL_NONFINITE;
+    } else if (rr <= cs.thr2[l]) {
+      cs.state[l] = ST_DONE;
+      cs.status[l] = ENS_COL_CONVERGED;
+    }
+    return;
+  }
+  const int fl = cs.flags[l];
+  cs.relres[l] = (fl & FL_ZERO_B) ? 0.0 : (fl & FL_EARLY) ? (double)NAN : sqrt((double)rr / (double)cs.bn2[l]);
+}
 
 #define ENS_ROWS(i)                                                                           \
   for (int64_t i = (int64_t)blockIdx.x * (kThreads / LANES) + threadIdx.x / LANES; i < A.n; \
@@ -182,12 +234,12 @@ __global__ void ENS_TILE_BOUNDS(Arith)
 
 // ----------------------------------------------------------------------------- p update
 // p = r + beta (p - omega v) for active columns; with the preconditioner also the first
-// Chebyshev term d0 = D^-1 p / theta, written to da and to ph (= z).
+// Chebyshev iterate z_1 = D^-1 p / theta.
 template <typename Arith, int VEC, int LANES, bool PREC>
 __global__ void __launch_bounds__(kThreads)
     k_p(MatView A, int32_t m, const typename Arith::T *__restrict__ r, typename Arith::T *p,
-        const typename Arith::T *__restrict__ v, typename Arith::T *__restrict__ da, typename Arith::T *__restrict__ ph,
-        typename Arith::T inv_theta, Cols<typename Arith::T> cs) {
+        const typename Arith::T *__restrict__ v, typename Arith::T *__restrict__ z1, typename Arith::T inv_theta,
+        Cols<typename Arith::T> cs) {
   using T = typename Arith::T;
   const int32_t c = (threadIdx.x % LANES) * VEC;
   if (c >= m) return;
@@ -212,8 +264,7 @@ __global__ void __launch_bounds__(kThreads)
       const T sc = Arith::dinv(A, i) * inv_theta;
 #pragma unroll
       for (int q = 0; q < VEC; ++q) pv[q] *= sc;
-      store_vec<T, VEC>(da + i * m + c, pv);
-      store_vec<T, VEC>(ph + i * m + c, pv);
+      store_vec<T, VEC>(z1 + i * m + c, pv);
     }
   }
 }
@@ -254,6 +305,35 @@ __global__ void __launch_bounds__(kThreads, ChebBlocks<Arith, VEC>::value)
   });
 }
 
+// The same step as a three-term recurrence of the iterates (the solver's preconditioner):
+//   z_k+1 = (1 + c1) z_k - c1 z_k-1 + c2 D^-1 (src - A z_k),   z_0 = 0 (FIRST), z_1 = D^-1 src / theta
+// It is the iteration of k_cheb with d_k = z_k+1 - z_k and the residual taken anew: five FP64 operations per
+// element instead of six (with the widening of the product) and four streams instead of six. z_k+1 may overwrite
+// z_k-1, which only its own row reads.
+template <typename Arith, int VEC, int LANES, bool FIRST>
+__global__ void __launch_bounds__(kThreads, ChebBlocks<Arith, VEC>::value)
+    k_cheb3(MatView A, int32_t m, const typename Arith::T *__restrict__ z, const typename Arith::T *zp,
+            const typename Arith::T *__restrict__ src, typename Arith::T *z1, typename Arith::T c1, typename Arith::T c2,
+            uint32_t mask) {
+  using T = typename Arith::T;
+  tile_rows<Arith, VEC, LANES>(A, m, z, mask, [&](int64_t i, int32_t cc, const T (&w)[VEC]) {
+    T zv[VEC], sv[VEC], pv[VEC];
+    load_vec<T, VEC>(src + i * m + cc, sv);
+    load_vec<T, VEC>(z + i * m + cc, zv);
+    if (!FIRST) load_vec_rw<T, VEC>(zp + i * m + cc, pv);
+    const T g = c2 * Arith::dinv(A, i), a = T(1) + c1;
+#pragma unroll
+    for (int q = 0; q < VEC; ++q) {
+      const T t = FIRST ? a * zv[q] : fma(a, zv[q], -(c1 * pv[q]));
+      zv[q] = fma(g, sv[q] - w[q], t);
+    }
+    store_vec<T, VEC>(z1 + i * m + cc, zv);
+  });
+}
+
+// k_cheb3 in split float64 with four columns per lane; false (nothing launched) for other lane counts.
+bool launch_cheb3_4_split(int lanes4, const MatView &A, int32_t m, const double *z, const double *zp, const double *src,
+                          double *z1, double c1, double c2, uint32_t mask, int num_sms, int64_t grid_cap, cudaStream_t st);
 // One Chebyshev step (k_cheb) in split float64 with four columns per lane, lanes4 lanes per row (one
 // pass over a block of m columns, m a multiple of 4): 12-13 % faster than two columns per lane for
 // the standalone GSpMV at m = 8 and 16 on GB300. Compiled in solver_cheb4.cu for lanes4 = 2, 4, 8;
@@ -286,27 +366,14 @@ __global__ void ENS_TILE_BOUNDS(Arith)
 #pragma unroll
     for (int q = 0; q < VEC; ++q) acc[0][q] += h[q] * y[q];
   });
-  reduce_cols<T, 1, VEC, LANES>(acc, m, partials, counter, [&](int l, const ColTotals<T, 1> &t) {
-    if (cs.state[l] != ST_ACTIVE) return;
-    cs.iters[l] = cs.it[0] + 1;
-    const T rv = t.v[0][l];
-    const T al = cs.rho[l] / rv;
-    if (rv == T(0) || !isfinite(al)) {  // breakdown; x keeps its last finite iterate
-      cs.state[l] = ST_DONE;
-      cs.status[l] = ENS_COL_BREAKDOWN;
-      if (cs.it[0] == 0) cs.flags[l] |= FL_NOSTEP;
-      return;
-    }
-    cs.alpha[l] = al;
-  });
+  reduce_cols<T, 1, VEC, LANES>(acc, m, partials, counter, [&](int l, const ColTotals<T, 1> &t) { step_alpha<T>(cs, l, t.v[0][l]); });
 }
 
 // ----------------------------------------------------------------------------- s update
 template <typename Arith, int VEC, int LANES, bool PREC>
 __global__ void __launch_bounds__(kThreads)
     k_s(MatView A, int32_t m, const typename Arith::T *__restrict__ r, const typename Arith::T *__restrict__ v,
-        typename Arith::T *__restrict__ s, typename Arith::T *__restrict__ da, typename Arith::T *__restrict__ sh,
-        typename Arith::T inv_theta, Cols<typename Arith::T> cs, typename Arith::T *partials, unsigned *counter) {
+        typename Arith::T *__restrict__ s, typename Arith::T *__restrict__ z1, typename Arith::T inv_theta, Cols<typename Arith::T> cs, typename Arith::T *partials, unsigned *counter) {
   using T = typename Arith::T;
   const int32_t c = (threadIdx.x % LANES) * VEC;
   T acc[1][VEC], al[VEC];
@@ -330,8 +397,7 @@ __global__ void __launch_bounds__(kThreads)
         const T sc = Arith::dinv(A, i) * inv_theta;
 #pragma unroll
         for (int q = 0; q < VEC; ++q) rv[q] *= sc;
-        store_vec<T, VEC>(da + i * m + c, rv);
-        store_vec<T, VEC>(sh + i * m + c, rv);
+        store_vec<T, VEC>(z1 + i * m + c, rv);
       }
     }
   }
@@ -360,18 +426,8 @@ __global__ void ENS_TILE_BOUNDS(Arith)
       acc[1][q] += y[q] * y[q];
     }
   });
-  reduce_cols<T, 2, VEC, LANES>(acc, m, partials, counter, [&](int l, const ColTotals<T, 2> &tt) {
-    if (cs.state[l] != ST_ACTIVE) return;
-    const T t2 = tt.v[1][l];
-    const T om = tt.v[0][l] / t2;
-    if (t2 == T(0) || !isfinite(om)) {  // breakdown before x is updated with a non-finite step
-      cs.state[l] = ST_DONE;
-      cs.status[l] = ENS_COL_BREAKDOWN;
-      if (cs.it[0] == 0) cs.flags[l] |= FL_NOSTEP;
-      return;
-    }
-    cs.omega[l] = om;
-  });
+  reduce_cols<T, 2, VEC, LANES>(acc, m, partials, counter,
+                                [&](int l, const ColTotals<T, 2> &tt) { step_omega<T>(cs, l, tt.v[0][l], tt.v[1][l]); });
 }
 
 // ----------------------------------------------------------------------------- x, r update
@@ -534,25 +590,8 @@ __global__ void ENS_TILE_BOUNDS(Arith)
     }
     if (r) store_vec<T, VEC>(r + i * m + cc, y);
   });
-  reduce_cols<T, 1, VEC, LANES>(acc, m, partials, counter, [&](int l, const ColTotals<T, 1> &t) {
-    const T rr = t.v[0][l];
-    if (outer) {
-      if (cs.state[l] != ST_ACTIVE) return;
-      cs.rn2[l] = rr;
-      cs.rn[l] = sqrt(rr);
-      cs.rn_inv[l] = rsqrt(rr);
-      if (!isfinite(rr)) {
-        cs.state[l] = ST_DONE;
-        cs.status[l] = ENS_COL_NONFINITE;
-      } else if (rr <= cs.thr2[l]) {
-        cs.state[l] = ST_DONE;
-        cs.status[l] = ENS_COL_CONVERGED;
-      }
-      return;
-    }
-    const int fl = cs.flags[l];
-    cs.relres[l] = (fl & FL_ZERO_B) ? 0.0 : (fl & FL_EARLY) ? (double)NAN : sqrt((double)rr / (double)cs.bn2[l]);
-  });
+  reduce_cols<T, 1, VEC, LANES>(acc, m, partials, counter,
+                                [&](int l, const ColTotals<T, 1> &t) { residual_norm<T>(cs, l, t.v[0][l], outer); });
 }
 
 // ----------------------------------------------------------------------------- mixed precision
@@ -842,6 +881,8 @@ struct AmgCycle {
     bool split = false;     // float64 split arithmetic usable on this level
     bool as_split = false;  // ... and on its scaled copy
     int grid = 0, egrid = 0, cgrid = 0, sms = 1;
+    BoxPlan box, as_box;            // row boxes of the level and of its scaled copy
+    bool boxes = false, as_boxes = false;
     T *r = nullptr, *z = nullptr, *res = nullptr, *cres = nullptr, *da = nullptr, *db = nullptr;
   };
   std::vector<Level> lev;
@@ -920,7 +961,8 @@ struct AmgCycle {
     }
   }
 
-  cudaError_t setup(Scratch &sc, const ens_amg *H, int mp_, int vec_, int lanes_) {
+  // aligned: r and z of the fine level are 32-byte aligned.
+  cudaError_t setup(Scratch &sc, const ens_amg *H, int mp_, int vec_, int lanes_, bool aligned) {
     o = H->opts;
     mp = mp_;
     vec = vec_;
@@ -943,6 +985,15 @@ struct AmgCycle {
         L.As = view_of(h.As);
         L.as_split = use_split(h.As);
         L.as_mask = std::is_same<Arith, ArithF64Split>::value && L.as_split ? share_mask(native_share(h.As, mp)) : 0u;
+      }
+      if constexpr (std::is_same<Arith, ArithF32>::value || std::is_same<Arith, ArithF64Split>::value) {
+        const int dt = std::is_same<T, float>::value ? ENS_F32 : ENS_F64;
+        L.boxes = aligned && box_width<T>(mp) && use_box(h.A, mp, dt);
+        L.box = h.A->box;
+        if (h.As) {
+          L.as_boxes = aligned && box_width<T>(mp) && use_box(h.As, mp, dt);
+          L.as_box = h.As->box;
+        }
       }
       const int64_t rows_per_block = kThreads / lanes;
       const int64_t sms = h.A->num_sms;
@@ -975,6 +1026,12 @@ struct AmgCycle {
     if (steps == 2 && L.has_as) {  // both updates in one pass over the scaled copy
       const double sigma = theta / delta, rho_prev = 1.0 / sigma, rho = 1.0 / (2.0 * sigma - rho_prev);
       const T c1 = (T)(rho * rho_prev), c2 = (T)(2.0 * rho / delta), it = (T)(1.0 / theta);
+      if constexpr (std::is_same<Ar, ArithF32>::value || std::is_same<Ar, ArithF64Split>::value) {
+        if (L.as_boxes) {
+          launch_box_smooth2(L.as_box, L.As, inv_diag(L.A), mp, add, src, z, it, c1, c2, L.sms, st);
+          return;
+        }
+      }
       if (small(L)) {
         launch_small_smooth2(SmallLevel<T>{L.As.rp, L.As.ci, values(L.As), inv_diag(L.A), (int32_t)L.n, mp, Ln}, V, add, src, z, it, c1,
                              c2, st);
@@ -1035,6 +1092,12 @@ struct AmgCycle {
   // L.res = r - A z on level L
   template <typename Ar, int V, int Ln>
   void resid(const Level &L, const T *z, const T *r, cudaStream_t st) {
+    if constexpr (std::is_same<Ar, ArithF32>::value || std::is_same<Ar, ArithF64Split>::value) {
+      if (L.boxes) {
+        launch_box_amg_resid(L.box, L.A, mp, z, r, L.res, L.sms, st);
+        return;
+      }
+    }
     if (small(L)) {
       launch_small_resid(SmallLevel<T>{L.A.rp, L.A.ci, values(L.A), inv_diag(L.A), (int32_t)L.n, mp, Ln}, V, z, r, L.res, st);
       return;
@@ -1113,7 +1176,9 @@ struct Bicg {
   uint32_t mask = 0;  // native-DFMA sweeps of the split arithmetic (hybrid tiles)
   double theta = 1, delta = 1;
   cudaStream_t s = nullptr;
-  T *r, *rh, *p, *v, *ph, *s_, *sh, *t, *da, *db, *res;
+  T *r, *rh, *p, *v, *ph, *s_, *sh, *t, *da;
+  BoxPlan box;         // row boxes of the matrix
+  bool boxes = false;  // ... and whether the products use them
   T *partials;
   unsigned *counter;
   Cols<T> cs;
@@ -1139,9 +1204,13 @@ struct Bicg {
     cheb_steps = o.cheb_steps;
     theta = 0.5 * (o.cheb_hi + o.cheb_lo);
     delta = 0.5 * (o.cheb_hi - o.cheb_lo);
+    if constexpr (std::is_same<Arith, ArithF32>::value || std::is_same<Arith, ArithF64Split>::value) {
+      boxes = box_width<T>(mp) && use_box(M, mp, std::is_same<T, float>::value ? ENS_F32 : ENS_F64);
+      box = M->box;
+    }
     const size_t blk = (size_t)n * mp;
     cudaError_t e = cudaSuccess;
-    r = rh = p = v = ph = s_ = sh = t = da = db = res = nullptr;
+    r = rh = p = v = ph = s_ = sh = t = da = nullptr;
     if (outer_only) {
       prec = false;
       e = sc.get(&r, blk);
@@ -1153,17 +1222,16 @@ struct Bicg {
     use_amg = !outer_only && o.precond == ENS_PRECOND_AMG && M->amg != nullptr;
     if (outer_only) {
     } else if (prec) {
-      T **pb[] = {&ph, &sh, &da, &db, &res};
+      T **pb[] = {&ph, &sh, &da};
       for (T **b : pb)
         if (e == cudaSuccess) e = sc.get(b, blk);
     } else if (use_amg) {
       if (e == cudaSuccess) e = sc.get(&ph, blk);
       if (e == cudaSuccess) e = sc.get(&sh, blk);
-      if (e == cudaSuccess) e = amg.setup(sc, M->amg, mp, vec, lanes);
+      if (e == cudaSuccess) e = amg.setup(sc, M->amg, mp, vec, lanes, true);
     } else {
       ph = p;
       sh = s_;
-      da = db = res = nullptr;
     }
     // the same for every width (not the grids of this one): a server fits the workspace as beta + gamma m
     if (e == cudaSuccess) e = sc.get(&partials, (size_t)num_sms * std::max(4, TileBlocks<Arith>::value) * 3 * kMaxSolveM);
@@ -1199,35 +1267,73 @@ struct Bicg {
     return e;
   }
 
-  // Chebyshev application z = p(D^-1 A) D^-1 src; the first term is already in da and z.
+  // Where the first Chebyshev iterate of an application with result z goes: the iterates alternate between da and
+  // z so that the last one lands in z.
+  T *first_iterate(T *z) const { return cheb_steps % 2 == 0 ? da : z; }
+
+  // Chebyshev application z = p(D^-1 A) D^-1 src; the first iterate is already in first_iterate(z).
   template <int V, int L>
   void cheb(const T *src, T *z, cudaStream_t st) {
     const double sigma = theta / delta;
     double rho_prev = 1.0 / sigma;
-    T *din = da, *dout = db;
+    T *cur = first_iterate(z), *other = cur == z ? da : z;
     for (int k = 1; k < cheb_steps; ++k) {
       const double rho = 1.0 / (2.0 * sigma - rho_prev);
       const T c1 = (T)(rho * rho_prev), c2 = (T)(2.0 * rho / delta);
-      const bool first = k == 1, last = k == cheb_steps - 1;
       bool done = false;
+      if constexpr (std::is_same<Arith, ArithF32>::value || std::is_same<Arith, ArithF64Split>::value) {
+        if (boxes) {
+          launch_box_cheb(box, A, mp, cur, k == 1 ? nullptr : other, src, other, c1, c2, num_sms, st);
+          done = true;
+        }
+      }
       if constexpr (std::is_same<Arith, ArithF64Split>::value && V == 2 && L >= 2) {
-        if (mp % 4 == 0)
-          done = launch_cheb4_split(L / 2, first, last, A, mp, din, dout, src, res, z, c1, c2, mask, num_sms,
-                                    tile_count(n, L / 2), st);
+        if (!done && mp % 4 == 0)
+          done = launch_cheb3_4_split(L / 2, A, mp, cur, k == 1 ? nullptr : other, src, other, c1, c2, mask, num_sms,
+                                      tile_count(n, L / 2), st);
       }
       if (done)
         ;
-      else if (first && last)
-        k_cheb<Arith, V, L, true, true><<<lgrid, kThreads, 0, st>>>(A, mp, din, dout, src, res, z, c1, c2, mask);
-      else if (first)
-        k_cheb<Arith, V, L, true, false><<<lgrid, kThreads, 0, st>>>(A, mp, din, dout, src, res, z, c1, c2, mask);
-      else if (last)
-        k_cheb<Arith, V, L, false, true><<<lgrid, kThreads, 0, st>>>(A, mp, din, dout, src, res, z, c1, c2, mask);
+      else if (k == 1)
+        k_cheb3<Arith, V, L, true><<<lgrid, kThreads, 0, st>>>(A, mp, cur, nullptr, src, other, c1, c2, mask);
       else
-        k_cheb<Arith, V, L, false, false><<<lgrid, kThreads, 0, st>>>(A, mp, din, dout, src, res, z, c1, c2, mask);
-      std::swap(din, dout);
+        k_cheb3<Arith, V, L, false><<<lgrid, kThreads, 0, st>>>(A, mp, cur, other, src, other, c1, c2, mask);
+      std::swap(cur, other);
       rho_prev = rho;
     }
+  }
+
+  // v = A ph with (rhat, v), and t = A sh with (t, s), (t, t).
+  template <int V, int L>
+  void product_v(cudaStream_t st) {
+    if constexpr (std::is_same<Arith, ArithF32>::value || std::is_same<Arith, ArithF64Split>::value) {
+      if (boxes) {
+        launch_box_v(box, A, mp, ph, v, rh, cs, partials, counter, num_sms, st);
+        return;
+      }
+    }
+    k_v<Arith, V, L><<<tgrid, kThreads, 0, st>>>(A, mp, ph, v, rh, cs, partials, counter, mask);
+  }
+  template <int V, int L>
+  void product_t(cudaStream_t st) {
+    if constexpr (std::is_same<Arith, ArithF32>::value || std::is_same<Arith, ArithF64Split>::value) {
+      if (boxes) {
+        launch_box_t(box, A, mp, sh, t, s_, cs, partials, counter, num_sms, st);
+        return;
+      }
+    }
+    k_t<Arith, V, L><<<tgrid, kThreads, 0, st>>>(A, mp, sh, t, s_, cs, partials, counter, mask);
+  }
+  // ||b - A x||^2 (and the residual block r_out of the refinement loop).
+  template <int V, int L>
+  void residual(const T *b, const T *x, T *r_out, int outer, cudaStream_t st) {
+    if constexpr (std::is_same<Arith, ArithF64Split>::value) {
+      if (boxes) {
+        launch_box_resid(box, A, mp, b, x, r_out, outer, cs, partials, counter, num_sms, st);
+        return;
+      }
+    }
+    k_resid<Arith, V, L><<<tgrid, kThreads, 0, st>>>(A, mp, b, x, r_out, outer, cs, partials, counter, mask);
   }
 
   // One BiCGStab iteration for every column (frozen columns are no-ops); the iteration number
@@ -1237,21 +1343,21 @@ struct Bicg {
     return with_vl<kVec4>(vec, lanes, [&](auto Vc, auto Lc) {
       constexpr int V = decltype(Vc)::value, L = decltype(Lc)::value;
       if (prec) {
-        k_p<Arith, V, L, true><<<grid, kThreads, 0, st>>>(A, mp, r, p, v, da, ph, inv_theta, cs);
+        k_p<Arith, V, L, true><<<grid, kThreads, 0, st>>>(A, mp, r, p, v, first_iterate(ph), inv_theta, cs);
         cheb<V, L>(p, ph, st);
       } else {
-        k_p<Arith, V, L, false><<<grid, kThreads, 0, st>>>(A, mp, r, p, v, da, ph, inv_theta, cs);
+        k_p<Arith, V, L, false><<<grid, kThreads, 0, st>>>(A, mp, r, p, v, nullptr, inv_theta, cs);
         if (use_amg) amg.template cycle<V, L>(0, p, ph, st);
       }
-      k_v<Arith, V, L><<<tgrid, kThreads, 0, st>>>(A, mp, ph, v, rh, cs, partials, counter, mask);
+      this->template product_v<V, L>(st);
       if (prec) {
-        k_s<Arith, V, L, true><<<grid, kThreads, 0, st>>>(A, mp, r, v, s_, da, sh, inv_theta, cs, partials, counter);
+        k_s<Arith, V, L, true><<<grid, kThreads, 0, st>>>(A, mp, r, v, s_, first_iterate(sh), inv_theta, cs, partials, counter);
         cheb<V, L>(s_, sh, st);
       } else {
-        k_s<Arith, V, L, false><<<grid, kThreads, 0, st>>>(A, mp, r, v, s_, da, sh, inv_theta, cs, partials, counter);
+        k_s<Arith, V, L, false><<<grid, kThreads, 0, st>>>(A, mp, r, v, s_, nullptr, inv_theta, cs, partials, counter);
         if (use_amg) amg.template cycle<V, L>(0, s_, sh, st);
       }
-      k_t<Arith, V, L><<<tgrid, kThreads, 0, st>>>(A, mp, sh, t, s_, cs, partials, counter, mask);
+      this->template product_t<V, L>(st);
       k_xr<Arith, V, L><<<grid, kThreads, 0, st>>>(A, mp, x, ph, sh, s_, t, r, rh, max_iter, cs, partials, counter, lc);
       return cudaGetLastError();
     });
@@ -1385,7 +1491,7 @@ struct Bicg {
         k_colsum<Arith, V, L><<<grid, kThreads, 0, st>>>(A, mp, x, (T)(1.0 / (double)n), cs, partials, counter);
       }
       k_fix<Arith, V, L><<<grid, kThreads, 0, st>>>(A, mp, x, singular, cs);
-      k_resid<Arith, V, L><<<tgrid, kThreads, 0, st>>>(A, mp, b, x, nullptr, 0, cs, partials, counter, mask);
+      this->template residual<V, L>(b, x, nullptr, 0, st);
       return cudaGetLastError();
     });
   }
@@ -1394,7 +1500,7 @@ struct Bicg {
     if (!st) st = s;
     return with_vl<kVec4>(vec, lanes, [&](auto Vc, auto Lc) {
       constexpr int V = decltype(Vc)::value, L = decltype(Lc)::value;
-      k_resid<Arith, V, L><<<tgrid, kThreads, 0, st>>>(A, mp, b, x, r, 1, cs, partials, counter, mask);
+      this->template residual<V, L>(b, x, r, 1, st);
       return cudaGetLastError();
     });
   }
