@@ -104,6 +104,23 @@ __device__ __forceinline__ void box_acc2(uint64_t ah, uint64_t al, uint64_t xh, 
   sh = s;
 }
 
+// hi + lo as a double without the FP64 pipe: TwoSum makes |lo| at most half an ulp of hi, which in units of the
+// double's last place is an integer below 2^29; it is added to the widened hi as an integer. Rounds like the FP64
+// addition. Not for hi outside box_sum_range's window, and not for a power of two, where a negative lo would
+// borrow from the exponent (box_mantissa 0): the caller sends those to split_to_double.
+__device__ __forceinline__ double box_add(float &hi, float lo) {
+  float s, e;
+  two_sum(hi, lo, s, e);
+  hi = s;
+  const uint32_t b = __float_as_uint(s);
+  // e / 2^(E - 52) with the sign of s, E the exponent of s
+  const float scale = __uint_as_float((((52u + 254u) << 23) - (b & 0x7F800000u)) | (b & 0x80000000u));
+  const int32_t r = __float2int_rn(e * scale);
+  const int64_t w = __double_as_longlong(box_widen(s));
+  return __longlong_as_double(w + (int64_t)r);
+}
+__device__ __forceinline__ uint32_t box_mantissa(float hi) { return __float_as_uint(hi) << 9; }
+
 // N consecutive elements, of which those at column offsets below `left` exist (the others keep what they held);
 // ACC elements per access, aligned to it: one 32-byte access for four doubles or eight floats. Volatile: these
 // are prefetches, and the compiler would otherwise sink them to the first use of their values.
@@ -175,9 +192,12 @@ struct BoxShape {
 // takes every chunk of its boxes in turn (matrix entries read once); otherwise one chunk, blockIdx.x modulo the
 // chunks, so that a thread keeps its columns. ACC: elements per global access of X, to which its rows are
 // aligned. FULL: m is a multiple of CW (checks of the last chunk cost 8-11 % where they are not needed). K0: slots
-// per row where it is known at compile time (0: B.K).
-template <typename T, int CW, int ACC, bool FULL, int K0, bool INNER, typename Epi>
-__device__ __forceinline__ void box_rows(const BoxPlan &B, const MatView &A, int32_t m, const T *__restrict__ X, Epi &&epi) {
+// per row where it is known at compile time (0: B.K). ADD64: a float64 sum is widened with one FP64 addition; else
+// in integer arithmetic, which frees the FP64 pipe for an epilogue that needs it (the solver's Chebyshev step 235 ->
+// 212 us on cubes 192 x 128 x 96, m = 8) but costs the plain product 5 %. ahead(row, first column) runs before the
+// products: the epilogue's own reads can be asked for there.
+template <typename T, int CW, int ACC, bool FULL, int K0, bool INNER, bool ADD64, typename Pre, typename Epi>
+__device__ __forceinline__ void box_rows(const BoxPlan &B, const MatView &A, int32_t m, const T *__restrict__ X, Pre &&ahead, Epi &&epi) {
   using S = BoxShape<T, CW>;
   constexpr bool kF64 = S::kF64;
   constexpr int NT = S::kThr, NP = S::kPlanes, PL = S::kPlane;
@@ -278,6 +298,7 @@ __device__ __forceinline__ void box_rows(const BoxPlan &B, const MatView &A, int
       const V *const va = reinterpret_cast<const V *>(en) + r;
       const uint16_t *const loc = reinterpret_cast<const uint16_t *>(en + kBoxRows * K * sizeof(V)) + r;
       const int64_t i = reinterpret_cast<const int32_t *>(en + kBoxRows * K * (sizeof(V) + 2))[r];
+      ahead(i, c);
       T y[CW];
       if constexpr (kF64) {
         uint64_t sh[2 * NP], sl[2 * NP];
@@ -315,8 +336,21 @@ __device__ __forceinline__ void box_rows(const BoxPlan &B, const MatView &A, int
           f2_unpack(sl[p], w[2 * p], w[2 * p + 1]);
           if (FULL || c + 4 * (p / 2) < m) worst = max(worst, max(box_sum_range(h[2 * p]), box_sum_range(h[2 * p + 1])));
         }
+        if constexpr (ADD64) {
 #pragma unroll
-        for (int q = 0; q < CW; ++q) y[q] = box_widen(h[q]) + box_widen(w[q]);
+          for (int q = 0; q < CW; ++q) y[q] = box_widen(h[q]) + box_widen(w[q]);
+        } else {
+          uint32_t least = 0xFFFFFFFFu;
+          float g[CW];
+#pragma unroll
+          for (int q = 0; q < CW; ++q) {
+            g[q] = h[q];
+            y[q] = box_add(g[q], w[q]);
+            least = min(least, box_mantissa(g[q]));
+            worst = max(worst, box_sum_range(g[q]));
+          }
+          if (least == 0u) worst = kBoxSumWindow;
+        }
         if (worst >= kBoxSumWindow) {
           // tiny and zero sums; values outside the split range or sums beyond float: native DFMA
           const int32_t j0 = __ldg(A.rp + i), j1 = __ldg(A.rp + i + 1);

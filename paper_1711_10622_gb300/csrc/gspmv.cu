@@ -94,7 +94,7 @@ __global__ void __launch_bounds__(kThreads)
 template <typename T, int CW, int ACC, bool FULL, int K0>
 __global__ void __launch_bounds__(BoxShape<T, CW>::kThr, BoxShape<T, CW>::kBlocks)
     gspmv_kernel_box(BoxPlan B, MatView A, int32_t m, const T *__restrict__ X, T *__restrict__ Y) {
-  box_rows<T, CW, ACC, FULL, K0, true>(B, A, m, X, [&](int64_t i, int32_t c, const T (&y)[CW]) {
+  box_rows<T, CW, ACC, FULL, K0, true, true>(B, A, m, X, [](int64_t, int32_t) {}, [&](int64_t i, int32_t c, const T (&y)[CW]) {
     store_cols_cs<T, CW, ACC>(Y + i * m + c, FULL ? CW : m - c, y);
   });
 }

@@ -14,6 +14,12 @@ namespace ens {
 namespace solver {
 namespace {
 
+// Asks for the line of a row of another block that the epilogue will read, while the products are formed.
+template <typename T>
+__device__ __forceinline__ void ask(const T *p) {
+  asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+}
+
 // CW elements as 32-byte (float32 x 4: 16-byte) accesses.
 template <typename T, int CW>
 __device__ __forceinline__ void load_row(const T *p, T (&v)[CW]) {
@@ -111,7 +117,7 @@ ENS_BOX_KERNEL(T, CW)
          unsigned *counter) {
   T acc[1][CW];
   clear<T, CW>(acc[0]);
-  box_rows<T, CW, wide<T, CW>(), true, K0, false>(B, A, m, ph, [&](int64_t i, int32_t c, const T (&y)[CW]) {
+  box_rows<T, CW, wide<T, CW>(), true, K0, false, false>(B, A, m, ph, [&](int64_t i, int32_t c) { ask(rh + i * m + c); }, [&](int64_t i, int32_t c, const T (&y)[CW]) {
     T h[CW];
     load_row<T, CW>(rh + i * m + c, h);
     store_row<T, CW>(v + i * m + c, y);
@@ -128,7 +134,7 @@ ENS_BOX_KERNEL(T, CW)
   T acc[2][CW];
   clear<T, CW>(acc[0]);
   clear<T, CW>(acc[1]);
-  box_rows<T, CW, wide<T, CW>(), true, K0, false>(B, A, m, sh, [&](int64_t i, int32_t c, const T (&y)[CW]) {
+  box_rows<T, CW, wide<T, CW>(), true, K0, false, false>(B, A, m, sh, [&](int64_t i, int32_t c) { ask(s + i * m + c); }, [&](int64_t i, int32_t c, const T (&y)[CW]) {
     T sv[CW];
     load_row<T, CW>(s + i * m + c, sv);
     store_row<T, CW>(t + i * m + c, y);
@@ -147,7 +153,7 @@ ENS_BOX_KERNEL(T, CW)
              T *partials, unsigned *counter) {
   T acc[1][CW];
   clear<T, CW>(acc[0]);
-  box_rows<T, CW, wide<T, CW>(), true, K0, false>(B, A, m, x, [&](int64_t i, int32_t c, const T (&ax)[CW]) {
+  box_rows<T, CW, wide<T, CW>(), true, K0, false, false>(B, A, m, x, [&](int64_t i, int32_t c) { ask(b + i * m + c); }, [&](int64_t i, int32_t c, const T (&ax)[CW]) {
     T y[CW];
     load_row<T, CW>(b + i * m + c, y);
 #pragma unroll
@@ -172,7 +178,11 @@ ENS_BOX_KERNEL(T, CW)
     else
       return A.dinv32;
   }();
-  box_rows<T, CW, wide<T, CW>(), true, K0, true>(B, A, m, z, [&](int64_t i, int32_t c, const T (&w)[CW]) {
+  auto ahead = [&](int64_t i, int32_t c) {
+    ask(src + i * m + c);
+    if (!FIRST) ask(zp + i * m + c);
+  };
+  box_rows<T, CW, wide<T, CW>(), true, K0, true, false>(B, A, m, z, ahead, [&](int64_t i, int32_t c, const T (&w)[CW]) {
     T zv[CW], pv[CW], sv[CW];
     load_row<T, CW>(src + i * m + c, sv);
     load_row<T, CW>(z + i * m + c, zv);
@@ -190,7 +200,7 @@ ENS_BOX_KERNEL(T, CW)
 template <typename T, int CW, int K0>
 ENS_BOX_KERNEL(T, CW)
     kb_amg_resid(BoxPlan B, MatView A, int32_t m, const T *__restrict__ z, const T *__restrict__ r, T *__restrict__ res) {
-  box_rows<T, CW, wide<T, CW>(), true, K0, true>(B, A, m, z, [&](int64_t i, int32_t c, const T (&w)[CW]) {
+  box_rows<T, CW, wide<T, CW>(), true, K0, true, false>(B, A, m, z, [&](int64_t i, int32_t c) { ask(r + i * m + c); }, [&](int64_t i, int32_t c, const T (&w)[CW]) {
     T rv[CW];
     load_row<T, CW>(r + i * m + c, rv);
 #pragma unroll
@@ -202,7 +212,10 @@ ENS_BOX_KERNEL(T, CW)
 template <typename T, int CW, int K0, bool ADD>
 ENS_BOX_KERNEL(T, CW)
     kb_amg_smooth2(BoxPlan B, MatView As, const T *__restrict__ dinv, int32_t m, const T *__restrict__ src, T *z, T inv_theta, T c1, T c2) {
-  box_rows<T, CW, wide<T, CW>(), true, K0, true>(B, As, m, src, [&](int64_t i, int32_t c, const T (&w)[CW]) {
+  auto ahead = [&](int64_t i, int32_t c) {
+    if (ADD) ask(z + i * m + c);
+  };
+  box_rows<T, CW, wide<T, CW>(), true, K0, true, false>(B, As, m, src, ahead, [&](int64_t i, int32_t c, const T (&w)[CW]) {
     T sv[CW], zv[CW];
     load_row<T, CW>(src + i * m + c, sv);
     if (ADD) load_row<T, CW>(z + i * m + c, zv);

@@ -236,7 +236,7 @@ __global__ void ENS_TILE_BOUNDS(Arith)
 // p = r + beta (p - omega v) for active columns; with the preconditioner also the first
 // Chebyshev iterate z_1 = D^-1 p / theta.
 template <typename Arith, int VEC, int LANES, bool PREC>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, 4)
     k_p(MatView A, int32_t m, const typename Arith::T *__restrict__ r, typename Arith::T *p,
         const typename Arith::T *__restrict__ v, typename Arith::T *__restrict__ z1, typename Arith::T inv_theta,
         Cols<typename Arith::T> cs) {
@@ -371,16 +371,19 @@ __global__ void ENS_TILE_BOUNDS(Arith)
 
 // ----------------------------------------------------------------------------- s update
 template <typename Arith, int VEC, int LANES, bool PREC>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, 4)
     k_s(MatView A, int32_t m, const typename Arith::T *__restrict__ r, const typename Arith::T *__restrict__ v,
         typename Arith::T *__restrict__ s, typename Arith::T *__restrict__ z1, typename Arith::T inv_theta, Cols<typename Arith::T> cs, typename Arith::T *partials, unsigned *counter) {
   using T = typename Arith::T;
   const int32_t c = (threadIdx.x % LANES) * VEC;
   T acc[1][VEC], al[VEC];
+  int32_t on[VEC];  // an integer: tested per element, a floating comparison would take the FP64 pipe again
 #pragma unroll
   for (int q = 0; q < VEC; ++q) {
     acc[0][q] = T(0);
     al[q] = (c + q < m && cs.state[c + q] == ST_ACTIVE) ? cs.alpha[c + q] : T(0);
+    on[q] = al[q] != T(0) ? 1 : 0;
+    asm volatile("" : "+r"(on[q]));
   }
   if (c < m) {
     ENS_ROWS(i) {
@@ -389,7 +392,7 @@ __global__ void __launch_bounds__(kThreads)
       load_vec<T, VEC>(v + i * m + c, vv);
 #pragma unroll
       for (int q = 0; q < VEC; ++q) {
-        rv[q] = al[q] != T(0) ? rv[q] - al[q] * vv[q] : rv[q];
+        rv[q] = on[q] ? rv[q] - al[q] * vv[q] : rv[q];
         acc[0][q] += rv[q] * rv[q];
       }
       store_vec<T, VEC>(s + i * m + c, rv);
@@ -1168,6 +1171,9 @@ struct Bicg {
   MatView A;
   int64_t n = 0;
   int mp = 0, vec = 2, lanes = 1, grid = 0, tgrid = 0, lgrid = 0;  // grid: streaming kernels, tgrid / lgrid: GSpMV kernels
+  // The vector updates k_p and k_s take four columns per thread in float64 too where the width allows: at two,
+  // 1024 threads per SM keep only 48 KB of loads in flight.
+  int svec = 2, slanes = 1, sgrid = 0;
   int num_sms = 1;
   bool prec = false;
   bool use_amg = false;
@@ -1194,10 +1200,14 @@ struct Bicg {
     vec = mp == 1 ? 1 : (kVec4 && mp % 4 == 0) ? 4 : 2;
     lanes = 1;
     while (lanes * vec < mp) lanes <<= 1;
+    svec = mp % 4 == 0 ? 4 : vec;
+    slanes = 1;
+    while (slanes * svec < mp) slanes <<= 1;
     num_sms = M->num_sms;
     // no more blocks than the rows fill: an idle block of a reduction still adds its zeros and its partial
     const int64_t tiles = tile_count(n, lanes), need = (n * lanes + kThreads - 1) / kThreads;
     grid = (int)std::min<int64_t>((int64_t)M->num_sms * 4, need);
+    sgrid = (int)std::min<int64_t>((int64_t)M->num_sms * 4, (n * slanes + kThreads - 1) / kThreads);
     tgrid = (int)std::min<int64_t>((int64_t)M->num_sms * TileBlocks<Arith>::value, tiles);
     lgrid = (int)std::min<int64_t>((int64_t)M->num_sms * LightBlocks<Arith>::value, tiles);
     prec = o.precond == ENS_PRECOND_CHEBYSHEV;
@@ -1340,27 +1350,50 @@ struct Bicg {
   // lives on the device, so the same launches can be captured once and replayed.
   cudaError_t iteration(T *x, int max_iter, cudaStream_t st, LoopCond lc = LoopCond{}) {
     const T inv_theta = (T)(1.0 / theta);
-    return with_vl<kVec4>(vec, lanes, [&](auto Vc, auto Lc) {
+    // the vector updates are the same code in every float64 arithmetic
+    using Ar = typename std::conditional<std::is_same<T, float>::value, ArithF32, ArithF64Native>::type;
+    auto stream = [&](auto &&launch) { return with_vl<true>(svec, slanes, launch); };
+    auto products = [&](auto &&launch) { return with_vl<kVec4>(vec, lanes, launch); };
+    cudaError_t e = stream([&](auto Vc, auto Lc) {
       constexpr int V = decltype(Vc)::value, L = decltype(Lc)::value;
-      if (prec) {
-        k_p<Arith, V, L, true><<<grid, kThreads, 0, st>>>(A, mp, r, p, v, first_iterate(ph), inv_theta, cs);
-        cheb<V, L>(p, ph, st);
-      } else {
-        k_p<Arith, V, L, false><<<grid, kThreads, 0, st>>>(A, mp, r, p, v, nullptr, inv_theta, cs);
-        if (use_amg) amg.template cycle<V, L>(0, p, ph, st);
-      }
-      this->template product_v<V, L>(st);
-      if (prec) {
-        k_s<Arith, V, L, true><<<grid, kThreads, 0, st>>>(A, mp, r, v, s_, first_iterate(sh), inv_theta, cs, partials, counter);
-        cheb<V, L>(s_, sh, st);
-      } else {
-        k_s<Arith, V, L, false><<<grid, kThreads, 0, st>>>(A, mp, r, v, s_, nullptr, inv_theta, cs, partials, counter);
-        if (use_amg) amg.template cycle<V, L>(0, s_, sh, st);
-      }
-      this->template product_t<V, L>(st);
-      k_xr<Arith, V, L><<<grid, kThreads, 0, st>>>(A, mp, x, ph, sh, s_, t, r, rh, max_iter, cs, partials, counter, lc);
+      if (prec)
+        k_p<Ar, V, L, true><<<sgrid, kThreads, 0, st>>>(A, mp, r, p, v, first_iterate(ph), inv_theta, cs);
+      else
+        k_p<Ar, V, L, false><<<sgrid, kThreads, 0, st>>>(A, mp, r, p, v, nullptr, inv_theta, cs);
       return cudaGetLastError();
     });
+    if (e == cudaSuccess)
+      e = products([&](auto Vc, auto Lc) {
+        constexpr int V = decltype(Vc)::value, L = decltype(Lc)::value;
+        if (prec) cheb<V, L>(p, ph, st);
+        if (use_amg) amg.template cycle<V, L>(0, p, ph, st);
+        this->template product_v<V, L>(st);
+        return cudaGetLastError();
+      });
+    if (e == cudaSuccess)
+      e = stream([&](auto Vc, auto Lc) {
+        constexpr int V = decltype(Vc)::value, L = decltype(Lc)::value;
+        if (prec)
+          k_s<Ar, V, L, true><<<sgrid, kThreads, 0, st>>>(A, mp, r, v, s_, first_iterate(sh), inv_theta, cs, partials, counter);
+        else
+          k_s<Ar, V, L, false><<<sgrid, kThreads, 0, st>>>(A, mp, r, v, s_, nullptr, inv_theta, cs, partials, counter);
+        return cudaGetLastError();
+      });
+    if (e == cudaSuccess)
+      e = products([&](auto Vc, auto Lc) {
+        constexpr int V = decltype(Vc)::value, L = decltype(Lc)::value;
+        if (prec) cheb<V, L>(s_, sh, st);
+        if (use_amg) amg.template cycle<V, L>(0, s_, sh, st);
+        this->template product_t<V, L>(st);
+        return cudaGetLastError();
+      });
+    if (e == cudaSuccess)
+      e = products([&](auto Vc, auto Lc) {  // six blocks in: four columns would not leave four blocks per SM
+        constexpr int V = decltype(Vc)::value, L = decltype(Lc)::value;
+        k_xr<Ar, V, L><<<grid, kThreads, 0, st>>>(A, mp, x, ph, sh, s_, t, r, rh, max_iter, cs, partials, counter, lc);
+        return cudaGetLastError();
+      });
+    return e;
   }
 
   cudaError_t states(std::vector<int32_t> &h) {
