@@ -113,6 +113,18 @@ def test_ranges(ens, m):
             _check(o, one.cpu().numpy(), ens.gspmv(A, one).cpu().numpy())
 
 
+@pytest.mark.parametrize("ex", [-72, -71, -70, -57, -56, -55])
+def test_smallest_products(ens, ex):
+    """Matrix values at the bottom of the split range (2^-40) times values around the bottom of X's window: the
+    error terms of the products must not fall below the smallest floats."""
+    op = _op("dirichlet41")
+    val = np.ldexp(op.val / np.abs(op.val).min(), -40)
+    op = gen.Operator(op.name, op.shape, op.bcs, op.row_ptr, op.col_idx, val, False)
+    X = np.ldexp(1.0 + np.random.default_rng(3).random((op.n, 8)), ex) * np.where(np.arange(op.n)[:, None] % 3 == 0, -1.0, 1.0)
+    with ens.Matrix.from_operator(op) as A:
+        _check(op, X, ens.gspmv(A, torch.from_numpy(X).cuda()).cpu().numpy())
+
+
 @pytest.mark.parametrize("dtype", [np.float64, np.float32])
 def test_nonfinite(ens, dtype):
     """Infinities and NaN reach exactly the rows whose entries name them, as in the definition."""
