@@ -41,9 +41,9 @@ constexpr int kBoxRows = 256, kBoxCols = 576, kBoxLineX = 16, kBoxLinesY = 4, kB
 constexpr int kBoxMaxLen = 16;       // longest row with a plan
 constexpr int64_t kBoxMinRows = 65536;  // fewer than 256 boxes leave SMs idle
 
-// X values of the split form: |x| in [2^-56, 2^88) or 0. Matrix values are at least 2^-40, so a product is at least
-// 2^-96 and its error terms, down to 2^-144, stay above the spacing of the smallest floats (2^-149).
-constexpr uint32_t kBoxELo = 967u, kBoxEHi = 1111u;  // biased exponents of 2^-56 and 2^88
+// X values of the split form: |x| in [2^-40, 2^88), as in split_range, or 0. Matrix values are at least 2^-40, so a
+// product is at least 2^-80 and what is lost below the smallest normal float (2^-126) stays below 2^-46 of it.
+constexpr uint32_t kBoxELo = kSplitELo, kBoxEHi = kSplitELo + 128u;  // biased exponents of 2^-40 and 2^88
 
 // x -> hi + lo: hi = x rounded to 24 bits (half up on the 29 bits below), lo = the remainder rounded to 24
 // bits: |x - hi - lo| <= 2^-49 |x|, a quarter of split_f64's truncation. The remainder is the low 29 bits as a
