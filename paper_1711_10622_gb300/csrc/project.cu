@@ -10,6 +10,7 @@
 #include <new>
 #include <vector>
 
+#include "boxprod.cuh"
 #include "ens_internal.cuh"
 #include "ensemble_project.h"
 #include "rowprod.cuh"
@@ -306,6 +307,241 @@ __global__ void __launch_bounds__(kThreads)
   }
 }
 
+// Grids without solid cells: the place of a thread is its cell x and states c on a line, and the lines y0 .. y1 of plane
+// z that it takes; a cell costs no index divisions and which faces are open follows from the position. One block:
+// up to 256 (x, states) pairs.
+struct March {
+  int32_t x, c, y0, y1, z;
+  bool on;
+};
+template <int VEC, int MARCH>
+__device__ __forceinline__ March march_place(const GridView &g, int32_t m) {
+  const int32_t groups = m / VEC, width = g.N[0] * groups;
+  const int32_t xb = (width + (int32_t)blockDim.x - 1) / (int32_t)blockDim.x, yc = (g.N[1] + MARCH - 1) / MARCH;
+  const int32_t bx = blockIdx.x % xb, rest = blockIdx.x / xb;
+  const int32_t e = bx * (int32_t)blockDim.x + (int32_t)threadIdx.x;
+  March p;
+  p.on = e < width;
+  p.x = e / groups;
+  p.c = (e - p.x * groups) * VEC;
+  p.y0 = (rest % yc) * MARCH;
+  p.y1 = min(p.y0 + MARCH, g.N[1]);
+  p.z = rest / yc;
+  return p;
+}
+
+// Four (VEC = 2: two) values as hi and lo floats; values outside the split range come out as NaN.
+template <int VEC>
+__device__ __forceinline__ void split_states(const double (&u)[VEC], float (&h)[VEC], float (&l)[VEC]) {
+  const double x[4] = {u[0], u[1], u[VEC - 2], u[VEC - 1]};
+  float4 a, b;
+  box_split4(x, a, b);
+  h[0] = a.x, h[1] = a.y, l[0] = b.x, l[1] = b.y;
+  if constexpr (VEC == 4) h[2] = a.z, h[3] = a.w, l[2] = b.z, l[3] = b.w;
+}
+
+// The divergence with split-float products (box_acc2), marching along y: five face values are read and converted per
+// cell, the sixth is the previous line's. Bound by issue (about 110 instructions per cell and state) and, beside it,
+// HBM. Lines per thread on the 128^3 channel, m = 8: 1 181 us, 2 154, 4 137, 8 130.
+constexpr int kDivMarch = 8;
+template <int VEC, int MARCH>
+__global__ void __launch_bounds__(256, VEC == 4 ? 2 : 4)
+    k_divergence_march(GridView g, int32_t m, double scale, const double *__restrict__ U, const double *__restrict__ V,
+                       const double *__restrict__ W, double *__restrict__ D) {
+  constexpr int NP = VEC / 2;
+  constexpr uint64_t kSign2 = 0x8000000080000000ull;
+  const March p = march_place<VEC, MARCH>(g, m);
+  if (!p.on) return;
+  const int32_t nx = g.N[0], ny = g.N[1], nz = g.N[2];
+  const bool wx = g.bc[0] == ENS_BC_WALL, wy = g.bc[1] == ENS_BC_WALL, wz = g.bc[2] == ENS_BC_WALL;
+  const bool lx = !(wx && p.x == 0), hx = !(wx && p.x == nx - 1), lz = !(wz && p.z == 0), hz = !(wz && p.z == nz - 1);
+  const int32_t xh = g.bc[0] == ENS_BC_PERIODIC && p.x + 1 == nx ? 0 : p.x + 1, zh = g.bc[2] == ENS_BC_PERIODIC && p.z + 1 == nz ? 0 : p.z + 1;
+  const double *pu = U + (p.x + (int64_t)g.F[0] * (p.y0 + (int64_t)ny * p.z)) * m + p.c;
+  const double *pv = V + (p.x + (int64_t)nx * ((int64_t)g.F[1] * p.z)) * m + p.c;  // line 0
+  const double *pw = W + (p.x + (int64_t)nx * (p.y0 + (int64_t)ny * p.z)) * m + p.c;
+  double *pd = D + (p.x + (int64_t)nx * (p.y0 + (int64_t)ny * p.z)) * m + p.c;
+  const int64_t du = (int64_t)(xh - p.x) * m, dw = (int64_t)(zh - p.z) * nx * ny * m, sv = (int64_t)nx * m, su = (int64_t)g.F[0] * m;
+  const uint64_t zero = (uint64_t)(uint32_t)(m >> 31);
+  const double ay = g.area[1][p.x + (int64_t)nx * p.z];
+  float ayh, ayl;
+  box_split(ay, ayh, ayl);
+  const uint64_t YH = f2_pack(ayh, ayh), YL = f2_pack(ayl, ayl);
+  float vh[VEC], vl[VEC];  // the low face of the current line
+  const bool ly0 = !(wy && p.y0 == 0);
+  if (ly0) {
+    double v[VEC];
+    ldv<VEC>(pv + p.y0 * sv, v);
+    split_states<VEC>(v, vh, vl);
+  }
+  for (int32_t y = p.y0; y < p.y1; ++y, pu += su, pw += sv, pd += sv) {
+    const bool ly = !(wy && y == 0), hy = !(wy && y == ny - 1);
+    const int32_t yh = g.bc[1] == ENS_BC_PERIODIC && y + 1 == ny ? 0 : y + 1;
+    const double ax = g.area[0][y + (int64_t)ny * p.z], az = g.area[2][p.x + (int64_t)nx * y];
+    double u0[VEC], u1[VEC], v1[VEC], w0[VEC], w1[VEC];
+    if (hx) ldv<VEC>(pu + du, u1);
+    if (lx) ldv<VEC>(pu, u0);
+    if (hy) ldv<VEC>(pv + yh * sv, v1);
+    if (hz) ldv<VEC>(pw + dw, w1);
+    if (lz) ldv<VEC>(pw, w0);
+    uint64_t sh[NP], sl[NP];
+#pragma unroll
+    for (int q = 0; q < NP; ++q) sh[q] = sl[q] = 0ull;
+    auto add = [&](uint64_t ah, uint64_t al, const float (&h)[VEC], const float (&l)[VEC]) {
+#pragma unroll
+      for (int q = 0; q < NP; ++q) box_acc2(ah, al, f2_pack(h[2 * q], h[2 * q + 1]), f2_pack(l[2 * q], l[2 * q + 1]), zero, sh[q], sl[q]);
+    };
+    float h[VEC], l[VEC], a0, a1;
+    box_split(ax, a0, a1);
+    uint64_t AH = f2_pack(a0, a0), AL = f2_pack(a1, a1);
+    if (hx) {
+      split_states<VEC>(u1, h, l);
+      add(AH, AL, h, l);
+    }
+    if (lx) {
+      split_states<VEC>(u0, h, l);
+      add(AH ^ kSign2, AL ^ kSign2, h, l);
+    }
+    float nh[VEC], nl[VEC];
+    if (hy) {
+      split_states<VEC>(v1, nh, nl);
+      add(YH, YL, nh, nl);
+    }
+    if (ly) add(YH ^ kSign2, YL ^ kSign2, vh, vl);
+    box_split(az, a0, a1);
+    AH = f2_pack(a0, a0), AL = f2_pack(a1, a1);
+    if (hz) {
+      split_states<VEC>(w1, h, l);
+      add(AH, AL, h, l);
+    }
+    if (lz) {
+      split_states<VEC>(w0, h, l);
+      add(AH ^ kSign2, AL ^ kSign2, h, l);
+    }
+    float s[VEC], t[VEC];
+    double out[VEC];
+    uint32_t worst = 0u, least = 0xFFFFFFFFu;
+#pragma unroll
+    for (int q = 0; q < NP; ++q) {
+      f2_unpack(sh[q], s[2 * q], s[2 * q + 1]);
+      f2_unpack(sl[q], t[2 * q], t[2 * q + 1]);
+    }
+#pragma unroll
+    for (int q = 0; q < VEC; ++q) {
+      float sum = s[q];
+      out[q] = box_add(sum, t[q]);
+      worst = max(worst, max(box_sum_range(s[q]), box_sum_range(sum)));
+      least = min(least, box_mantissa(sum));
+    }
+    if (worst >= kBoxSumWindow || least == 0u) {
+#pragma unroll
+      for (int q = 0; q < VEC; ++q) {
+        if (split_finite(s[q]) && split_finite(t[q])) {
+          out[q] = split_to_double(s[q], t[q]);
+        } else {  // a face value outside the split range: native products for this state
+          double acc = 0.0;
+          if (hx) acc = fma(ax, __ldg(pu + du + q), acc);
+          if (lx) acc = fma(-ax, __ldg(pu + q), acc);
+          if (hy) acc = fma(ay, __ldg(pv + yh * sv + q), acc);
+          if (ly) acc = fma(-ay, __ldg(pv + y * sv + q), acc);
+          if (hz) acc = fma(az, __ldg(pw + dw + q), acc);
+          if (lz) acc = fma(-az, __ldg(pw + q), acc);
+          out[q] = acc;
+        }
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < VEC; ++q) {
+      out[q] *= scale;
+      vh[q] = nh[q];
+      vl[q] = nl[q];
+    }
+    stv<VEC>(pd, out);
+  }
+}
+
+// The correction, one line per block: a difference and an update per face and state, six FP64 operations on a pipe of
+// two per clock and SM, and 0.75 more for the coefficients with four states per thread (186 us for 128^3 cells, m = 8;
+// measured 209, 220 with the index divisions of k_grad_correct). Slower: coefficients shared by the block (226: a
+// barrier before the first load), marching along y as the divergence does (345: the next line's loads wait for
+// this line's stores).
+template <int VEC>
+__global__ void __launch_bounds__(256)
+    k_grad_correct_lines(GridView g, int32_t m, double tau, const double *__restrict__ P, double *U, double *V, double *W) {
+  const March p = march_place<VEC, 1>(g, m);
+  const int32_t nx = g.N[0], ny = g.N[1], nz = g.N[2], y = p.y0;
+  if (!p.on) return;
+  const bool lx = !(g.bc[0] == ENS_BC_WALL && p.x == 0), ly = !(g.bc[1] == ENS_BC_WALL && y == 0), lz = !(g.bc[2] == ENS_BC_WALL && p.z == 0);
+  const bool zx = g.bc[0] == ENS_BC_DIRICHLET && p.x == 0, zy = g.bc[1] == ENS_BC_DIRICHLET && y == 0,
+             zz = g.bc[2] == ENS_BC_DIRICHLET && p.z == 0;  // p = 0 beyond
+  const double cx = tau * g.inv_dist[0][p.x], cy = tau * g.inv_dist[1][y], cz = tau * g.inv_dist[2][p.z];
+  const int64_t sp = (int64_t)nx * m, line = (int64_t)ny * p.z + y;
+  const double *pp = P + (p.x + nx * line) * m + p.c;
+  double *pu = U + (p.x + g.F[0] * line) * m + p.c;
+  double *pv = V + (p.x + nx * (y + (int64_t)g.F[1] * p.z)) * m + p.c;
+  double *pw = W + (p.x + nx * line) * m + p.c;
+  double pc[VEC], px[VEC], py[VEC], pz[VEC], u[VEC], v[VEC], w[VEC];
+  ldv<VEC>(pp, pc);
+  auto low = [&](bool has, int64_t off, double (&q)[VEC]) {
+    if (has)
+      ldv<VEC>(pp + off, q);
+    else
+#pragma unroll
+      for (int k = 0; k < VEC; ++k) q[k] = 0.0;
+  };
+  low(lx && !zx, (int64_t)(p.x == 0 ? nx - 1 : -1) * m, px);
+  low(ly && !zy, (y == 0 ? ny - 1 : -1) * sp, py);
+  low(lz && !zz, (p.z == 0 ? nz - 1 : -1) * sp * ny, pz);
+  if (lx) ldv_rw<VEC>(pu, u);
+  if (ly) ldv_rw<VEC>(pv, v);
+  if (lz) ldv_rw<VEC>(pw, w);
+  auto update = [&](double *f, double coef, const double (&q)[VEC], double (&a)[VEC]) {
+#pragma unroll
+    for (int k = 0; k < VEC; ++k) a[k] = fma(-coef, pc[k] - q[k], a[k]);
+    stv<VEC>(f, a);
+  };
+  if (lx) update(pu, cx, px, u);
+  if (ly) update(pv, cy, py, v);
+  if (lz) update(pw, cz, pz, w);
+  auto edge = [&](double *f, double coef) {  // a Dirichlet boundary face on the high side
+    double a[VEC];
+    ldv_rw<VEC>(f, a);
+#pragma unroll
+    for (int k = 0; k < VEC; ++k) a[k] = fma(-coef, 0.0 - pc[k], a[k]);
+    stv<VEC>(f, a);
+  };
+  if (g.bc[0] == ENS_BC_DIRICHLET && p.x == nx - 1) edge(pu + m, tau * g.inv_dist[0][nx]);
+  if (g.bc[1] == ENS_BC_DIRICHLET && y == ny - 1) edge(pv + sp, tau * g.inv_dist[1][ny]);
+  if (g.bc[2] == ENS_BC_DIRICHLET && p.z == nz - 1) edge(pw + sp * ny, tau * g.inv_dist[2][nz]);
+}
+
+// Threads and blocks of a marching launch over lines of MARCH (0 blocks: more than a grid dimension holds).
+struct MarchLaunch {
+  int threads;
+  int64_t blocks;
+};
+template <int VEC, int MARCH>
+MarchLaunch march_launch(const ens_grid *G, int m) {
+  const int64_t width = (int64_t)G->N[0] * (m / VEC), xb = (width + 255) / 256;
+  const int threads = (int)(((width + xb - 1) / xb + 31) / 32 * 32);
+  const int64_t blocks = (width + threads - 1) / threads * ((G->N[1] + MARCH - 1) / MARCH) * G->N[2];
+  return MarchLaunch{threads, width <= INT32_MAX && blocks <= INT32_MAX ? blocks : 0};
+}
+// Both return false (nothing launched) where the grid is too large for one launch.
+template <int VEC>
+bool divergence_march(const ens_grid *G, const GridView &g, int m, double scale, const double *U, const double *V, const double *W, double *D,
+                      cudaStream_t s) {
+  const MarchLaunch l = march_launch<VEC, kDivMarch>(G, m);
+  if (l.blocks > 0) k_divergence_march<VEC, kDivMarch><<<(unsigned)l.blocks, l.threads, 0, s>>>(g, m, scale, U, V, W, D);
+  return l.blocks > 0;
+}
+template <int VEC>
+bool grad_correct_lines(const ens_grid *G, const GridView &g, int m, double tau, const double *P, double *U, double *V, double *W,
+                        cudaStream_t s) {
+  const MarchLaunch l = march_launch<VEC, 1>(G, m);
+  if (l.blocks > 0) k_grad_correct_lines<VEC><<<(unsigned)l.blocks, l.threads, 0, s>>>(g, m, tau, P, U, V, W);
+  return l.blocks > 0;
+}
+
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 int grid_blocks(const ens_grid *G, int64_t work) {
@@ -536,6 +772,11 @@ extern "C" ens_status ens_divergence(const ens_grid *G, int32_t m, double scale,
   const GridView g = view_of(G);
   cudaStream_t s = (cudaStream_t)stream;
   const int64_t work = (int64_t)G->n * (m / vec);
+  if (vec > 1 && G->all_fluid && G->split_area &&
+      (vec == 4 ? divergence_march<4>(G, g, m, scale, U, V, W, D, s) : divergence_march<2>(G, g, m, scale, U, V, W, D, s))) {
+    ENS_CUDA_TRY(cudaGetLastError());
+    return ENS_OK;
+  }
   // split-float products on the FP32 pipe for two or four states per thread (native for one)
   if (vec == 4 && G->split_area)
     k_divergence_split<4><<<grid_blocks(G, work), kThreads, 0, s>>>(g, m, scale, U, V, W, D);
@@ -572,6 +813,12 @@ extern "C" ens_status ens_grad_correct(const ens_grid *G, int32_t m, double tau,
   const GridView g = view_of(G);
   cudaStream_t s = (cudaStream_t)stream;
   const int64_t work = (int64_t)G->n * (m / vec);
+  if (G->all_fluid && (vec == 4   ? grad_correct_lines<4>(G, g, m, tau, P, U, V, W, s)
+                       : vec == 2 ? grad_correct_lines<2>(G, g, m, tau, P, U, V, W, s)
+                                  : grad_correct_lines<1>(G, g, m, tau, P, U, V, W, s))) {
+    ENS_CUDA_TRY(cudaGetLastError());
+    return ENS_OK;
+  }
   if (vec == 4)
     k_grad_correct<4><<<grid_blocks(G, work), kThreads, 0, s>>>(g, m, tau, P, U, V, W);
   else if (vec == 2)
