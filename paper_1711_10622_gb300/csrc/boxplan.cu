@@ -13,7 +13,6 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
-#include <cstring>
 #include <new>
 #include <thread>
 #include <unordered_map>
@@ -45,10 +44,10 @@ void common_steps(int64_t n, const int32_t *rp, const int32_t *ci, int64_t &shor
   long_step = b == 0 ? 0 : std::max(a, b);
 }
 
-struct Part {  // boxes of one range of rows
-  std::vector<int32_t> rows, cols;        // concatenated
-  std::vector<uint16_t> loc;              // kBoxRows * K per box, slot-major
-  std::vector<int32_t> nrows, ncols;
+struct Part {  // boxes of one range of rows, in the layout of BoxPlan
+  std::vector<int32_t> rows, cols;
+  std::vector<uint16_t> loc;
+  std::vector<int2> cnt;
   int64_t ucols = 0;
 };
 
@@ -92,7 +91,13 @@ void build_part(int64_t r0, int64_t r1, const int32_t *rp, const int32_t *ci, in
     }
     return step(base, d);
   };
-  std::vector<int32_t> rows;
+  std::vector<int32_t> rows, cols;
+  rows.reserve(kBoxRows);
+  cols.reserve(kBoxCols);
+  const size_t guess = (size_t)(n / 224 + 16);
+  P.rows.reserve(guess * kBoxRows);
+  P.cols.reserve(guess * kBoxCols);
+  P.loc.reserve(guess * kBoxRows * K);
   int64_t next = r0;
   while (next < r1) {
     if (used[next - r0]) {
@@ -100,8 +105,8 @@ void build_part(int64_t r0, int64_t r1, const int32_t *rp, const int32_t *ci, in
       continue;
     }
     rows.clear();
+    cols.clear();
     cs.clear();
-    const size_t col0 = P.cols.size();
     // a row joins when the box has room for it and for its new columns
     auto take = [&](int64_t i) -> bool {
       if ((int)rows.size() == kBoxRows) return false;
@@ -114,7 +119,7 @@ void build_part(int64_t r0, int64_t r1, const int32_t *rp, const int32_t *ci, in
           cs.stamp[at] = cs.now;
           cs.key[at] = ci[j];
           cs.pos[at] = cs.count++;
-          P.cols.push_back(ci[j]);
+          cols.push_back(ci[j]);
         }
       rows.push_back((int32_t)i);
       used[i - r0] = 1;
@@ -142,13 +147,13 @@ void build_part(int64_t r0, int64_t r1, const int32_t *rp, const int32_t *ci, in
     }
     // Columns in ascending order: neighbouring rows of the box then read neighbouring X rows, staged from
     // whole lines of memory and read from shared memory without bank conflicts.
-    std::sort(P.cols.begin() + col0, P.cols.end());
+    std::sort(cols.begin(), cols.end());
     cs.clear();
-    for (size_t q = col0; q < P.cols.size(); ++q) {
+    for (int32_t c : cols) {
       uint32_t at;
-      cs.find(P.cols[q], at);
+      cs.find(c, at);
       cs.stamp[at] = cs.now;
-      cs.key[at] = P.cols[q];
+      cs.key[at] = c;
       cs.pos[at] = cs.count++;
     }
     const size_t l0 = P.loc.size();
@@ -158,10 +163,12 @@ void build_part(int64_t r0, int64_t r1, const int32_t *rp, const int32_t *ci, in
       uint32_t at;
       for (int32_t j = rp[i]; j < rp[i + 1]; ++j) P.loc[l0 + (size_t)(j - rp[i]) * kBoxRows + r] = (uint16_t)cs.find(ci[j], at);
     }
+    P.cnt.push_back(make_int2((int32_t)rows.size(), (int32_t)cols.size()));
+    P.ucols += (int64_t)cols.size();
+    rows.resize(kBoxRows, -1);
+    cols.resize(kBoxCols, 0);
     P.rows.insert(P.rows.end(), rows.begin(), rows.end());
-    P.nrows.push_back((int32_t)rows.size());
-    P.ncols.push_back((int32_t)(P.cols.size() - col0));
-    P.ucols += cs.count;
+    P.cols.insert(P.cols.end(), cols.begin(), cols.end());
   }
 }
 
@@ -186,13 +193,6 @@ __global__ void k_box_values(int32_t boxes, int32_t K, const int32_t *__restrict
     bvs[e] = v;
     bv32[e] = f;
   }
-}
-
-template <typename T>
-cudaError_t upload(T **dst, const std::vector<T> &src, cudaStream_t s) {
-  cudaError_t e = cudaMalloc(reinterpret_cast<void **>(dst), std::max<size_t>(src.size(), 1) * sizeof(T));
-  if (e == cudaSuccess && !src.empty()) e = cudaMemcpyAsync(*dst, src.data(), src.size() * sizeof(T), cudaMemcpyHostToDevice, s);
-  return e;
 }
 
 }  // namespace
@@ -243,38 +243,28 @@ cudaError_t build_box(ens_matrix *A, const int32_t *rp, const int32_t *ci, cudaS
   }
   if (!memory) return cudaSuccess;  // no plan
   int64_t boxes = 0, ucols = 0;
-  for (auto &p : part) boxes += (int64_t)p.nrows.size(), ucols += p.ucols;
+  for (auto &p : part) boxes += (int64_t)p.cnt.size(), ucols += p.ucols;
   if (ucols > (int64_t)(0.45 * (double)nnz) || boxes * kBoxRows > n + n / 4 * 3 + 64 * kBoxRows) return cudaSuccess;
-  std::vector<int32_t> row, col;
-  std::vector<int2> cnt;
-  std::vector<uint16_t> loc;
-  try {
-    row.assign((size_t)boxes * kBoxRows, -1);
-    col.assign((size_t)boxes * kBoxCols, 0);
-    loc.reserve((size_t)boxes * kBoxRows * K);
-    cnt.reserve(boxes);
-    for (auto &p : part) {
-      size_t r = 0, c = 0;
-      for (size_t b = 0; b < p.nrows.size(); ++b) {
-        std::memcpy(row.data() + cnt.size() * kBoxRows, p.rows.data() + r, p.nrows[b] * sizeof(int32_t));
-        std::memcpy(col.data() + cnt.size() * kBoxCols, p.cols.data() + c, p.ncols[b] * sizeof(int32_t));
-        r += p.nrows[b];
-        c += p.ncols[b];
-        cnt.push_back(make_int2(p.nrows[b], p.ncols[b]));
-      }
-      loc.insert(loc.end(), p.loc.begin(), p.loc.end());
-    }
-  } catch (const std::bad_alloc &) {
-    return cudaSuccess;
-  }
   BoxPlan &B = A->box;
   B.boxes = (int32_t)boxes;
   B.K = K;
   const size_t slots = (size_t)boxes * K * kBoxRows;
-  cudaError_t e = upload(&B.row, row, s);
-  if (e == cudaSuccess) e = upload(&B.cnt, cnt, s);
-  if (e == cudaSuccess) e = upload(&B.col, col, s);
-  if (e == cudaSuccess) e = upload(&B.loc, loc, s);
+  cudaError_t e = cudaMalloc((void **)&B.row, (size_t)boxes * kBoxRows * sizeof(int32_t));
+  if (e == cudaSuccess) e = cudaMalloc((void **)&B.col, (size_t)boxes * kBoxCols * sizeof(int32_t));
+  if (e == cudaSuccess) e = cudaMalloc((void **)&B.cnt, (size_t)boxes * sizeof(int2));
+  if (e == cudaSuccess) e = cudaMalloc((void **)&B.loc, slots * sizeof(uint16_t));
+  size_t at = 0;  // boxes of the parts before
+  for (auto &p : part) {
+    auto put = [&](auto *dst, const auto &src, size_t per_box) {
+      if (e == cudaSuccess && !src.empty())
+        e = cudaMemcpyAsync(dst + at * per_box, src.data(), src.size() * sizeof(src[0]), cudaMemcpyHostToDevice, s);
+    };
+    put(B.row, p.rows, kBoxRows);
+    put(B.col, p.cols, kBoxCols);
+    put(B.cnt, p.cnt, 1);
+    put(B.loc, p.loc, (size_t)kBoxRows * K);
+    at += p.cnt.size();
+  }
   if (e == cudaSuccess) e = cudaMalloc((void **)&B.vs, slots * sizeof(float2));
   if (e == cudaSuccess) e = cudaMalloc((void **)&B.v32, slots * sizeof(float));
   if (e == cudaSuccess) {
