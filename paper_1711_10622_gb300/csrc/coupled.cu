@@ -715,7 +715,7 @@ ens_status solve_coupled(const ens_matrix *M, int32_t m, const double *B, double
   ens_status gst = ENS_OK;
   int it = 0;
   {
-    Scratch sc(s, o);
+    Scratch sc(s, M, o);
     // per-column start checks on the device: ||b||^2, sum(b), non-finite entries of b and x0
     const int rgrid = (int)std::max<int64_t>(1, std::min<int64_t>((n * m + 255) / 256, (int64_t)M->num_sms * 4));
     double *rpart = nullptr, *rout = nullptr;

@@ -42,6 +42,24 @@ ens_status cuda_fail(cudaError_t e, const char *what) {
 
 void clear_error() { g_last_error.clear(); }
 
+cudaMemPool_t scratch_pool(const ens_matrix *A) {
+  std::call_once(A->pool_once, [A] {
+    cudaMemPoolProps p = {};
+    p.allocType = cudaMemAllocationTypePinned;
+    p.location.type = cudaMemLocationTypeDevice;
+    p.location.id = A->device;
+    cudaMemPool_t pool = nullptr;
+    uint64_t keep = kPoolKeep;
+    if (cudaMemPoolCreate(&pool, &p) != cudaSuccess) {
+      (void)cudaGetLastError();
+      return;
+    }
+    if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) (void)cudaGetLastError();
+    A->pool = pool;
+  });
+  return A->pool;
+}
+
 namespace {
 
 // Per-row set-up: inverse diagonal (Jacobi scaling) and the float32 / split copies of val.
@@ -95,6 +113,7 @@ void free_matrix(ens_matrix *A) {
     if (ev) cudaEventDestroy(ev);
   if (A->pipe_h2d) cudaStreamDestroy(A->pipe_h2d);
   if (A->pipe_d2h) cudaStreamDestroy(A->pipe_d2h);
+  if (A->pool) cudaMemPoolDestroy(A->pool);
   delete A;
 }
 

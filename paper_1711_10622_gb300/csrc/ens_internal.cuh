@@ -5,6 +5,7 @@
 
 #include <cstdint>
 #include <cstdio>
+#include <mutex>
 #include <vector>
 
 #include "ensemble_solve.h"
@@ -60,6 +61,10 @@ struct ens_matrix {
   int64_t pipe_block_rows = 1;
   cudaStream_t pipe_h2d = nullptr, pipe_d2h = nullptr;
   std::vector<cudaEvent_t> pipe_ev;
+  // Scratch of the solves on this matrix comes from a pool of its own that keeps up to kPoolKeep bytes between
+  // calls (scratch_pool); made by the first solve, given back with the matrix.
+  mutable std::once_flag pool_once;
+  mutable cudaMemPool_t pool = nullptr;
   // aggregation multigrid hierarchy (ens_amg_setup), owned
   ens_amg *amg = nullptr;
 };
@@ -81,6 +86,11 @@ struct ens_amg {
 };
 
 namespace ens {
+
+// The memory pool of A's scratch (nullptr: the device's default pool). The default pool gives everything back at
+// every synchronisation, so each solve mapped its blocks anew. Any thread, any stream.
+constexpr uint64_t kPoolKeep = 128ull << 20;
+cudaMemPool_t scratch_pool(const ens_matrix *A);
 
 // Release a hierarchy (coarse matrices and maps; not the fine matrix).
 void free_amg(ens_amg *H);

@@ -129,7 +129,7 @@ ens_status ens_solve_batch(int32_t nsys, const ens_batch_item *items, const ens_
   }
   cudaError_t e = cudaSuccess;
   {
-    solver::Scratch sc(s, o);
+    solver::Scratch sc(s, items[0].A, o);
     for (auto &p : sys)
       if (e == cudaSuccess) e = p->setup(sc);
     // one graph: a branch per system forked from and joined into a private capture stream
@@ -225,7 +225,7 @@ ens_status amg_apply_impl(const ens_matrix *A, int32_t m, const void *R, void *Z
   const int64_t n = A->n;
   cudaError_t e = cudaSuccess;
   {
-    solver::Scratch sc(s);
+    solver::Scratch sc(s, A);
     const T *r = (const T *)R;
     T *z = (T *)Z;
     T *rp = nullptr, *zp = nullptr;

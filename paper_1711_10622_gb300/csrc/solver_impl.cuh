@@ -707,12 +707,14 @@ cudaError_t with_vl(int vec, int lanes, F &&f) {
 // ens_last_workspace_bytes(); a workspace that is too small ends the call with ENS_ERR_BUDGET.
 struct Scratch {
   cudaStream_t s;
+  cudaMemPool_t pool = nullptr;
   std::vector<void *> ptrs;
   char *arena = nullptr;
   size_t cap = 0, used = 0;
   bool overflow = false;
-  explicit Scratch(cudaStream_t st) : s(st) {}
-  Scratch(cudaStream_t st, const ens_solve_opts &o) : s(st), arena((char *)o.workspace), cap(o.workspace_bytes) {}
+  Scratch(cudaStream_t st, const ens_matrix *A) : s(st), pool(scratch_pool(A)) {}
+  Scratch(cudaStream_t st, const ens_matrix *A, const ens_solve_opts &o)
+      : s(st), pool(o.workspace ? nullptr : scratch_pool(A)), arena((char *)o.workspace), cap(o.workspace_bytes) {}
   ~Scratch() {
     for (void *p : ptrs) cudaFreeAsync(p, s);
     record_workspace(used, overflow);
@@ -731,7 +733,7 @@ struct Scratch {
       return cudaSuccess;
     }
     void *q = nullptr;
-    cudaError_t e = cudaMallocAsync(&q, bytes, s);
+    cudaError_t e = pool ? cudaMallocFromPoolAsync(&q, bytes, pool, s) : cudaMallocAsync(&q, bytes, s);
     if (e != cudaSuccess) return e;
     ptrs.push_back(q);
     used += bytes;
@@ -1545,7 +1547,7 @@ ens_status solve_f64(const ens_matrix *M, int32_t m, const double *B, double *X,
   const int mp = m == 1 ? 1 : (m + 1) / 2 * 2;
   const int64_t n = M->n;
   const int singular = (M->flags & ENS_MATRIX_SINGULAR) ? 1 : 0;
-  Scratch sc(s, o);
+  Scratch sc(s, M, o);
   double *b = nullptr, *x = nullptr;
   cudaError_t e = sc.get(&b, (size_t)n * mp);
   if (e == cudaSuccess) e = sc.get(&x, (size_t)n * mp);
