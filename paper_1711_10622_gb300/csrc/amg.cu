@@ -11,6 +11,7 @@
 #include <new>
 #include <vector>
 
+#include "amg_small.cuh"
 #include "ens_internal.cuh"
 
 namespace ens {
@@ -125,6 +126,34 @@ cudaError_t upload(T **dst, const std::vector<T> &src, cudaStream_t s) {
   return cudaMemcpyAsync(*dst, src.data(), src.size() * sizeof(T), cudaMemcpyHostToDevice, s);
 }
 
+// The coarsest level's updates as a dense matrix, where the level is small and has its diagonal.
+cudaError_t dense_coarsest(ens_amg *H, cudaStream_t s) {
+  const ens_matrix *A = H->lev.back().A;
+  const ens_amg_opts &o = H->opts;
+  if (A->n > solver::kDenseRows || o.coarse_steps > solver::kMaxCoarseSteps || !A->full_diag) return cudaSuccess;
+  const double theta = 0.5 * (o.cheb_hi + o.cheb_lo), delta = 0.5 * (o.cheb_hi - o.cheb_lo), sigma = theta / delta;
+  std::vector<double> k(2 * solver::kMaxCoarseSteps, 0.0);
+  double rho_prev = 1.0 / sigma;
+  for (int i = 1; i < solver::kMaxCoarseSteps; ++i) {
+    const double rho = 1.0 / (2.0 * sigma - rho_prev);
+    k[i] = rho * rho_prev;
+    k[solver::kMaxCoarseSteps + i] = 2.0 * rho / delta;
+    rho_prev = rho;
+  }
+  double *dk = nullptr;
+  cudaError_t e = upload(&dk, k, s);
+  const size_t nn = (size_t)A->n * A->n;
+  if (e == cudaSuccess) e = cudaMalloc((void **)&H->dense, nn * sizeof(double));
+  if (e == cudaSuccess) e = cudaMalloc((void **)&H->dense32, nn * sizeof(float));
+  if (e == cudaSuccess) {
+    const MatView v{(int32_t)A->n, A->row, A->col, A->val, A->val32, A->valsplit, A->dinv, A->dinv32};
+    e = solver::coarse_matrix(v, o.coarse_steps, 1.0 / theta, dk, dk + solver::kMaxCoarseSteps, H->dense, H->dense32, s);
+  }
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // dk and k are used until here
+  cudaFree(dk);
+  return e;
+}
+
 ens_status check_opts(const ens_amg_opts &o) {
   if (!(o.theta >= 0.0) || !(o.theta < 1.0)) return fail(ENS_ERR_INVALID, "amg_setup: theta must lie in [0, 1)");
   if (o.max_levels < 2 || o.max_levels > 16) return fail(ENS_ERR_INVALID, "amg_setup: max_levels must lie in [2, 16]");
@@ -146,6 +175,8 @@ void free_amg(ens_amg *H) {
     cudaFree(l.agg_ptr);
     cudaFree(l.members);
   }
+  cudaFree(H->dense);
+  cudaFree(H->dense32);
   delete H;
 }
 
@@ -238,6 +269,7 @@ static ens_status amg_setup_impl(ens_matrix *A, const ens_amg_opts *opts, void *
     H->lev.push_back(ens_amg_lev{Mc, true});
     L = std::move(C);
   }
+  if (e == cudaSuccess) e = dense_coarsest(H, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) {
     free_amg(H);

@@ -6,8 +6,9 @@
 //     for), whose sums are added by shuffles; each thread has four gathers in flight.
 //   * k_amg_tail: every level below a few thousand rows, down and up again, in one launch of one
 //     thread-block cluster. The stages are separated by the cluster's hardware barrier instead of kernel
-//     boundaries; blocks exchange vectors through L2. The coarsest level's updates run in one block on
-//     vectors held in shared memory.
+//     boundaries; blocks exchange vectors through L2. The coarsest level's updates, one fixed linear operator,
+//     are applied as its dense matrix, formed at set-up (levels of at most kDenseRows rows; otherwise update by
+//     update in one block, on vectors in shared memory where they fit: 43 of a launch's 80-135 us).
 // The bound is latency throughout (a stage is one or two dependent gathers); the sums are native FMA in the
 // type of the cycle, rows summed in a fixed order of S interleaved parts.
 #include <cuda_runtime.h>
@@ -42,7 +43,9 @@ __device__ __forceinline__ void load_cg(const T *p, T (&v)[VEC]) {
 
 // This thread's part of row i's product with X, columns [c, c + VEC): nonzeros j0 + sub, j0 + sub + S, ...,
 // four gathers at a time, then the sum over the S threads of the row (lanes of one warp, `lanes` apart). Every
-// thread of a warp calls this the same number of times (valid = false: no row).
+// thread of a warp calls this the same number of times (valid = false: no row). (Dealing the rest of rows longer
+// than 16 to the whole warp was tried for the few rows of a hundred nonzeros among rows of nine: the mixed AMG solve
+// on 96^3 took 62.6 ms against 54.6.)
 template <typename T, int VEC, bool SHARED>
 __device__ __forceinline__ void row_part(bool valid, const int32_t *__restrict__ rp, const int32_t *__restrict__ ci,
                                          const T *__restrict__ va, int32_t i, const T *X, int32_t m, int32_t c, int32_t sub,
@@ -245,6 +248,74 @@ __device__ __forceinline__ void coarse_updates(const TailArgs<T> &a, const TailL
   }
 }
 
+// The coarsest level's z = M r, M the dense matrix of its updates: one warp per row and VEC columns, its lanes along
+// the row; r from shared memory. Every block of the cluster takes a share of the rows.
+template <typename T, int VEC>
+__device__ __forceinline__ void coarse_dense(const TailArgs<T> &a, const TailLevel<T> &L, T *r) {
+  const int32_t n = L.n, m = a.m, nv = m / VEC, lane = threadIdx.x & 31;
+  for (int32_t t = threadIdx.x; t < n * nv; t += kTailThreads) {
+    T v[VEC];
+    load_cg<T, VEC>(L.r + (int64_t)t * VEC, v);
+    store_vec<T, VEC>(r + (int64_t)t * VEC, v);
+  }
+  __syncthreads();
+  for (int32_t t = blockIdx.x * (kTailThreads / 32) + threadIdx.x / 32; t < n * nv; t += kTailBlocks * (kTailThreads / 32)) {
+    const int32_t i = t / nv, c = (t - i * nv) * VEC;
+    const T *row = a.dense + (int64_t)i * n;
+    T w[VEC];
+#pragma unroll
+    for (int q = 0; q < VEC; ++q) w[q] = T(0);
+    for (int32_t j = lane; j < n; j += 128) {
+      T f[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) f[u] = j + 32 * u < n ? __ldg(row + j + 32 * u) : T(0);
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (j + 32 * u < n) {
+          T v[VEC];
+          load_vec_rw<T, VEC>(r + (int64_t)(j + 32 * u) * m + c, v);
+#pragma unroll
+          for (int q = 0; q < VEC; ++q) w[q] = fma(f[u], v[q], w[q]);
+        }
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1)
+#pragma unroll
+      for (int q = 0; q < VEC; ++q) w[q] += __shfl_xor_sync(0xffffffffu, w[q], off);
+    if (lane == 0) store_vec<T, VEC>(L.z + (int64_t)i * m + c, w);
+  }
+}
+
+// Column blockIdx.x of the dense matrix of z = S_steps(r), in float64: the updates applied to a unit vector.
+__global__ void __launch_bounds__(256) k_coarse_matrix(MatView A, int32_t steps, double inv_theta, const double *__restrict__ k1,
+                                                       const double *__restrict__ k2, double *__restrict__ M, float *__restrict__ M32) {
+  extern __shared__ __align__(16) unsigned char raw[];
+  const int32_t n = A.n, col = blockIdx.x;
+  double *d0 = reinterpret_cast<double *>(raw), *d1 = d0 + n, *res = d1 + n, *z = res + n;
+  for (int32_t i = threadIdx.x; i < n; i += 256) {
+    res[i] = i == col ? 1.0 : 0.0;
+    d0[i] = z[i] = res[i] * A.dinv[i] * inv_theta;
+  }
+  __syncthreads();
+  for (int k = 1; k < steps; ++k) {
+    for (int32_t i = threadIdx.x; i < n; i += 256) {
+      double w = 0.0;
+      for (int32_t j = A.rp[i]; j < A.rp[i + 1]; ++j) w = fma(A.val[j], d0[A.ci[j]], w);
+      res[i] -= w;
+      d1[i] = k1[k] * d0[i] + k2[k] * (A.dinv[i] * res[i]);
+      z[i] += d1[i];
+    }
+    __syncthreads();
+    double *t = d0;
+    d0 = d1;
+    d1 = t;
+  }
+  for (int32_t i = threadIdx.x; i < n; i += 256) {
+    M[(int64_t)i * n + col] = z[i];
+    M32[(int64_t)i * n + col] = (float)z[i];
+  }
+}
+
 template <typename T, int VEC>
 __global__ void __launch_bounds__(kTailThreads) k_amg_tail(const __grid_constant__ TailArgs<T> a, int32_t S, int in_smem) {
   extern __shared__ __align__(16) unsigned char raw[];
@@ -261,7 +332,9 @@ __global__ void __launch_bounds__(kTailThreads) k_amg_tail(const __grid_constant
     restrict_rows<T, VEC>(p, L.ptr, L.mem, L.nc, m, a.lanes, S, L.res, C.r);
     cluster_barrier();
   }
-  if (rank == 0) {
+  if (a.dense) {
+    coarse_dense<T, VEC>(a, a.lev[last], reinterpret_cast<T *>(raw));
+  } else if (rank == 0) {
     const TailLevel<T> &L = a.lev[last];
     if (in_smem) {
       const int64_t blk = (int64_t)L.n * m;
@@ -301,13 +374,14 @@ cudaError_t run_tail(const TailArgs<T> &a, cudaStream_t st) {
   const TailLevel<T> &C = a.lev[a.nl - 1];
   const size_t need = 4 * (size_t)C.n * a.m * sizeof(T);
   const bool in_smem = need <= kTailSmem;
+  const bool dense = a.dense != nullptr && need / 4 <= kTailSmem;
   auto k = k_amg_tail<T, VEC>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTailSmem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(kTailBlocks);
   cfg.blockDim = dim3(kTailThreads);
-  cfg.dynamicSmemBytes = in_smem ? need : 0;
+  cfg.dynamicSmemBytes = dense ? need / 4 : in_smem ? need : 0;
   cfg.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
@@ -318,7 +392,10 @@ cudaError_t run_tail(const TailArgs<T> &a, cudaStream_t st) {
   // Four threads per row, on the coarsest level too (channel 96^3, m = 8, mixed solve: 59.5 ms; 8 threads
   // there 63.0, 16: 69.6; 8 or 16 on the other levels as well: 62.0 and 67.8).
   const int32_t S = std::min(4, 32 / a.lanes);
-  return cudaLaunchKernelEx(&cfg, k, a, S, in_smem ? 1 : 0);
+  if (dense || !a.dense) return cudaLaunchKernelEx(&cfg, k, a, S, in_smem ? 1 : 0);
+  TailArgs<T> b = a;  // r does not fit: the updates themselves
+  b.dense = nullptr;
+  return cudaLaunchKernelEx(&cfg, k, b, S, in_smem ? 1 : 0);
 }
 
 // Threads per row: the rows of the level spread over the GPU's resident threads (152 SMs x 2048), at most 16
@@ -376,6 +453,12 @@ cudaError_t launch_small_restrict(const int32_t *ptr, const int32_t *mem, int32_
 cudaError_t launch_small_restrict(const int32_t *ptr, const int32_t *mem, int32_t nc, int32_t m, int32_t lanes, int vec, const double *res,
                                   double *rc, cudaStream_t st) {
   return small_restrict<double>(ptr, mem, nc, m, lanes, vec, res, rc, st);
+}
+cudaError_t coarse_matrix(const MatView &A, int32_t steps, double inv_theta, const double *k1, const double *k2, double *M, float *M32,
+                          cudaStream_t st) {
+  const size_t smem = 4 * (size_t)A.n * sizeof(double);
+  k_coarse_matrix<<<A.n, 256, smem, st>>>(A, steps, inv_theta, k1, k2, M, M32);
+  return cudaGetLastError();
 }
 cudaError_t launch_amg_tail(const TailArgs<float> &a, int vec, cudaStream_t st) {
   return with_vec<float>(vec, [&](auto V) { return run_tail<float, decltype(V)::value>(a, st); });

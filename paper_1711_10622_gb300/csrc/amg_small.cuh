@@ -17,6 +17,8 @@ constexpr int kMaxTailLevels = 8;
 // there; the levels above it at most kTailRows (float32) or kTailRowsF64: the cluster's eight SMs have 1/19
 // of the GPU's FP64 rate, so float64 levels leave it earlier.
 constexpr int64_t kTailCoarseRows = 4096;
+// The coarsest level's updates as a dense matrix, up to this many rows (1 MB in float32, formed once at set-up).
+constexpr int64_t kDenseRows = 512;
 constexpr int64_t kTailRows = 4096;
 constexpr int64_t kTailRowsF64 = 1024;
 
@@ -36,11 +38,15 @@ template <typename T>
 struct TailArgs {
   int32_t nl, m, lanes, steps;  // levels, block width, threads across a row's columns, coarsest updates
   T inv_theta, c1, c2;          // two-update smoothing
+  const T *dense;               // matrix of the coarsest level's updates, n x n (nullptr: none)
   T *da, *db, *res;             // coarsest level's blocks (when its vectors do not fit shared memory)
   T k1[kMaxCoarseSteps], k2[kMaxCoarseSteps];
   TailLevel<T> lev[kMaxTailLevels];
 };
 
+// The dense matrix of `steps` updates on A (A.n <= kDenseRows): M and its float32 copy; k1, k2 [steps] on the device.
+cudaError_t coarse_matrix(const MatView &A, int32_t steps, double inv_theta, const double *k1, const double *k2, double *M, float *M32,
+                          cudaStream_t st);
 // z of level 0 of `a` (its first level) from that level's r: the V-cycle from there down, in one cluster.
 cudaError_t launch_amg_tail(const TailArgs<float> &a, int vec, cudaStream_t st);
 cudaError_t launch_amg_tail(const TailArgs<double> &a, int vec, cudaStream_t st);

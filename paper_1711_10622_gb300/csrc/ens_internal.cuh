@@ -82,6 +82,8 @@ struct ens_amg_lev {
 };
 struct ens_amg {
   ens_amg_opts opts;
+  double *dense = nullptr;   // the coarsest level's updates as a dense matrix (amg_small.cuh; NULL: none)
+  float *dense32 = nullptr;
   std::vector<ens_amg_lev> lev;
 };
 

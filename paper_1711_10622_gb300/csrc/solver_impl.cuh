@@ -896,6 +896,8 @@ struct AmgCycle {
   // Levels from tail_at down run in one launch of one cluster (amg_small.cuh); lev.size(): none.
   size_t tail_at = 0;
   TailArgs<T> tail;
+  const double *dense = nullptr;  // the coarsest level's matrix (ens_amg)
+  const float *dense32 = nullptr;
 
   // Values of a level's matrix in the type of the cycle.
   static const T *values(const MatView &A) {
@@ -942,6 +944,10 @@ struct AmgCycle {
     a.c1 = a.k1[1];
     a.c2 = a.k2[1];
     const Level &C = lev[nl - 1];
+    if constexpr (std::is_same<T, float>::value)
+      a.dense = dense32;
+    else
+      a.dense = dense;
     a.da = C.da;
     a.db = C.db;
     a.res = C.cres;
@@ -969,6 +975,8 @@ struct AmgCycle {
   // aligned: r and z of the fine level are 32-byte aligned.
   cudaError_t setup(Scratch &sc, const ens_amg *H, int mp_, int vec_, int lanes_, bool aligned) {
     o = H->opts;
+    dense = H->dense;
+    dense32 = H->dense32;
     mp = mp_;
     vec = vec_;
     lanes = lanes_;
