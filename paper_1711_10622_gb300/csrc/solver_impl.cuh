@@ -224,11 +224,10 @@ __global__ void ENS_TILE_BOUNDS(Arith)
     cs.status[l] = status;
     cs.flags[l] = fl;
     cs.iters[l] = 0;
-  }, [&]() {
-    int32_t any = 0;
-    for (int l = 0; l < m; ++l) any |= cs.state[l] != ST_DONE;
+    return st != ST_DONE;
+  }, [&](bool any) {
     cs.it[0] = 0;
-    cs.it[1] = any;
+    cs.it[1] = any ? 1 : 0;
   });
 }
 
@@ -482,42 +481,44 @@ __global__ void __launch_bounds__(kThreads)
     }
   }
   const int32_t it = cs.it[0] + 1;  // the iteration this launch completes
-  reduce_cols<T, 2, VEC, LANES>(acc, m, partials, counter, [&](int l, const ColTotals<T, 2> &tt) {
+  reduce_cols<T, 2, VEC, LANES>(acc, m, partials, counter, [&](int l, const ColTotals<T, 2> &tt) -> bool {
     const int st = cs.state[l];
     if (st == ST_HALF) {
       cs.state[l] = ST_DONE;
       cs.status[l] = ENS_COL_CONVERGED;
-      return;
+      return false;
     }
-    if (st != ST_ACTIVE) return;
+    if (st != ST_ACTIVE) return st != ST_DONE;
     const T rn2 = tt.v[0][l], rr = tt.v[1][l];
     cs.rn2[l] = rn2;
+    bool on = false;
     if (!isfinite(rn2)) {
-      cs.state[l] = ST_DONE;
       cs.status[l] = ENS_COL_NONFINITE;
     } else if (rn2 <= cs.thr2[l]) {
-      cs.state[l] = ST_DONE;
       cs.status[l] = ENS_COL_CONVERGED;
     } else if (cs.omega[l] == T(0)) {
-      cs.state[l] = ST_DONE;
       cs.status[l] = ENS_COL_BREAKDOWN;
     } else if (it < max_iter) {  // the next iteration begins: rho and its breakdown test
+      // |rho| <= tiny ||rhat|| ||r||; the product of the norms is at most the larger square, so the roots are
+      // only taken when that already fails
+      const T rh2 = cs.rh2[l], a = fabs(rr);
       if (!isfinite(rr)) {
-        cs.state[l] = ST_DONE;
         cs.status[l] = ENS_COL_NONFINITE;
         cs.iters[l] = it + 1;
-      } else if (fabs(rr) <= Tiny<T>::v * sqrt(cs.rh2[l]) * sqrt(rn2)) {
-        cs.state[l] = ST_DONE;
+      } else if (a <= T(2) * Tiny<T>::v * fmax(rh2, rn2) && a <= Tiny<T>::v * sqrt(rh2) * sqrt(rn2)) {
         cs.status[l] = ENS_COL_BREAKDOWN;
         cs.iters[l] = it + 1;
       } else {
         cs.beta[l] = (rr / cs.rho[l]) * (cs.alpha[l] / cs.omega[l]);
         cs.rho[l] = rr;
+        on = true;
       }
+    } else {
+      on = true;  // out of iterations: the column ends as it is
     }
-  }, [&]() {
-    int32_t any = 0;
-    for (int l = 0; l < m; ++l) any |= cs.state[l] != ST_DONE;
+    if (!on) cs.state[l] = ST_DONE;
+    return on;
+  }, [&](bool any) {
     cs.it[0] = it;
     const bool go = any && it < max_iter;
     cs.it[1] = go;
