@@ -18,6 +18,7 @@
 //     whose X values fall outside the split range are recomputed with native DFMA.
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <type_traits>
 
 #include <cstdint>
@@ -90,6 +91,21 @@ __global__ void __launch_bounds__(kThreads)
                                  [&](int64_t i, int32_t c, const T (&y)[VEC]) { store_vec_cs<T, VEC>(Y + i * m + c, y); });
 }
 
+// Resident blocks per SM of a kernel (threads, dynamic shared memory), asked for once per kernel instance and kept in
+// its caller's `known` (0: not yet): the query costs a microsecond or two of every small product's launch. All GPUs
+// this library is built for are the same part.
+int resident(std::atomic<int> &known, const void *kernel, int threads, size_t smem) {
+  int n = known.load(std::memory_order_relaxed);
+  if (n > 0) return n;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, threads, smem) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return 1;
+  }
+  n = n < 1 ? 1 : n;
+  known.store(n, std::memory_order_relaxed);
+  return n;
+}
+
 // Product by row boxes (boxprod.cuh).
 template <typename T, int CW, int ACC, bool FULL, int K0>
 __global__ void __launch_bounds__(BoxShape<T, CW>::kThr, BoxShape<T, CW>::kBlocks)
@@ -105,10 +121,9 @@ cudaError_t run_box(const ens_matrix *A, int m, const void *X, void *Y, cudaStre
   auto k = gspmv_kernel_box<T, CW, ACC, FULL, K0>;
   const size_t smem = S::smem(A->box.K);
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  int per_sm = 0;
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, S::kThr, smem);
   if (e != cudaSuccess) return e;
-  const int64_t full = (int64_t)A->num_sms * (per_sm < 1 ? 1 : per_sm);
+  static std::atomic<int> known[kBoxMaxLen + 1];  // by row length: the shared memory depends on it
+  const int64_t full = (int64_t)A->num_sms * resident(known[A->box.K], (const void *)k, S::kThr, smem);
   k<<<(unsigned)(full < A->box.boxes ? full : (int64_t)A->box.boxes), S::kThr, smem, s>>>(A->box, view_of(A), m, (const T *)X, (T *)Y);
   return cudaGetLastError();
 }
@@ -143,10 +158,7 @@ struct Rows {
 };
 static_assert(kPipeAlignRows % kTileRows == 0, "row chunks must be whole tiles");
 
-int grid_for(const ens_matrix *A, int64_t rows, const void *kernel, int64_t rows_per_block) {
-  int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreads, 0);
-  if (per_sm < 1) per_sm = 1;
+int grid_for(const ens_matrix *A, int64_t rows, int per_sm, int64_t rows_per_block) {
   const int64_t need = (rows + rows_per_block - 1) / rows_per_block;
   const int64_t full = (int64_t)A->num_sms * per_sm;
   return (int)(need < full ? need : full);
@@ -164,16 +176,19 @@ cudaError_t run(const ens_matrix *A, int m, const void *X, void *Y, uint32_t mas
   if constexpr (!std::is_same<Arith, ArithF64Hybrid>::value) {
     if (direct) {
       auto k = capped ? gspmv_kernel_direct<Arith, VEC, LANES> : gspmv_kernel_direct_free<Arith, VEC, LANES>;
-      k<<<grid_for(A, v.n, (const void *)k, kThreads / LANES), kThreads, 0, s>>>(v, m, (const T *)X, y, mask);
+      static std::atomic<int> known{0};
+      k<<<grid_for(A, v.n, resident(known, (const void *)k, kThreads, 0), kThreads / LANES), kThreads, 0, s>>>(v, m, (const T *)X, y, mask);
       return cudaGetLastError();
     }
   }
   if constexpr (capped) {
     auto k = gspmv_kernel_capped<Arith, VEC, LANES>;
-    k<<<grid_for(A, v.n, (const void *)k, tile_rows_for(v.n, LANES)), kThreads, 0, s>>>(v, m, (const T *)X, y, mask);
+    static std::atomic<int> known{0};
+    k<<<grid_for(A, v.n, resident(known, (const void *)k, kThreads, 0), tile_rows_for(v.n, LANES)), kThreads, 0, s>>>(v, m, (const T *)X, y, mask);
   } else {
     auto k = gspmv_kernel<Arith, VEC, LANES>;
-    k<<<grid_for(A, v.n, (const void *)k, tile_rows_for(v.n, LANES)), kThreads, 0, s>>>(v, m, (const T *)X, y, mask);
+    static std::atomic<int> known{0};
+    k<<<grid_for(A, v.n, resident(known, (const void *)k, kThreads, 0), tile_rows_for(v.n, LANES)), kThreads, 0, s>>>(v, m, (const T *)X, y, mask);
   }
   return cudaGetLastError();
 }
