@@ -2,6 +2,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdint>
@@ -173,10 +174,19 @@ ens_status ens::create_matrix(int64_t n, int64_t ncols, int64_t nnz, const int32
     if (len > max_len) max_len = len;
   }
   if (row_ptr[n] != nnz) return fail(ENS_ERR_INVALID, "create_matrix: row_ptr[n] = %d != nnz = %lld", row_ptr[n], (long long)nnz);
-  for (int64_t j = 0; j < nnz; ++j)
-    if (col_idx[j] < 0 || col_idx[j] >= ncols)
-      return fail(ENS_ERR_INVALID, "create_matrix: col_idx[%lld] = %d outside [0, %lld)", (long long)j, col_idx[j],
-                  (long long)ncols);
+  std::atomic<int64_t> bad{INT64_MAX};  // the first column index out of range
+  host_parallel(nnz, 1 << 20, [&](int64_t b, int64_t e) {
+    for (int64_t j = b; j < e; ++j)
+      if (col_idx[j] < 0 || col_idx[j] >= ncols) {
+        int64_t seen = bad.load();
+        while (j < seen && !bad.compare_exchange_weak(seen, j)) {
+        }
+        return;
+      }
+  });
+  if (const int64_t j = bad.load(); j != INT64_MAX)
+    return fail(ENS_ERR_INVALID, "create_matrix: col_idx[%lld] = %d outside [0, %lld)", (long long)j, col_idx[j],
+                (long long)ncols);
 
   cudaStream_t s = (cudaStream_t)stream;
   ens_matrix *A = new ens_matrix();
@@ -233,16 +243,19 @@ ens_status ens::create_matrix(int64_t n, int64_t ncols, int64_t nnz, const int32
     const int64_t chunks = std::min<int64_t>(kPipeChunks, tiles);
     const int64_t per = (tiles + chunks - 1) / chunks * kPipeAlignRows;
     A->pipe_block_rows = std::max<int64_t>(1, (ncols + kPipeBlocks - 1) / kPipeBlocks);
-    for (int64_t r0 = 0; r0 < n; r0 += per) {
-      const int64_t r1 = std::min<int64_t>(n, r0 + per);
-      uint64_t mask[kPipeMaskWords] = {};
-      for (int64_t j = row_ptr[r0]; j < row_ptr[r1]; ++j) {
-        const int64_t b = (int64_t)col_idx[j] / A->pipe_block_rows;
-        mask[b / 64] |= 1ull << (b % 64);
+    const int64_t count = (n + per - 1) / per;
+    for (int64_t k = 0; k < count; ++k) A->pipe_row.push_back(k * per);
+    A->pipe_mask.assign((size_t)count * kPipeMaskWords, 0);
+    host_parallel(count, nnz > (1 << 20) ? 1 : count, [&](int64_t k0, int64_t k1) {  // whole chunks: no two threads share a mask
+      for (int64_t k = k0; k < k1; ++k) {
+        uint64_t *mask = A->pipe_mask.data() + k * kPipeMaskWords;
+        const int64_t r1 = std::min<int64_t>(n, (k + 1) * per);
+        for (int64_t j = row_ptr[k * per]; j < row_ptr[r1]; ++j) {
+          const uint32_t b = (uint32_t)col_idx[j] / (uint32_t)A->pipe_block_rows;
+          mask[b / 64] |= 1ull << (b % 64);
+        }
       }
-      A->pipe_row.push_back(r0);
-      A->pipe_mask.insert(A->pipe_mask.end(), mask, mask + kPipeMaskWords);
-    }
+    });
     A->pipe_row.push_back(n);
   }
   *out = A;

@@ -6,6 +6,8 @@
 #include <cstdint>
 #include <cstdio>
 #include <mutex>
+#include <algorithm>
+#include <thread>
 #include <vector>
 
 #include "ensemble_solve.h"
@@ -88,6 +90,24 @@ struct ens_amg {
 };
 
 namespace ens {
+
+// f(begin, end) over [0, n) on the host, in up to 16 threads of at least `grain` elements each.
+template <typename F>
+void host_parallel(int64_t n, int64_t grain, F &&f) {
+  const int64_t cores = std::max(1u, std::thread::hardware_concurrency());
+  const int64_t parts = std::max<int64_t>(1, std::min<int64_t>({cores, 16, n / grain}));
+  auto at = [&](int64_t p) { return n * p / parts; };
+  std::vector<std::thread> th;
+  int64_t started = 1;
+  try {
+    th.reserve(parts);
+    for (; started < parts; ++started) th.emplace_back([&, started] { f(at(started), at(started + 1)); });
+  } catch (...) {  // no more threads: the rest runs here
+  }
+  f(at(0), at(1));
+  for (int64_t p = started; p < parts; ++p) f(at(p), at(p + 1));
+  for (auto &t : th) t.join();
+}
 
 // The memory pool of A's scratch (nullptr: the device's default pool). The default pool gives everything back at
 // every synchronisation, so each solve mapped its blocks anew. Any thread, any stream.
