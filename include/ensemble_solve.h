@@ -75,7 +75,10 @@ typedef enum {
  *   val      float64[nnz]
  *   flags    ENS_MATRIX_SINGULAR or 0
  * The library also keeps a float32 copy of val (for ENS_F32 products), the inverse diagonal
- * (Jacobi scaling of the Chebyshev preconditioner) and a split-float copy of val.
+ * (Jacobi scaling of the Chebyshev preconditioner) and a split-float copy of val; for n >= 65536 and
+ * stencil-like structure (rows of at most 16 nonzeros) also the rows grouped into boxes (about 110 bytes
+ * per row of a seven-point operator; left out where device memory does not suffice). Solves on the matrix
+ * keep up to 128 MB of scratch between calls, freed with it.
  * Synchronous: returns after the copies end. *out receives the handle.
  * Errors: ENS_ERR_INVALID (structure), ENS_ERR_OOM, ENS_ERR_CUDA.
  */
@@ -102,7 +105,8 @@ ens_status ens_set_native_share(ens_matrix *A, int32_t share);
 /*
  * Autotuner: time the GSpMV launch candidates for block width m (1..64) and dtype on this matrix
  * (lanes per row, i.e. rows per warp and column-tile width; tiled or untiled rows; for FP64 also native
- * DFMA vs split-float with native shares 0, 8, 12, 16, 24 of 32, and the column hybrid) and keep the fastest for later
+ * DFMA vs split-float with native shares 0, 8, 12, 16, 24 of 32, and the column hybrid; row boxes where
+ * the matrix has them and m >= 3) and keep the fastest for later
  * ens_gspmv calls and for the solver's products of that width. Uses temporary device blocks of
  * n x m (stream-ordered, freed before return). Synchronous. Optional outputs: chosen lanes, chosen
  * share (32 = native, 64 = column hybrid), and the best time per launch in microseconds. A share
@@ -239,7 +243,7 @@ void ens_default_solve_opts(ens_solve_opts *o);
  * With ENS_MATRIX_SINGULAR the operator's null space is the constants: a column whose sum exceeds
  * 1e-10 sqrt(n) ||b_l|| is rejected (ENS_COL_INCOMPATIBLE) and every solution is returned with
  * zero mean. Supports 1 <= m <= 64. Synchronous: returns when X and stats are written.
- * Workspace (about 8-13 n x m blocks) is allocated stream-ordered for the call and released, or taken
+ * Workspace (about 8-11 n x m blocks) is allocated stream-ordered for the call and released, or taken
  * from opts->workspace when given (then nothing is allocated).
  */
 ens_status ens_solve_block(const ens_matrix *A, int32_t m, const double *B, double *X, const double *tol,
