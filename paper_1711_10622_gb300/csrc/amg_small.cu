@@ -27,20 +27,6 @@ constexpr int kTailBlocks = 8;  // portable cluster size; 16 gave 3 % on the mix
 constexpr int kTailThreads = 1024;
 constexpr size_t kTailSmem = 96 * 1024;
 
-// VEC elements written by another block of the cluster, or read once: from L2.
-template <typename T, int VEC>
-__device__ __forceinline__ void load_cg(const T *p, T (&v)[VEC]) {
-  using A = Access<T, VEC>;
-  using V = typename A::type;
-#pragma unroll
-  for (int h = 0; h < VEC / A::n; ++h) {
-    const V t = __ldcg(reinterpret_cast<const V *>(p) + h);
-    const T *e = reinterpret_cast<const T *>(&t);
-#pragma unroll
-    for (int q = 0; q < A::n; ++q) v[h * A::n + q] = e[q];
-  }
-}
-
 // This thread's part of row i's product with X, columns [c, c + VEC): nonzeros j0 + sub, j0 + sub + S, ...,
 // four gathers at a time, then the sum over the S threads of the row (lanes of one warp, `lanes` apart). Every
 // thread of a warp calls this the same number of times (valid = false: no row). (Dealing the rest of rows longer
@@ -69,7 +55,7 @@ __device__ __forceinline__ void row_part(bool valid, const int32_t *__restrict__
           if constexpr (SHARED)
             load_vec_rw<T, VEC>(X + (int64_t)k[u] * m + c, x[u]);
           else
-            load_cg<T, VEC>(X + (int64_t)k[u] * m + c, x[u]);
+            load_l2<VEC>(X + (int64_t)k[u] * m + c, x[u]);
         }
 #pragma unroll
       for (int u = 0; u < 4; ++u)
@@ -109,7 +95,7 @@ __device__ __forceinline__ void resid_rows(const Place &p, const int32_t *rp, co
     row_part<T, VEC, false>(ok, rp, ci, va, i, z, m, p.c, p.sub, S, lanes, w);
     if (ok && p.sub == 0) {
       T rv[VEC];
-      load_cg<T, VEC>(r + (int64_t)i * m + p.c, rv);
+      load_l2<VEC>(r + (int64_t)i * m + p.c, rv);
 #pragma unroll
       for (int q = 0; q < VEC; ++q) rv[q] -= w[q];
       store_vec<T, VEC>(res + (int64_t)i * m + p.c, rv);
@@ -129,8 +115,8 @@ __device__ __forceinline__ void smooth2_rows(const Place &p, const int32_t *rp, 
     row_part<T, VEC, false>(ok, rp, ci, va, i, src, m, p.c, p.sub, S, lanes, w);
     if (ok && p.sub == 0) {
       T sv[VEC], zv[VEC];
-      load_cg<T, VEC>(src + (int64_t)i * m + p.c, sv);
-      if (add) load_cg<T, VEC>(z + (int64_t)i * m + p.c, zv);
+      load_l2<VEC>(src + (int64_t)i * m + p.c, sv);
+      if (add) load_l2<VEC>(z + (int64_t)i * m + p.c, zv);
       const T dv = __ldg(dinv + i);
 #pragma unroll
       for (int q = 0; q < VEC; ++q) {
@@ -160,7 +146,7 @@ __device__ __forceinline__ void restrict_rows(const Place &p, const int32_t *__r
         T v[4][VEC];
 #pragma unroll
         for (int u = 0; u < 4; ++u)
-          if (t + u * S < t1) load_cg<T, VEC>(res + (int64_t)__ldg(mem + t + u * S) * m + p.c, v[u]);
+          if (t + u * S < t1) load_l2<VEC>(res + (int64_t)__ldg(mem + t + u * S) * m + p.c, v[u]);
 #pragma unroll
         for (int u = 0; u < 4; ++u)
           if (t + u * S < t1)
@@ -208,7 +194,7 @@ __device__ __forceinline__ void coarse_updates(const TailArgs<T> &a, const TailL
   for (int32_t i = p.grp; i < L.n; i += p.groups)
     if (p.col && p.sub == 0) {
       T sv[VEC], dv[VEC];
-      load_cg<T, VEC>(L.r + (int64_t)i * m + p.c, sv);
+      load_l2<VEC>(L.r + (int64_t)i * m + p.c, sv);
       const T sc = __ldg(L.dinv + i) * a.inv_theta;
 #pragma unroll
       for (int q = 0; q < VEC; ++q) dv[q] = sv[q] * sc;
@@ -255,7 +241,7 @@ __device__ __forceinline__ void coarse_dense(const TailArgs<T> &a, const TailLev
   const int32_t n = L.n, m = a.m, nv = m / VEC, lane = threadIdx.x & 31;
   for (int32_t t = threadIdx.x; t < n * nv; t += kTailThreads) {
     T v[VEC];
-    load_cg<T, VEC>(L.r + (int64_t)t * VEC, v);
+    load_l2<VEC>(L.r + (int64_t)t * VEC, v);
     store_vec<T, VEC>(r + (int64_t)t * VEC, v);
   }
   __syncthreads();
@@ -355,8 +341,8 @@ __global__ void __launch_bounds__(kTailThreads) k_amg_tail(const __grid_constant
     const TailLevel<T> &L = a.lev[l], &C = a.lev[l + 1];
     for (int32_t i = e.grp; i < L.n && e.col; i += e.groups) {
       T zv[VEC], cv[VEC];
-      load_cg<T, VEC>(L.z + (int64_t)i * m + e.c, zv);
-      load_cg<T, VEC>(C.z + (int64_t)__ldg(L.agg + i) * m + e.c, cv);
+      load_l2<VEC>(L.z + (int64_t)i * m + e.c, zv);
+      load_l2<VEC>(C.z + (int64_t)__ldg(L.agg + i) * m + e.c, cv);
 #pragma unroll
       for (int q = 0; q < VEC; ++q) zv[q] += cv[q];
       store_vec<T, VEC>(L.z + (int64_t)i * m + e.c, zv);

@@ -31,15 +31,9 @@ struct NoAfter {
   __device__ void operator()(bool) const {}
 };
 
-// after(any): runs once, on thread 0 of the last block, when every column's fin() has finished; any: some fin()
-// returned true (fin may return bool).
-template <typename T, int ND, int VEC, int LANES, typename Fin, typename After = NoAfter>
-__device__ __forceinline__ void reduce_cols(T (&acc)[ND][VEC], int32_t m, T *__restrict__ partials,
-                                            unsigned *__restrict__ counter, Fin &&fin, After &&after = After()) {
-  constexpr int kWarps = kThreads / 32;
-  __shared__ T wsum[kWarps][ND][LANES * VEC];
-  __shared__ ColTotals<T, ND> tot;
-  __shared__ bool is_last;
+// The warp's sums of every value and column, to wsum[warp] (no barrier).
+template <typename T, int ND, int VEC, int LANES>
+__device__ __forceinline__ void warp_cols(const T (&acc)[ND][VEC], T (&wsum)[kThreads / 32][ND][LANES * VEC]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   // Sums over the warp's row groups. While a lane holds several values it gives half of them to its partner and
   // adds the partner's share of the others, so ND * VEC values cost about that many additions instead of that many
@@ -77,6 +71,19 @@ __device__ __forceinline__ void reduce_cols(T (&acc)[ND][VEC], int32_t m, T *__r
         if (k < kVals) wsum[warp][k / VEC][(lane % LANES) * VEC + k % VEC] = v[i];
       }
   }
+}
+
+// after(any): runs once, on thread 0 of the last block, when every column's fin() has finished; any: some fin()
+// returned true (fin may return bool).
+template <typename T, int ND, int VEC, int LANES, typename Fin, typename After = NoAfter>
+__device__ __forceinline__ void reduce_cols(T (&acc)[ND][VEC], int32_t m, T *__restrict__ partials,
+                                            unsigned *__restrict__ counter, Fin &&fin, After &&after = After()) {
+  constexpr int kWarps = kThreads / 32;
+  __shared__ T wsum[kWarps][ND][LANES * VEC];
+  __shared__ ColTotals<T, ND> tot;
+  __shared__ bool is_last;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  warp_cols<T, ND, VEC, LANES>(acc, wsum);
   __syncthreads();
   for (int t = threadIdx.x; t < ND * m; t += kThreads) {  // block sums, warp by warp in a fixed order
     const int d = t / m, c = t - d * m;

@@ -75,6 +75,58 @@ __device__ __forceinline__ void load_vec(const T *__restrict__ p, T (&v)[VEC]) {
   }
 }
 
+// Elements written by other blocks of the same launch: from L2. Volatile: a load that is repeated after a barrier
+// between blocks must not be replaced by an earlier one's value.
+template <int VEC>
+__device__ __forceinline__ void load_l2(const double *p, double (&v)[VEC]) {
+  if constexpr (VEC == 1) {
+    asm volatile("ld.global.cg.f64 %0, [%1];" : "=d"(v[0]) : "l"(p) : "memory");
+  } else {
+#pragma unroll
+    for (int h = 0; h < VEC; h += 2) asm volatile("ld.global.cg.v2.f64 {%0, %1}, [%2];" : "=d"(v[h]), "=d"(v[h + 1]) : "l"(p + h) : "memory");
+  }
+}
+template <int VEC>
+__device__ __forceinline__ void load_l2(const float *p, float (&v)[VEC]) {
+  if constexpr (VEC == 1) {
+    asm volatile("ld.global.cg.f32 %0, [%1];" : "=f"(v[0]) : "l"(p) : "memory");
+  } else if constexpr (VEC == 2) {
+    asm volatile("ld.global.cg.v2.f32 {%0, %1}, [%2];" : "=f"(v[0]), "=f"(v[1]) : "l"(p) : "memory");
+  } else {
+#pragma unroll
+    for (int h = 0; h < VEC; h += 4)
+      asm volatile("ld.global.cg.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v[h]), "=f"(v[h + 1]), "=f"(v[h + 2]), "=f"(v[h + 3]) : "l"(p + h) : "memory");
+  }
+}
+
+// How a row product reads X: through the read-only path (X is not written while the kernel runs), or by ordinary
+// loads (X was written earlier in the launch by other blocks and acquired at a barrier since, which drops older lines
+// from L1; volatile as in load_l2).
+struct ReadOnly {
+  template <typename T, int VEC>
+  __device__ __forceinline__ static void load(const T *p, T (&v)[VEC]) {
+    load_vec<T, VEC>(p, v);
+  }
+  __device__ __forceinline__ static double2 load2(const double2 *p) { return __ldg(p); }
+};
+struct Coherent {
+  template <typename T, int VEC>
+  __device__ __forceinline__ static void load(const T *p, T (&v)[VEC]) {
+    static_assert(std::is_same<T, double>::value && VEC <= 2, "the widths in use");
+    if constexpr (VEC == 1) {
+      asm volatile("ld.global.f64 %0, [%1];" : "=d"(v[0]) : "l"(p) : "memory");
+    } else {
+      const double2 t = load2(reinterpret_cast<const double2 *>(p));
+      v[0] = t.x, v[1] = t.y;
+    }
+  }
+  __device__ __forceinline__ static double2 load2(const double2 *p) {
+    double2 t;
+    asm volatile("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(t.x), "=d"(t.y) : "l"(p) : "memory");
+    return t;
+  }
+};
+
 // Same, for data written earlier in the same kernel launch by this thread (no read-only path).
 template <typename T, int VEC>
 __device__ __forceinline__ void load_vec_rw(const T *p, T (&v)[VEC]) {
@@ -127,9 +179,9 @@ constexpr int kUnroll = 4;
 // round trips instead of four); for double data the extra registers of that form cost more
 // occupancy than they save (measured on GB300: native m = 2, 129 us against 159 us), so the tail
 // is processed one nonzero at a time.
-template <typename T, typename V, int VEC>
+template <typename T, typename V, int VEC, typename LD = ReadOnly>
 __device__ __forceinline__ void row_plain(int32_t j0, int32_t j1, const int32_t *ci, const V *va, int32_t m,
-                                          int32_t c, const T *__restrict__ X, T (&acc)[VEC]) {
+                                          int32_t c, const T *X, T (&acc)[VEC]) {
   constexpr bool kGroupTail = sizeof(T) == 4;
   constexpr int U = kUnroll;
 #pragma unroll
@@ -145,7 +197,7 @@ __device__ __forceinline__ void row_plain(int32_t j0, int32_t j1, const int32_t 
     }
     T x[U][VEC];
 #pragma unroll
-    for (int u = 0; u < U; ++u) load_vec<T, VEC>(X + (int64_t)k[u] * m + c, x[u]);
+    for (int u = 0; u < U; ++u) LD::template load<T, VEC>(X + (int64_t)k[u] * m + c, x[u]);
 #pragma unroll
     for (int u = 0; u < U; ++u)
 #pragma unroll
@@ -166,7 +218,7 @@ __device__ __forceinline__ void row_plain(int32_t j0, int32_t j1, const int32_t 
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         if (u < len) {
-          load_vec<T, VEC>(X + (int64_t)k[u] * m + c, x[u]);
+          LD::template load<T, VEC>(X + (int64_t)k[u] * m + c, x[u]);
         } else {
 #pragma unroll
           for (int q = 0; q < VEC; ++q) x[u][q] = T(0);
@@ -183,7 +235,7 @@ __device__ __forceinline__ void row_plain(int32_t j0, int32_t j1, const int32_t 
       const int32_t k = ci[j];
       const T a = (T)va[j];
       T x[VEC];
-      load_vec<T, VEC>(X + (int64_t)k * m + c, x);
+      LD::template load<T, VEC>(X + (int64_t)k * m + c, x);
 #pragma unroll
       for (int q = 0; q < VEC; ++q) acc[q] = fma(a, x[q], acc[q]);
     }
@@ -305,17 +357,17 @@ __device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
 }
 
 // Native DFMA row product (the split path's fallback and the FP64 share of hybrid tiles).
-template <int VEC>
+template <int VEC, typename LD = ReadOnly>
 __device__ __forceinline__ void row_native_f64(int32_t j0, int32_t j1, const int32_t *ci, const double *__restrict__ vn,
                                                int32_t m, int32_t c, const double *__restrict__ X, double (&z)[VEC]) {
-  row_plain<double, double, VEC>(j0, j1, ci, vn, m, c, X, z);
+  row_plain<double, double, VEC, LD>(j0, j1, ci, vn, m, c, X, z);
 }
 
 // Split-float row product. ci / vs (hi, lo pairs) are indexed by j in [j0, j1) and point into a
 // shared-memory tile or into global memory; vn is the float64 value array under the same index
 // (global), used when a column's X values leave the split range. Each column decides on its own,
 // so one column's values never change another column's result.
-template <int VEC>
+template <int VEC, typename LD = ReadOnly>
 __device__ __forceinline__ void row_split(int32_t j0, int32_t j1, const int32_t *ci, const float2 *vs,
                                           const double *__restrict__ vn, int32_t m, int32_t c,
                                           const double *__restrict__ X, double (&y)[VEC]) {
@@ -332,7 +384,7 @@ __device__ __forceinline__ void row_split(int32_t j0, int32_t j1, const int32_t 
 #pragma unroll
     for (int u = 0; u < kUnroll; ++u) {
       const int32_t k = ci[u < len ? j + u : j];
-      load_vec<double, VEC>(X + (int64_t)k * m + c, x[u]);
+      LD::template load<double, VEC>(X + (int64_t)k * m + c, x[u]);
     }
 #pragma unroll
     for (int u = 0; u < kUnroll; ++u) {
@@ -357,7 +409,7 @@ __device__ __forceinline__ void row_split(int32_t j0, int32_t j1, const int32_t 
   }
   if (!all_ok) {
     double z[VEC];
-    row_native_f64<VEC>(j0, j1, ci, vn, m, c, X, z);
+    row_native_f64<VEC, LD>(j0, j1, ci, vn, m, c, X, z);
 #pragma unroll
     for (int q = 0; q < VEC; ++q) y[q] = ok[q] ? y[q] : z[q];
   }
@@ -407,7 +459,7 @@ __device__ __forceinline__ const double2 *xrow(const char *xc, int32_t k, uint32
   return reinterpret_cast<const double2 *>(xc + (uint64_t)(uint32_t)k * row_bytes);
 }
 
-template <typename AV>
+template <typename AV, typename LD = ReadOnly>
 __device__ __forceinline__ void row_split2(int32_t j0, int32_t j1, const int32_t *ci, const AV *va,
                                            const double *__restrict__ vn, int32_t m, int32_t c,
                                            const double *__restrict__ X, double (&y)[2]) {
@@ -420,7 +472,7 @@ __device__ __forceinline__ void row_split2(int32_t j0, int32_t j1, const int32_t
   for (; j + kUnroll <= j1; j += kUnroll) {
     double2 x[kUnroll];
 #pragma unroll
-    for (int u = 0; u < kUnroll; ++u) x[u] = __ldg(xrow(xc, ci[j + u], rb));
+    for (int u = 0; u < kUnroll; ++u) x[u] = LD::load2(xrow(xc, ci[j + u], rb));
 #pragma unroll
     for (int u = 0; u < kUnroll; ++u) split_acc2(split_pair(va[j + u]), x[u].x, x[u].y, g23, sh, sl, rng0, rng1);
   }
@@ -432,7 +484,7 @@ __device__ __forceinline__ void row_split2(int32_t j0, int32_t j1, const int32_t
     for (int u = 0; u < kUnroll - 1; ++u) {
       const bool v = u < len;
       const int32_t jj = v ? j + u : j;
-      x[u] = __ldg(xrow(xc, ci[jj], rb));
+      x[u] = LD::load2(xrow(xc, ci[jj], rb));
       a[u] = split_pair(va[jj]);
       if (!v) a[u] = SplitPair{0ull, 0ull};
     }
@@ -447,7 +499,7 @@ __device__ __forceinline__ void row_split2(int32_t j0, int32_t j1, const int32_t
   y[1] = split_to_double(h1, l1);
   if (!(ok0 && ok1)) {
     double z[2];
-    row_native_f64<2>(j0, j1, ci, vn, m, c, X, z);
+    row_native_f64<2, LD>(j0, j1, ci, vn, m, c, X, z);
     y[0] = ok0 ? y[0] : z[0];
     y[1] = ok1 ? y[1] : z[1];
   }
@@ -632,10 +684,10 @@ struct ArithF32 {
     stage16<int32_t>(sm.ci, A.ci + ab, ae - ab);
     stage16<float>(sm.va, A.val32 + ab, ae - ab);
   }
-  template <int VEC>
+  template <int VEC, typename LD = ReadOnly>
   __device__ __forceinline__ static void row_s(const Tile &sm, const MatView &, int32_t, int32_t j0, int32_t j1,
                                                int32_t m, int32_t c, const float *X, float (&y)[VEC], bool) {
-    row_plain<float, float, VEC>(j0, j1, sm.ci, sm.va, m, c, X, y);
+    row_plain<float, float, VEC, LD>(j0, j1, sm.ci, sm.va, m, c, X, y);
   }
   template <int VEC>
   __device__ __forceinline__ static void row_g(const MatView &A, int32_t ab, int32_t j0, int32_t j1, int32_t m,
@@ -651,10 +703,10 @@ struct ArithF64Native {
     stage16<int32_t>(sm.ci, A.ci + ab, ae - ab);
     stage16<double>(sm.va, A.val + ab, ae - ab);
   }
-  template <int VEC>
+  template <int VEC, typename LD = ReadOnly>
   __device__ __forceinline__ static void row_s(const Tile &sm, const MatView &, int32_t, int32_t j0, int32_t j1,
                                                int32_t m, int32_t c, const double *X, double (&y)[VEC], bool) {
-    row_plain<double, double, VEC>(j0, j1, sm.ci, sm.va, m, c, X, y);
+    row_plain<double, double, VEC, LD>(j0, j1, sm.ci, sm.va, m, c, X, y);
   }
   template <int VEC>
   __device__ __forceinline__ static void row_g(const MatView &A, int32_t ab, int32_t j0, int32_t j1, int32_t m,
@@ -674,30 +726,30 @@ struct ArithF64Split {
     stage16<int32_t>(sm.ci, A.ci + ab, ae - ab);
     stage16<float2>(sm.va, A.vs + ab, ae - ab);
   }
-  template <int VEC>
+  template <int VEC, typename LD = ReadOnly>
   __device__ __forceinline__ static void row_s(const Tile &sm, const MatView &A, int32_t ab, int32_t j0, int32_t j1,
                                                int32_t m, int32_t c, const double *X, double (&y)[VEC], bool native) {
     if (native) {
-      row_native_f64<VEC>(j0, j1, sm.ci, A.val + ab, m, c, X, y);
+      row_native_f64<VEC, LD>(j0, j1, sm.ci, A.val + ab, m, c, X, y);
     } else if constexpr (VEC == 2) {
-      row_split2<float2>(j0, j1, sm.ci, sm.va, A.val + ab, m, c, X, y);
+      row_split2<float2, LD>(j0, j1, sm.ci, sm.va, A.val + ab, m, c, X, y);
     } else if constexpr (VEC == 4) {
       row_split_pairs<2, float2>(j0, j1, sm.ci, sm.va, A.val + ab, m, c, X, y);
     } else {
-      row_split<VEC>(j0, j1, sm.ci, A.vs + ab, A.val + ab, m, c, X, y);
+      row_split<VEC, LD>(j0, j1, sm.ci, A.vs + ab, A.val + ab, m, c, X, y);
     }
   }
-  template <int VEC>
+  template <int VEC, typename LD = ReadOnly>
   __device__ __forceinline__ static void row_g(const MatView &A, int32_t ab, int32_t j0, int32_t j1, int32_t m,
                                                int32_t c, const double *X, double (&y)[VEC], bool native) {
     if (native) {
-      row_native_f64<VEC>(j0, j1, A.ci + ab, A.val + ab, m, c, X, y);
+      row_native_f64<VEC, LD>(j0, j1, A.ci + ab, A.val + ab, m, c, X, y);
     } else if constexpr (VEC == 2) {
-      row_split2<float2>(j0, j1, A.ci + ab, A.vs + ab, A.val + ab, m, c, X, y);
+      row_split2<float2, LD>(j0, j1, A.ci + ab, A.vs + ab, A.val + ab, m, c, X, y);
     } else if constexpr (VEC == 4) {
       row_split_pairs<2, float2>(j0, j1, A.ci + ab, A.vs + ab, A.val + ab, m, c, X, y);
     } else {
-      row_split<VEC>(j0, j1, A.ci + ab, A.vs + ab, A.val + ab, m, c, X, y);
+      row_split<VEC, LD>(j0, j1, A.ci + ab, A.vs + ab, A.val + ab, m, c, X, y);
     }
   }
   __device__ __forceinline__ static double dinv(const MatView &A, int64_t i) { return __ldg(A.dinv + i); }

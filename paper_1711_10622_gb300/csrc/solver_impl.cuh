@@ -36,6 +36,7 @@
 #include "ens_internal.cuh"
 #include "reduce.cuh"
 #include "rowprod.cuh"
+#include "solver_small.cuh"
 
 namespace ens {
 
@@ -97,6 +98,51 @@ __device__ __forceinline__ void step_omega(const Cols<T> &cs, int l, T ts, T t2)
     return;
   }
   cs.omega[l] = om;
+}
+// After (s, s): a column that meets its tolerance ends with the half step.
+template <typename T>
+__device__ __forceinline__ void step_half(const Cols<T> &cs, int l, T ss) {
+  if (cs.state[l] == ST_ACTIVE && ss <= cs.thr2[l]) cs.state[l] = ST_HALF;
+}
+// After ||r||^2 and (rhat, r), which end iteration `it`: convergence and breakdown tests, beta and rho of the next
+// iteration. True if the column goes on.
+template <typename T>
+__device__ __forceinline__ bool step_end(const Cols<T> &cs, int l, T rn2, T rr, int32_t it, int32_t max_iter) {
+  const int st = cs.state[l];
+  if (st == ST_HALF) {
+    cs.state[l] = ST_DONE;
+    cs.status[l] = ENS_COL_CONVERGED;
+    return false;
+  }
+  if (st != ST_ACTIVE) return st != ST_DONE;
+  cs.rn2[l] = rn2;
+  bool on = false;
+  if (!isfinite(rn2)) {
+    cs.status[l] = ENS_COL_NONFINITE;
+  } else if (rn2 <= cs.thr2[l]) {
+    cs.status[l] = ENS_COL_CONVERGED;
+  } else if (cs.omega[l] == T(0)) {
+    cs.status[l] = ENS_COL_BREAKDOWN;
+  } else if (it < max_iter) {  // the next iteration begins: rho and its breakdown test
+    // |rho| <= tiny ||rhat|| ||r||; the product of the norms is at most the larger square, so the roots are
+    // only taken when that already fails
+    const T rh2 = cs.rh2[l], a = fabs(rr);
+    if (!isfinite(rr)) {
+      cs.status[l] = ENS_COL_NONFINITE;
+      cs.iters[l] = it + 1;
+    } else if (a <= T(2) * Tiny<T>::v * fmax(rh2, rn2) && a <= Tiny<T>::v * sqrt(rh2) * sqrt(rn2)) {
+      cs.status[l] = ENS_COL_BREAKDOWN;
+      cs.iters[l] = it + 1;
+    } else {
+      cs.beta[l] = (rr / cs.rho[l]) * (cs.alpha[l] / cs.omega[l]);
+      cs.rho[l] = rr;
+      on = true;
+    }
+  } else {
+    on = true;  // out of iterations: the column ends as it is
+  }
+  if (!on) cs.state[l] = ST_DONE;
+  return on;
 }
 // After ||b - A x||^2: the reported residual, or (outer) the convergence test of the refinement loop.
 template <typename T>
@@ -404,7 +450,7 @@ __global__ void __launch_bounds__(kThreads, 4)
     }
   }
   reduce_cols<T, 1, VEC, LANES>(acc, m, partials, counter, [&](int l, const ColTotals<T, 1> &t) {
-    if (cs.state[l] == ST_ACTIVE && t.v[0][l] <= cs.thr2[l]) cs.state[l] = ST_HALF;
+    step_half<T>(cs, l, t.v[0][l]);
   });
 }
 
@@ -482,42 +528,7 @@ __global__ void __launch_bounds__(kThreads)
   }
   const int32_t it = cs.it[0] + 1;  // the iteration this launch completes
   reduce_cols<T, 2, VEC, LANES>(acc, m, partials, counter, [&](int l, const ColTotals<T, 2> &tt) -> bool {
-    const int st = cs.state[l];
-    if (st == ST_HALF) {
-      cs.state[l] = ST_DONE;
-      cs.status[l] = ENS_COL_CONVERGED;
-      return false;
-    }
-    if (st != ST_ACTIVE) return st != ST_DONE;
-    const T rn2 = tt.v[0][l], rr = tt.v[1][l];
-    cs.rn2[l] = rn2;
-    bool on = false;
-    if (!isfinite(rn2)) {
-      cs.status[l] = ENS_COL_NONFINITE;
-    } else if (rn2 <= cs.thr2[l]) {
-      cs.status[l] = ENS_COL_CONVERGED;
-    } else if (cs.omega[l] == T(0)) {
-      cs.status[l] = ENS_COL_BREAKDOWN;
-    } else if (it < max_iter) {  // the next iteration begins: rho and its breakdown test
-      // |rho| <= tiny ||rhat|| ||r||; the product of the norms is at most the larger square, so the roots are
-      // only taken when that already fails
-      const T rh2 = cs.rh2[l], a = fabs(rr);
-      if (!isfinite(rr)) {
-        cs.status[l] = ENS_COL_NONFINITE;
-        cs.iters[l] = it + 1;
-      } else if (a <= T(2) * Tiny<T>::v * fmax(rh2, rn2) && a <= Tiny<T>::v * sqrt(rh2) * sqrt(rn2)) {
-        cs.status[l] = ENS_COL_BREAKDOWN;
-        cs.iters[l] = it + 1;
-      } else {
-        cs.beta[l] = (rr / cs.rho[l]) * (cs.alpha[l] / cs.omega[l]);
-        cs.rho[l] = rr;
-        on = true;
-      }
-    } else {
-      on = true;  // out of iterations: the column ends as it is
-    }
-    if (!on) cs.state[l] = ST_DONE;
-    return on;
+    return step_end<T>(cs, l, tt.v[0][l], tt.v[1][l], it, max_iter);
   }, [&](bool any) {
     cs.it[0] = it;
     const bool go = any && it < max_iter;
@@ -1260,8 +1271,8 @@ struct Bicg {
     }
     // the same for every width (not the grids of this one): a server fits the workspace as beta + gamma m
     if (e == cudaSuccess) e = sc.get(&partials, (size_t)num_sms * std::max(4, TileBlocks<Arith>::value) * 3 * kMaxSolveM);
-    if (e == cudaSuccess) e = sc.get(&counter, 1);
-    if (e == cudaSuccess) e = cudaMemsetAsync(counter, 0, sizeof(unsigned), s);
+    if (e == cudaSuccess) e = sc.get(&counter, 3);  // of the reductions; [1], [2]: barrier of iterate_small
+    if (e == cudaSuccess) e = cudaMemsetAsync(counter, 0, 3 * sizeof(unsigned), s);
     if (e == cudaSuccess) e = alloc_cols(sc, mp, cs);
     return e;
   }
@@ -1527,7 +1538,28 @@ struct Bicg {
     return e;
   }
 
+  // The loop in one launch where the system is small enough for every block to be resident (solver_small.cu): the
+  // same bits as the graph.
+  bool iterate_small(T *x, int max_iter, int *ran, cudaError_t *e) {
+    if constexpr (std::is_same<Arith, ArithF64Split>::value) {
+      if (prec || use_amg || boxes || max_iter <= 0) return false;
+      const SmallSolve a{A, mp, max_iter, tgrid, grid, sgrid, mask, x, r, p, v, s_, t, rh, partials, counter + 1};
+      const int blocks = small_solve_blocks(a, tile_count(n, lanes), num_sms);
+      if (!blocks) return false;
+      unsigned gave_up = 0;
+      *e = cudaMemsetAsync(counter + 1, 0, 2 * sizeof(unsigned), s);
+      if (*e == cudaSuccess) *e = launch_small_solve(a, cs, blocks, s);
+      if (*e == cudaSuccess) *e = cudaMemcpyAsync(&gave_up, counter + 2, sizeof(unsigned), cudaMemcpyDeviceToHost, s);
+      if (*e == cudaSuccess) *e = iterations_run(ran);
+      if (*e == cudaSuccess && gave_up) *e = cudaErrorLaunchTimeout;
+      return true;
+    }
+    return false;
+  }
+
   cudaError_t iterate(T *x, int max_iter, int check_every, bool graph, int *ran) {
+    cudaError_t e = cudaSuccess;
+    if (graph && iterate_small(x, max_iter, ran, &e)) return e;
     return graph ? iterate_graph(x, max_iter, ran) : iterate_host(x, max_iter, check_every, ran);
   }
 
