@@ -715,7 +715,9 @@ ens_status solve_coupled(const ens_matrix *M, int32_t m, const double *B, double
   ens_status gst = ENS_OK;
   int it = 0;
   {
-    Scratch sc(s, M, o);
+    // From the default pool: ens_block_dots takes its scratch there in every iteration, and with nothing else in use the
+    // default pool unmaps at each synchronisation (32^3 rows, m = 4: 487 us an iteration from the matrix's pool, 211 so).
+    Scratch sc(s);
     // per-column start checks on the device: ||b||^2, sum(b), non-finite entries of b and x0
     const int rgrid = (int)std::max<int64_t>(1, std::min<int64_t>((n * m + 255) / 256, (int64_t)M->num_sms * 4));
     double *rpart = nullptr, *rout = nullptr;

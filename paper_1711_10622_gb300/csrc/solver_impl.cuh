@@ -724,6 +724,7 @@ struct Scratch {
   char *arena = nullptr;
   size_t cap = 0, used = 0;
   bool overflow = false;
+  explicit Scratch(cudaStream_t st) : s(st) {}  // from the device's default pool
   Scratch(cudaStream_t st, const ens_matrix *A) : s(st), pool(scratch_pool(A)) {}
   Scratch(cudaStream_t st, const ens_matrix *A, const ens_solve_opts &o)
       : s(st), pool(o.workspace ? nullptr : scratch_pool(A)), arena((char *)o.workspace), cap(o.workspace_bytes) {}
