@@ -213,7 +213,7 @@ cudaError_t build_box(ens_matrix *A, const int32_t *rp, const int32_t *ci, cudaS
   if (n < kBoxMinRows || K < 1 || K > kBoxMaxLen || (double)nnz < 0.75 * (double)K * (double)n) return cudaSuccess;
   int64_t s1 = 0, s2 = 0;
   common_steps(n, rp, ci, s1, s2);
-  const int64_t per_min = 1 << 16;
+  const int64_t per_min = 1 << 13;
   const int parts = (int)std::max<int64_t>(1, std::min<int64_t>({(int64_t)std::max(1u, std::thread::hardware_concurrency()), 16, n / per_min}));
   std::vector<Part> part(parts);
   // ranges end on whole bricks of planes where the planes are known
