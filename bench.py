@@ -32,7 +32,7 @@ WORKLOAD = "channel256x128x128"
 M_SWEEP = (1, 2, 4, 8, 16, 32)
 FALLBACK_HBM_GBS = 6800.0
 PROFILE_SUMMARY = os.path.join(ROOT, "profiles", "gspmv_tile_m32_channel.md")
-KERNEL_SOURCES = [os.path.join(ROOT, "paper_1711_10622_gb300", "csrc", f) for f in ("rowprod.cuh", "gspmv.cu")]
+KERNEL_SOURCES = [os.path.join(ROOT, "paper_1711_10622_gb300", "csrc", f) for f in ("rowprod.cuh", "boxprod.cuh", "gspmv.cu")]
 
 
 def alg_bytes(n: int, nnz: int, m: int, sv: int = 8, sx: int = 8) -> int:
