@@ -120,8 +120,15 @@ cudaError_t run_box(const ens_matrix *A, int m, const void *X, void *Y, cudaStre
   using S = BoxShape<T, CW>;
   auto k = gspmv_kernel_box<T, CW, ACC, FULL, K0>;
   const size_t smem = S::smem(A->box.K);
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
+  // Once per kernel instance and device, for the longest rows: the call costs a tenth of a small product's launch, and
+  // a size by row length could be lowered by another thread before this one launches.
+  static std::atomic<uint64_t> allowed{0};
+  const uint64_t bit = A->device < 64 ? 1ull << A->device : 0;
+  if (!(allowed.load(std::memory_order_acquire) & bit)) {
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem(kBoxMaxLen));
+    if (e != cudaSuccess) return e;
+    allowed.fetch_or(bit, std::memory_order_release);
+  }
   static std::atomic<int> known[kBoxMaxLen + 1];  // by row length: the shared memory depends on it
   const int64_t full = (int64_t)A->num_sms * resident(known[A->box.K], (const void *)k, S::kThr, smem);
   k<<<(unsigned)(full < A->box.boxes ? full : (int64_t)A->box.boxes), S::kThr, smem, s>>>(A->box, view_of(A), m, (const T *)X, (T *)Y);

@@ -246,7 +246,8 @@ template <typename T, int CW, typename Kern, typename... Args>
 cudaError_t go(const BoxPlan &B, int chunks, int sms, cudaStream_t st, Kern k, Args... args) {
   using S = BoxShape<T, CW>;
   const size_t smem = S::smem(B.K);
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // for the longest rows: a size by row length could be lowered by another thread before this one launches
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem(kBoxMaxLen));
   if (e != cudaSuccess) return e;
   int64_t per = (int64_t)sms * S::kBlocks / chunks;
   per = std::max<int64_t>(1, std::min<int64_t>(per, B.boxes));

@@ -26,13 +26,15 @@ def ens():
     return ens
 
 
-def _stencil9(nx, ny):
-    """A two-dimensional nine-point operator with missing entries: rows of 4 to 9 nonzeros, some empty."""
+def _stencil9(nx, ny, points=9):
+    """A two-dimensional nine-point (or five-point) operator with missing entries: rows of 4 to 9 nonzeros, some empty."""
     rng = np.random.default_rng(nx)
     j, i = np.divmod(np.arange(nx * ny), nx)
     cols, keep = [], []
     for dj in (-1, 0, 1):
         for di in (-1, 0, 1):
+            if points == 5 and di and dj:
+                continue
             a, b = i + di, j + dj
             cols.append(b * nx + a)
             keep.append((a >= 0) & (a < nx) & (b >= 0) & (b < ny))
@@ -146,3 +148,32 @@ def test_repeatable(ens):
     with ens.Matrix.from_operator(op) as A:
         Y = ens.gspmv(A, X)
         assert all(torch.equal(Y, ens.gspmv(A, X)) for _ in range(3))
+
+
+def test_threads_with_rows_of_different_lengths(ens):
+    """Two threads multiply with matrices whose boxes need different amounts of shared memory."""
+    import threading
+
+    ops = [_stencil9(301, 257), _stencil9(301, 257, 5)]
+    X = gen.rhs_normal(ops[0].n, 8, 4)
+    bad = []
+
+    def work(op):
+        try:
+            s = torch.cuda.Stream()
+            with torch.cuda.stream(s), ens.Matrix.from_operator(op) as A:
+                x = torch.from_numpy(X).cuda()
+                want = ens.gspmv(A, x)
+                for _ in range(300):
+                    if not torch.equal(ens.gspmv(A, x), want):
+                        bad.append(op.name)
+                _check(op, X, want.cpu().numpy())
+        except Exception as e:  # noqa: BLE001
+            bad.append(e)
+
+    ts = [threading.Thread(target=work, args=(op,)) for op in ops]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join()
+    assert not bad
