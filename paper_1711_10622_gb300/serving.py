@@ -281,8 +281,7 @@ class Server:
         hierarchy); beta, gamma per operator from the workspace bytes of probe solves."""
         import torch
 
-        from .api import Matrix, solve_block
-        from . import _native as N
+        from .api import Matrix
 
         alpha, rows, samples = {}, {}, {}
         for name, op in operators.items():
@@ -295,17 +294,34 @@ class Server:
             alpha[name] = max(0, free0 - torch.cuda.mem_get_info()[0])
             self.mats[name] = A
             rows[name] = op.n
-            pts = []
-            for m in sorted({w for w in self.PROBE_WIDTHS if w <= max_cols} | {max_cols}):
-                B = torch.zeros((op.n, m), dtype=torch.float64, device="cuda")
-                # b = 0: every column finishes at the start; the call still sets up its full workspace
-                solve_block(A, B, None, tol=1e-8, precond=self.precond, precision=self.precision, max_iter=1,
-                            max_outer=1, inner_max_iter=0)
-                pts.append((m, int(N.lib().ens_last_workspace_bytes())))
-                del B
+            widths = sorted({w for w in self.PROBE_WIDTHS if w <= max_cols} | {max_cols})
+            pts = [(m, self._probe_workspace(A, op.n, m)) for m in widths]
             samples[name] = pts
-        torch.cuda.empty_cache()
+            torch.cuda.empty_cache()
         return MemoryModel.fit(alpha, rows, samples)
+
+    def _probe_workspace(self, A, n, m) -> int:
+        """Bytes that a solve of m columns takes, from a probe in a workspace of its own, grown until the solve fits:
+        scratch of the library's would stay with the matrix (up to 128 MB) beside the pool that served solves run in."""
+        import torch
+
+        from .api import solve_block
+        from . import _native as N
+
+        B = torch.zeros((n, m), dtype=torch.float64, device="cuda")
+        size = 8 * 8 * n * (m + m % 2) + (1 << 20)
+        while True:
+            ws = torch.empty(size, dtype=torch.uint8, device="cuda")
+            try:
+                # b = 0: every column finishes at the start; the call still sets up its full workspace
+                solve_block(A, B, None, tol=1e-8, precond=self.precond, precision=self.precision, max_iter=1, max_outer=1,
+                            inner_max_iter=0, workspace=ws.data_ptr(), workspace_bytes=size)
+                return int(N.lib().ens_last_workspace_bytes())
+            except N.EnsError as e:
+                if e.status != N.ENS_ERR_BUDGET:
+                    raise
+                ws = None
+                size = max(size + size // 4, int(N.lib().ens_last_workspace_bytes()))
 
     def _reserve_pool(self, model: MemoryModel) -> int:
         import torch

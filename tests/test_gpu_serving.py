@@ -122,3 +122,22 @@ def test_memory_model_fitted_on_the_device(ens):
             assert (r.stats["status"] == 0).all()
             assert r.workspace_bytes == M.cost(r.op, r.batch_cols)
         assert srv.sched.pool.in_use == 0 and srv.sched.pool.peak > 0
+
+
+def test_server_stays_inside_its_budget(ens):
+    """What the server holds on the device after start-up is its model's resident part and its pool: the probe
+    solves leave no scratch of theirs behind (32 MB beyond that for allocation granularity)."""
+    from paper_1711_10622_gb300.serving import Server
+
+    ops = {"a": gen.dirichlet_box(64), "b": gen.channel(64, 64, 64)}
+    for op in ops.values():  # kernels and graphs loaded before the first reading
+        with ens.Matrix.from_operator(op) as A:
+            ens.solve_block(A, torch.ones(op.n, 1, dtype=torch.float64, device="cuda"), tol=1e-2, precond="chebyshev", precision="mixed")
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    free0 = torch.cuda.mem_get_info()[0]
+    with Server(ops, budget_bytes=4e9, slots=1, max_cols=16) as srv:
+        torch.cuda.synchronize()
+        used = free0 - torch.cuda.mem_get_info()[0]
+        assert used <= srv.model.resident + srv.pool_tensor.numel() + (32 << 20)
+        assert used <= 4e9 + (32 << 20)
