@@ -127,6 +127,31 @@ def test_smallest_products(ens, ex):
         _check(op, X, ens.gspmv(A, torch.from_numpy(X).cuda()).cpu().numpy())
 
 
+def _us(f, n=9):
+    """Median time of f() in microseconds, after three untimed calls."""
+    t = []
+    for k in range(n + 3):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        f()
+        b.record()
+        torch.cuda.synchronize()
+        if k > 2:
+            t.append(a.elapsed_time(b) * 1e3)
+    return float(np.median(t))
+
+
+@pytest.mark.parametrize("m,most", [(8, 4.1), (16, 4.5)])
+def test_small_values_cost(ens, m, most):
+    """A block whose values all lie below the split range goes to native products, two columns per access: 3.5 and 3.7
+    times the time of one inside it (one column per access 4.6 and 5.7)."""
+    op = gen.channel(128, 128, 128)
+    X = torch.randn(op.n, m, dtype=torch.float64, device="cuda")
+    T, Y = X * 1e-30, torch.empty_like(X)
+    with ens.Matrix.from_operator(op) as A:
+        assert _us(lambda: ens.gspmv(A, T, Y)) <= most * _us(lambda: ens.gspmv(A, X, Y))
+
+
 @pytest.mark.parametrize("dtype", [np.float64, np.float32])
 def test_nonfinite(ens, dtype):
     """Infinities and NaN reach exactly the rows whose entries name them, as in the definition."""
