@@ -119,6 +119,21 @@ def test_vcycle_boxes(ens, m):
     _vcycle(ens, _cubes(), m, dict(theta=0.08, max_levels=8))
 
 
+@pytest.mark.parametrize("name", ["cubes97x43x37", "dirichlet48"])
+def test_float32_cycle_error(ens, name):
+    """The float32 cycle by row boxes (m = 8) is as close to the float64 one as row by row (the same columns with m = 6):
+    both round as often, so their errors agree to a few percent where no rounding repeats from row to row."""
+    op = _cubes() if name.startswith("cubes") else gen.dirichlet_box(48)
+    R = torch.randn(op.n, 8, device="cuda", generator=torch.Generator(device="cuda").manual_seed(5))
+    err = []
+    with ens.Matrix.from_operator(op) as A:
+        A.amg_setup()
+        Z = ens.amg_apply(A, R.double())[:, :6]
+        for m in (6, 8):
+            err.append(float((ens.amg_apply(A, R[:, :m].contiguous()).double()[:, :6] - Z).norm() / Z.norm()))
+    assert err[1] <= 1.15 * err[0], err
+
+
 @pytest.mark.parametrize("m", [1, 2, 5, 8, 33, 64])
 @pytest.mark.parametrize("nx,opts", [
     (45, dict(coarse_size=512, coarse_steps=16)),  # dense coarsest level
