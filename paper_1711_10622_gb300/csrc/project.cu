@@ -342,7 +342,8 @@ __device__ __forceinline__ void split_states(const double (&u)[VEC], float (&h)[
 
 // The divergence with split-float products (box_acc2), marching along y: five face values are read and converted per
 // cell, the sixth is the previous line's. Bound by issue (about 110 instructions per cell and state) and, beside it,
-// HBM. Lines per thread on the 128^3 channel, m = 8: 1 181 us, 2 154, 4 137, 8 130.
+// HBM. Lines per thread on the 128^3 channel, m = 8: 1 181 us, 2 154, 4 137, 8 130. With two states per thread it spills
+// 28 bytes at its 64 registers and is still 0.58-0.67 times k_divergence_split's time there (m = 2, 6, 10).
 constexpr int kDivMarch = 8;
 template <int VEC, int MARCH>
 __global__ void __launch_bounds__(256, VEC == 4 ? 2 : 4)
@@ -459,14 +460,15 @@ __global__ void __launch_bounds__(256, VEC == 4 ? 2 : 4)
   }
 }
 
-// The correction, one line per block: a difference and an update per face and state, six FP64 operations on a pipe of
-// two per clock and SM, and 0.75 more for the coefficients with four states per thread (186 us for 128^3 cells, m = 8;
+// The correction, one line per block and four states per thread: a difference and an update per face and state, six FP64
+// operations on a pipe of two per clock and SM, and 0.75 more for the coefficients (186 us for 128^3 cells, m = 8;
 // measured 209, 220 with the index divisions of k_grad_correct). Slower: coefficients shared by the block (226: a
 // barrier before the first load), marching along y as the divergence does (345: the next line's loads wait for
-// this line's stores).
-template <int VEC>
+// this line's stores), one or two states per thread (128^3, m = 1 75 us, 2 115, 6 307, 7 426 against 60, 80, 224, 344
+// of k_grad_correct, which takes these widths).
 __global__ void __launch_bounds__(256)
     k_grad_correct_lines(GridView g, int32_t m, double tau, const double *__restrict__ P, double *U, double *V, double *W) {
+  constexpr int VEC = 4;
   const March p = march_place<VEC, 1>(g, m);
   const int32_t nx = g.N[0], ny = g.N[1], nz = g.N[2], y = p.y0;
   if (!p.on) return;
@@ -526,19 +528,26 @@ MarchLaunch march_launch(const ens_grid *G, int m) {
   const int64_t blocks = (width + threads - 1) / threads * ((G->N[1] + MARCH - 1) / MARCH) * G->N[2];
   return MarchLaunch{threads, width <= INT32_MAX && blocks <= INT32_MAX ? blocks : 0};
 }
-// Both return false (nothing launched) where the grid is too large for one launch.
+// Both return false (nothing launched) where the general kernel runs: a grid too large for one launch, or (the
+// divergence) one whose lines of kDivMarch cells are too few for the chip. A thread's cells follow one another, so the
+// launch pays only while its waves of resident threads (by the kernels' registers) are mostly full: against the general
+// kernel, fill 0.14-0.47 with four states per thread 1.02-1.3 times its time (24^3 cells, m = 8 25 us against 20), 0.63
+// 0.95-1.02, 0.71 0.95, 0.84 0.84, 0.96 0.81; with two states per thread 0.1-0.2 1.1-1.2, 0.3 0.96, 0.6 0.8.
 template <int VEC>
 bool divergence_march(const ens_grid *G, const GridView &g, int m, double scale, const double *U, const double *V, const double *W, double *D,
                       cudaStream_t s) {
+  constexpr int64_t kRoom = VEC == 4 ? 512 : 1024;
+  constexpr double kFill = VEC == 4 ? 0.65 : 0.3;
   const MarchLaunch l = march_launch<VEC, kDivMarch>(G, m);
+  const int64_t wave = G->num_sms * (kRoom / l.threads), waves = (l.blocks + wave - 1) / wave;
+  if ((double)l.blocks * l.threads < kFill * (double)(waves * G->num_sms * kRoom)) return false;
   if (l.blocks > 0) k_divergence_march<VEC, kDivMarch><<<(unsigned)l.blocks, l.threads, 0, s>>>(g, m, scale, U, V, W, D);
   return l.blocks > 0;
 }
-template <int VEC>
 bool grad_correct_lines(const ens_grid *G, const GridView &g, int m, double tau, const double *P, double *U, double *V, double *W,
                         cudaStream_t s) {
-  const MarchLaunch l = march_launch<VEC, 1>(G, m);
-  if (l.blocks > 0) k_grad_correct_lines<VEC><<<(unsigned)l.blocks, l.threads, 0, s>>>(g, m, tau, P, U, V, W);
+  const MarchLaunch l = march_launch<4, 1>(G, m);
+  if (l.blocks > 0) k_grad_correct_lines<<<(unsigned)l.blocks, l.threads, 0, s>>>(g, m, tau, P, U, V, W);
   return l.blocks > 0;
 }
 
@@ -813,9 +822,7 @@ extern "C" ens_status ens_grad_correct(const ens_grid *G, int32_t m, double tau,
   const GridView g = view_of(G);
   cudaStream_t s = (cudaStream_t)stream;
   const int64_t work = (int64_t)G->n * (m / vec);
-  if (G->all_fluid && (vec == 4   ? grad_correct_lines<4>(G, g, m, tau, P, U, V, W, s)
-                       : vec == 2 ? grad_correct_lines<2>(G, g, m, tau, P, U, V, W, s)
-                                  : grad_correct_lines<1>(G, g, m, tau, P, U, V, W, s))) {
+  if (vec == 4 && G->all_fluid && grad_correct_lines(G, g, m, tau, P, U, V, W, s)) {
     ENS_CUDA_TRY(cudaGetLastError());
     return ENS_OK;
   }

@@ -149,6 +149,41 @@ def test_vcycle_small_levels(ens, m, nx, opts):
     _vcycle(ens, _made[nx], m, dict(dict(theta=0.08, max_levels=8), **opts))
 
 
+def _us(f, n=9):
+    """Median time of f() in microseconds, after three untimed calls."""
+    t = []
+    for k in range(n + 3):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        f()
+        b.record()
+        torch.cuda.synchronize()
+        if k > 2:
+            t.append(a.elapsed_time(b) * 1e3)
+    return float(np.median(t))
+
+
+def test_projection_cost(ens):
+    """The correction of one and two states per thread costs what the general kernel takes: m = 2 two thirds of m = 4's
+    time and m = 6 that of m = 8 (by lines 0.95 and 1.37 times); and a small grid's divergence of 32 states (four per
+    thread) at most 1.15 times that of 31 (one per thread; by lines of eight cells 1.4 times)."""
+    op = gen.channel(128, 128, 128)
+    with ens.Grid.from_grid(gen.grid_of(op)) as G:
+        t = {}
+        for m in (2, 4, 6, 8):
+            U, V, W, P = (torch.randn(k, m, dtype=torch.float64, device="cuda") for k in (op.n, op.n // 128 * 129, op.n, op.n))
+            t[m] = _us(lambda: ens.grad_correct(G, P, U, V, W, tau=1e-3))
+    assert t[2] <= 0.8 * t[4] and t[6] <= 1.15 * t[8], t
+    op = gen.dirichlet_box(20)
+    g = gen.grid_of(op)
+    with ens.Grid.from_grid(g) as G:
+        for m in (31, 32):
+            U, V, W = (torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in gen.predictor_velocity(g, m, 3, noise=0.1))
+            D = torch.empty(op.n, m, dtype=torch.float64, device="cuda")
+            t[m] = _us(lambda: [ens.divergence(G, U, V, W, scale=2.0, D=D) for _ in range(20)])
+    assert t[32] <= 1.15 * t[31], t
+
+
 @pytest.mark.parametrize("name", ["dirichlet33x17x9", "channel37x9x11", "channel64x16x8", "channel3x3x3", "dirichlet1x8x5"])
 @pytest.mark.parametrize("m", [1, 2, 4, 5, 6, 8, 12])
 def test_projection_lines(ens, name, m):
@@ -173,3 +208,21 @@ def test_projection_lines(ens, name, m):
     corr = oracle.grad_correct(g, P, *(np.zeros_like(c) for c in (U, V, W)), 0.013)
     for a, b, c, e in zip(got, ref, (U, V, W), corr):
         assert np.all(np.abs(a - b) <= 1e-14 * (np.abs(b) + np.abs(c) + np.abs(e)))
+
+
+@pytest.mark.parametrize("name,m", [("dirichlet45x61x47", 6), ("dirichlet45x61x47", 12), ("channel67x53x48", 6), ("channel67x53x48", 8),
+                                    ("channel67x53x48", 10)])
+def test_divergence_lines(ens, name, m):
+    """Grids large enough for the divergence by lines of eight cells, with ragged lines and runs; two and four states
+    per thread; boundary faces of every kind; face values outside the split range in some states."""
+    op = gen.dirichlet_box(45, nz=47, ny=61) if name.startswith("dirichlet") else gen.channel(67, 53, 48)
+    g = gen.grid_of(op)
+    U, V, W = (np.ascontiguousarray(a) for a in gen.predictor_velocity(g, m, 100 + m, noise=0.3))
+    W[:, 1] *= 1e-16
+    U[::7, 2] *= 1e30
+    with ens.Grid.from_grid(g) as G:
+        D = ens.divergence(G, *(torch.from_numpy(a).cuda() for a in (U, V, W)), scale=-2.5).cpu().numpy()
+    w = [np.diff(a) for a in g.nodes]
+    area = max(w[0].max() * w[1].max(), w[0].max() * w[2].max(), w[1].max() * w[2].max())
+    bound = 2.5 * 6 * area * np.maximum.reduce([np.abs(c).max(axis=0) for c in (U, V, W)])
+    assert np.all(np.abs(D - oracle.divergence(g, U, V, W, scale=-2.5)) <= 1e-14 * bound)
