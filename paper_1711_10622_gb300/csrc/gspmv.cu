@@ -150,6 +150,39 @@ cudaError_t launch_box_cw(const ens_matrix *A, int m, const void *X, void *Y, cu
     if (p % 16 == 0) return launch_box_acc<T, CW, kWide / 2, false>(A, m, X, Y, s);
   return launch_box_acc<T, CW, 1, false>(A, m, X, Y, s);
 }
+int pow2_at_least(int v, int cap) {
+  int p = 1;
+  while (p < v && p < cap) p <<= 1;
+  return p;
+}
+
+// Whether this product of a width that may take row boxes (use_box) is faster by them than row by row. It is wherever
+// the row-by-row launch leaves lanes without columns; where its lanes are (nearly) full, boxes lose
+//   * with rows that are not 32-byte aligned, whose X then comes in smaller pieces (128^3 channel: float64, rows aligned to
+//     16 bytes, m = 16 284 us against 248, 32 567 against 481, 64 1140 against 903, but 20 0.76, 24 0.87 and 8 0.87 times;
+//     float32, aligned to 8 bytes, m = 14 1.03 (rows of nine entries 0.83), 16 217 against 157, 24 345 against 295, but
+//     12 0.91 and 20 0.90 times;
+//     float32, aligned to 16, m = 16 1.03, 24 1.12);
+//   * in float64 from m = 16 on where the rounds of boxes per resident block take 1.3 times the rows there are (bricks cut
+//     off by the grid, a last round that is nearly empty: 112640 rows in 440 boxes, m = 16 1.04 times, 32 1.10, 64 1.19;
+//     85000 rows in 630 boxes 1.06, 1.10, 1.15; 221184 rows at 1.4 times 1.00; 331776 rows at 1.06 times 0.8-0.9). Not
+//     asked where the autotuner has timed both.
+// float32 blocks of four columns below 2^17 rows take one latency either way, by boxes 17 us against 16.
+bool box_pays(const ens_matrix *A, int m, int dtype, const void *X, const void *Y) {
+  const bool f32 = dtype == ENS_F32;
+  const uint64_t p = (uint64_t)(uintptr_t)X | (uint64_t)(uintptr_t)Y | (uint64_t)m * (f32 ? 4 : 8);
+  const int tile = pow2_at_least(m, 32);  // columns of a row-by-row tile
+  const double full = (double)m / ((m + tile - 1) / tile * tile);
+  const bool timed = m <= kTuneMaxM && A->tuned_lanes[f32 ? 1 : 0][m] > 0;
+  if (f32) {
+    if (m == 4 && A->n < (1 << 17) && !timed) return false;
+    return p % 32 == 0 || p % 8 != 0 || m < (A->box.K == 7 ? 14 : 16) || full < 0.75;
+  }
+  if (m < 16 || m % 4 != 0 || full < 0.875) return true;
+  if (p % 32 != 0 && p % 16 == 0) return false;
+  const int64_t round = A->num_sms * (int64_t)BoxShape<double, 8>::kBlocks, slots = (A->box.boxes + round - 1) / round * round;
+  return timed || p % 16 != 0 || 10 * slots * kBoxRows < 13 * A->n;
+}
 cudaError_t launch_box(const ens_matrix *A, int m, int dtype, const void *X, void *Y, cudaStream_t s) {
   if (dtype == ENS_F32) {
     if (m <= 4) return launch_box_cw<float, 4>(A, m, X, Y, s);
@@ -198,12 +231,6 @@ cudaError_t run(const ens_matrix *A, int m, const void *X, void *Y, uint32_t mas
     k<<<grid_for(A, v.n, resident(known, (const void *)k, kThreads, 0), tile_rows_for(v.n, LANES)), kThreads, 0, s>>>(v, m, (const T *)X, y, mask);
   }
   return cudaGetLastError();
-}
-
-int pow2_at_least(int v, int cap) {
-  int p = 1;
-  while (p < v && p < cap) p <<= 1;
-  return p;
 }
 
 bool aligned(const void *p, size_t a) { return ((uintptr_t)p % a) == 0; }
@@ -355,7 +382,7 @@ __global__ void k_tune_fill(int64_t count, double *x, float *x32) {
 
 ens_status launch_gspmv(const ens_matrix *A, int m, int dtype, const void *X, void *Y, cudaStream_t s) {
   if (A->n == 0) return ENS_OK;
-  cudaError_t e = use_box(A, m, dtype) ? launch_box(A, m, dtype, X, Y, s)
+  cudaError_t e = use_box(A, m, dtype) && box_pays(A, m, dtype, X, Y) ? launch_box(A, m, dtype, X, Y, s)
                                        : launch_cfg(A, m, dtype, X, Y, default_cfg(A, m, dtype, X, Y), Rows{0, A->n}, s);
   if (e != cudaSuccess) return cuda_fail(e, "gspmv launch");
   return ENS_OK;

@@ -152,6 +152,19 @@ def test_small_values_cost(ens, m, most):
         assert _us(lambda: ens.gspmv(A, T, Y)) <= most * _us(lambda: ens.gspmv(A, X, Y))
 
 
+@pytest.mark.parametrize("dims,dt,m,off", [((128, 128, 128), "float32", 16, 2), ((128, 128, 128), "float64", 32, 2), ((64, 40, 44), "float64", 64, 0)])
+def test_not_slower_than_rows(ens, dims, dt, m, off):
+    """Blocks whose rows are aligned to less than the boxes' widest access, and boxes whose last round is nearly empty:
+    the product is the row-by-row one, which a forced traversal also runs (by boxes 1.37, 1.18 and 1.19 times)."""
+    op = gen.channel(*dims)
+    dt = getattr(torch, dt)
+    with ens.Matrix.from_operator(op) as A, ens.Matrix.from_operator(op) as R:
+        R.set_untiled(0)
+        X, Y = (torch.randn(op.n * m + off, dtype=dt, device="cuda")[off:].view(op.n, m) for _ in range(2))
+        t = [_us(lambda: ens.gspmv(M, X, Y), 21) for M in (A, R)]
+    assert t[0] <= 1.1 * t[1], t
+
+
 @pytest.mark.parametrize("dtype", [np.float64, np.float32])
 def test_nonfinite(ens, dtype):
     """Infinities and NaN reach exactly the rows whose entries name them, as in the definition."""
@@ -202,3 +215,17 @@ def test_threads_with_rows_of_different_lengths(ens):
     for t in ts:
         t.join()
     assert not bad
+
+
+@pytest.mark.parametrize("name", ["cubes97x43x37", "channel64x40x44"])
+@pytest.mark.parametrize("dt,m,off", [("float64", 16, 2), ("float64", 28, 0), ("float64", 56, 2), ("float64", 64, 0), ("float32", 4, 0),
+                                      ("float32", 14, 0), ("float32", 16, 2), ("float32", 24, 4), ("float32", 24, 1)])
+def test_products_at_the_line_between_both_forms(ens, name, dt, m, off):
+    """Widths, alignments and sizes on either side of the choice between row boxes and rows."""
+    op = _op(name) if name in OPS else gen.channel(64, 40, 44)
+    dt = getattr(torch, dt)
+    ref = op if dt == torch.float64 else gen.Operator(op.name, op.shape, op.bcs, op.row_ptr, op.col_idx, op.val.astype(np.float32).astype(np.float64), False)
+    X, Y = (torch.randn(op.n * m + off, dtype=dt, device="cuda")[off:].view(op.n, m) for _ in range(2))
+    with ens.Matrix.from_operator(op) as A:
+        ens.gspmv(A, X, Y)
+    _check(ref, X.cpu().numpy(), Y.cpu().numpy(), 1e-12 if dt == torch.float64 else 9 * 2.0**-24)
