@@ -38,6 +38,7 @@ ens_status fail(ens_status st, const char *fmt, ...) {
 
 ens_status cuda_fail(cudaError_t e, const char *what) {
   const ens_status st = (e == cudaErrorMemoryAllocation) ? ENS_ERR_OOM : ENS_ERR_CUDA;
+  (void)cudaGetLastError();  // reported here: the next call's launches must not find it again
   return fail(st, "%s: %s (%s)", what, cudaGetErrorName(e), cudaGetErrorString(e));
 }
 

@@ -1,0 +1,68 @@
+"""Host-side failures of matrix creation and multigrid set-up, without a GPU: the library's objects linked with a fake
+CUDA runtime on host memory (fake_cudart.cpp) whose allocations, or whose operator new, fail on request."""
+
+import glob
+import os
+import subprocess
+import sys
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+SETUP = """
+import ctypes, sys
+sys.path.insert(0, sys.argv[2])
+import gen
+from paper_1711_10622_gb300 import _native as N
+L, fake = N.lib(), ctypes.CDLL(sys.argv[1])
+for f in ("fake_pending", "fake_live", "fake_bytes"):
+    getattr(fake, f).restype = ctypes.c_long
+
+def create(op):
+    A = ctypes.c_void_p()
+    st = L.ens_create_matrix(op.n, op.nnz, op.row_ptr.ctypes.data, op.col_idx.ctypes.data, op.val.ctypes.data, 0, None, ctypes.byref(A))
+    assert (st == N.ENS_OK) == bool(A)
+    return st, A
+
+def destroy(A):
+    assert L.ens_destroy_matrix(A) == N.ENS_OK
+"""
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    from paper_1711_10622_gb300 import build
+
+    build.build()
+    lib = str(tmp_path_factory.mktemp("fake") / "libfake.so")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-fPIC", "-shared", "-Wl,-Bsymbolic", "-o", lib, os.path.join(ROOT, "tests", "fake_cudart.cpp"),
+                    *sorted(glob.glob(os.path.join(build.OBJ_DIR, "*.o"))), "-lpthread"], check=True)
+    return lib
+
+
+def _run(fake, script):
+    """In a process of its own: an exception that leaves the library ends the process."""
+    r = subprocess.run([sys.executable, "-c", SETUP + script, fake, ROOT], capture_output=True, text=True, timeout=300,
+                       env=dict(os.environ, ENSEMBLE_SOLVE_LIB=fake))
+    assert r.returncode == 0, r.stderr[-2000:]
+
+
+def test_create_matrix_without_device_memory(fake):
+    """Each device allocation fails in turn: without its boxes' memory the matrix works, without its own the call ends."""
+    _run(fake, """
+op = gen.dirichlet_box(41)
+seen = []
+for k in range(1, 1000):
+    fake.fake_fail_alloc(ctypes.c_long(k))
+    st, A = create(op)
+    reached = not fake.fake_pending()
+    fake.fake_fail_alloc(ctypes.c_long(0))
+    seen.append(st)
+    if A:
+        destroy(A)
+    assert fake.fake_live() == 0
+    if not reached:
+        break
+assert set(seen) == {N.ENS_OK, N.ENS_ERR_OOM} and seen[0] == N.ENS_ERR_OOM and seen.count(N.ENS_OK) >= 2, seen
+""")
