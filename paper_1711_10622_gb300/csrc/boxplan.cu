@@ -207,7 +207,7 @@ void free_box(BoxPlan &B) {
   B = BoxPlan{};
 }
 
-cudaError_t build_box(ens_matrix *A, const int32_t *rp, const int32_t *ci, cudaStream_t s) {
+static cudaError_t build(ens_matrix *A, const int32_t *rp, const int32_t *ci, cudaStream_t s) {
   const int64_t n = A->n, nnz = A->nnz;
   const int32_t K = A->max_row_len;
   if (n < kBoxMinRows || K < 1 || K > kBoxMaxLen || (double)nnz < 0.75 * (double)K * (double)n) return cudaSuccess;
@@ -278,6 +278,14 @@ cudaError_t build_box(ens_matrix *A, const int32_t *rp, const int32_t *ci, cudaS
     e = cudaSuccess;
   }
   return e;
+}
+
+cudaError_t build_box(ens_matrix *A, const int32_t *rp, const int32_t *ci, cudaStream_t s) {
+  try {
+    return build(A, rp, ci, s);
+  } catch (const std::bad_alloc &) {  // no host memory for it: no plan
+    return cudaSuccess;
+  }
 }
 
 }  // namespace ens

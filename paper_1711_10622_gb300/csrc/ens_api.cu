@@ -8,6 +8,7 @@
 #include <cstdint>
 #include <cstdio>
 #include <cstring>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -154,10 +155,30 @@ ens_status ens_create_matrix(int64_t n, int64_t nnz, const int32_t *row_ptr, con
 
 }  // extern "C"
 
+static ens_status create_matrix_impl(int64_t n, int64_t ncols, int64_t nnz, const int32_t *row_ptr, const int32_t *col_idx,
+                                     const double *val, uint32_t flags, void *stream, ens_matrix *&A);
+
 ens_status ens::create_matrix(int64_t n, int64_t ncols, int64_t nnz, const int32_t *row_ptr, const int32_t *col_idx,
                               const double *val, uint32_t flags, void *stream, ens_matrix **out) {
   if (!out) return fail(ENS_ERR_INVALID, "create_matrix: out is NULL");
   *out = nullptr;
+  ens_matrix *A = nullptr;
+  ens_status st;
+  try {  // nothing may leave a C entry
+    st = create_matrix_impl(n, ncols, nnz, row_ptr, col_idx, val, flags, stream, A);
+  } catch (const std::bad_alloc &) {
+    st = fail(ENS_ERR_OOM, "create_matrix: host allocation failed");
+  }
+  if (st == ENS_OK)
+    *out = A;
+  else if (A)
+    free_matrix(A);
+  return st;
+}
+
+// A: the matrix as far as it was made, also when the call fails.
+static ens_status create_matrix_impl(int64_t n, int64_t ncols, int64_t nnz, const int32_t *row_ptr, const int32_t *col_idx,
+                                     const double *val, uint32_t flags, void *stream, ens_matrix *&A) {
   if (n < 1 || n > INT32_MAX) return fail(ENS_ERR_INVALID, "create_matrix: n = %lld outside [1, 2^31-1]", (long long)n);
   if (ncols < 1 || ncols > INT32_MAX)
     return fail(ENS_ERR_INVALID, "create_matrix: ncols = %lld outside [1, 2^31-1]", (long long)ncols);
@@ -190,7 +211,7 @@ ens_status ens::create_matrix(int64_t n, int64_t ncols, int64_t nnz, const int32
                 (long long)ncols);
 
   cudaStream_t s = (cudaStream_t)stream;
-  ens_matrix *A = new ens_matrix();
+  A = new ens_matrix();
   A->n = n;
   A->ncols = ncols;
   A->nnz = nnz;
@@ -226,17 +247,11 @@ ens_status ens::create_matrix(int64_t n, int64_t ncols, int64_t nnz, const int32
   if (e == cudaSuccess) e = cudaMemcpyAsync(&hflags, dflags, sizeof(unsigned), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   cudaFree(dflags);
-  if (e != cudaSuccess) {
-    free_matrix(A);
-    return cuda_fail(e, "create_matrix");
-  }
+  if (e != cudaSuccess) return cuda_fail(e, "create_matrix");
   A->split_ok = (hflags & 1u) == 0;
   A->full_diag = (hflags & 2u) == 0;
   e = build_box(A, row_ptr, col_idx, s);
-  if (e != cudaSuccess) {
-    free_matrix(A);
-    return cuda_fail(e, "create_matrix: row boxes");
-  }
+  if (e != cudaSuccess) return cuda_fail(e, "create_matrix: row boxes");
   // Row chunks of the pipelined host-buffer product: up to kPipeChunks chunks of whole tiles, each
   // with the set of X row blocks its column indices reach.
   {
@@ -259,7 +274,6 @@ ens_status ens::create_matrix(int64_t n, int64_t ncols, int64_t nnz, const int32
     });
     A->pipe_row.push_back(n);
   }
-  *out = A;
   return ENS_OK;
 }
 

@@ -48,6 +48,27 @@ def _run(fake, script):
     assert r.returncode == 0, r.stderr[-2000:]
 
 
+def test_create_matrix_without_host_memory(fake):
+    """Each host allocation of the call fails in turn: the call returns a matrix or ENS_ERR_OOM and keeps nothing."""
+    _run(fake, """
+op = gen.dirichlet_box(41)  # large enough for row boxes
+seen = set()
+for k in range(1, 100000):
+    fake.fake_fail_new(ctypes.c_long(k))
+    st, A = create(op)
+    reached = not fake.fake_pending()
+    fake.fake_fail_new(ctypes.c_long(0))
+    assert st in (N.ENS_OK, N.ENS_ERR_OOM), st
+    seen.add(st)
+    if A:
+        destroy(A)
+    assert fake.fake_live() == 0
+    if not reached:
+        break
+assert N.ENS_OK in seen and k > 20
+""")
+
+
 def test_create_matrix_without_device_memory(fake):
     """Each device allocation fails in turn: without its boxes' memory the matrix works, without its own the call ends."""
     _run(fake, """
