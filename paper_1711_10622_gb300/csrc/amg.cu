@@ -126,7 +126,7 @@ cudaError_t upload(T **dst, const std::vector<T> &src, cudaStream_t s) {
   return cudaMemcpyAsync(*dst, src.data(), src.size() * sizeof(T), cudaMemcpyHostToDevice, s);
 }
 
-// The coarsest level's updates as a dense matrix, where the level is small and has its diagonal.
+// The coarsest level's updates as a dense matrix, where the level is small, has its diagonal and there is memory for it.
 cudaError_t dense_coarsest(ens_amg *H, cudaStream_t s) {
   const ens_matrix *A = H->lev.back().A;
   const ens_amg_opts &o = H->opts;
@@ -151,6 +151,14 @@ cudaError_t dense_coarsest(ens_amg *H, cudaStream_t s) {
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // dk and k are used until here
   cudaFree(dk);
+  if (e == cudaErrorMemoryAllocation) {  // the cycle makes the updates one by one
+    (void)cudaGetLastError();
+    cudaFree(H->dense);
+    cudaFree(H->dense32);
+    H->dense = nullptr;
+    H->dense32 = nullptr;
+    e = cudaSuccess;
+  }
   return e;
 }
 

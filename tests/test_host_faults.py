@@ -87,3 +87,26 @@ for k in range(1, 1000):
         break
 assert set(seen) == {N.ENS_OK, N.ENS_ERR_OOM} and seen[0] == N.ENS_ERR_OOM and seen.count(N.ENS_OK) >= 2, seen
 """)
+
+
+def test_amg_setup_without_device_memory(fake):
+    """The coarsest level's dense matrix (the last three allocations of the set-up) is left out where it does not fit;
+    every other failed allocation ends the call with the matrix as it was."""
+    _run(fake, """
+op = gen.dirichlet_box(16)
+seen = []
+for k in range(1, 1000):
+    st, A = create(op)
+    held = fake.fake_live()
+    fake.fake_fail_alloc(ctypes.c_long(k))
+    st = L.ens_amg_setup(A, None, None)
+    reached = not fake.fake_pending()
+    fake.fake_fail_alloc(ctypes.c_long(0))
+    assert st == N.ENS_OK or (st == N.ENS_ERR_OOM and fake.fake_live() == held), st
+    destroy(A)
+    assert fake.fake_live() == 0
+    if not reached:
+        break
+    seen.append(st)
+assert seen[-3:] == [N.ENS_OK] * 3 and seen.count(N.ENS_ERR_OOM) >= 10, seen
+""")
