@@ -13,6 +13,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
+#include <memory>
 #include <new>
 #include <thread>
 #include <unordered_map>
@@ -51,21 +52,19 @@ struct Part {  // boxes of one range of rows, in the layout of BoxPlan
   int64_t ucols = 0;
 };
 
-// Columns of the box that is being filled -> position, by open addressing; cleared by a new stamp.
+// Columns of the box that is being filled -> position in the order of their first entry, by open addressing; cleared
+// by a new stamp.
 struct ColumnSet {
   static constexpr int kSize = 4096;
   std::vector<int32_t> key, pos, stamp;
-  int32_t now = 0, count = 0;
+  int32_t now = 0;
   ColumnSet() : key(kSize), pos(kSize), stamp(kSize, 0) {}
-  void clear() { ++now, count = 0; }
-  // Position of c, or -1 if it is not there; `at` is where it goes.
-  int32_t find(int32_t c, uint32_t &at) const {
-    at = ((uint32_t)c * 2654435761u) >> 20;
-    while (stamp[at] == now) {
-      if (key[at] == c) return pos[at];
-      at = (at + 1) & (kSize - 1);
-    }
-    return -1;
+  void clear() { ++now; }
+  // Slot of c, or the free one where it goes.
+  uint32_t slot(int32_t c) const {
+    uint32_t at = ((uint32_t)c * 2654435761u) >> 20;
+    while (stamp[at] == now && key[at] != c) at = (at + 1) & (kSize - 1);
+    return at;
   }
 };
 
@@ -91,9 +90,13 @@ void build_part(int64_t r0, int64_t r1, const int32_t *rp, const int32_t *ci, in
     }
     return step(base, d);
   };
-  std::vector<int32_t> rows, cols;
+  std::vector<int32_t> rows, cols, order, place;
+  std::vector<uint16_t> pos;  // of every entry of the box's rows: its column's position in `cols`
   rows.reserve(kBoxRows);
   cols.reserve(kBoxCols);
+  order.reserve(kBoxCols);
+  place.reserve(kBoxCols);
+  pos.reserve((size_t)kBoxRows * K);
   const size_t guess = (size_t)(n / 224 + 16);
   P.rows.reserve(guess * kBoxRows);
   P.cols.reserve(guess * kBoxCols);
@@ -106,21 +109,27 @@ void build_part(int64_t r0, int64_t r1, const int32_t *rp, const int32_t *ci, in
     }
     rows.clear();
     cols.clear();
+    pos.clear();
     cs.clear();
-    // a row joins when the box has room for it and for its new columns
+    // a row joins when the box has room for it and for its new columns; one that does not fit closes the box
     auto take = [&](int64_t i) -> bool {
       if ((int)rows.size() == kBoxRows) return false;
-      int32_t fresh = 0;
-      uint32_t at;
-      for (int32_t j = rp[i]; j < rp[i + 1]; ++j) fresh += cs.find(ci[j], at) < 0;
-      if (cs.count + fresh > kBoxCols) return false;
-      for (int32_t j = rp[i]; j < rp[i + 1]; ++j)
-        if (cs.find(ci[j], at) < 0) {
+      const size_t ncols = cols.size(), nent = pos.size();
+      for (int32_t j = rp[i]; j < rp[i + 1]; ++j) {
+        const uint32_t at = cs.slot(ci[j]);
+        if (cs.stamp[at] != cs.now) {
+          if ((int)cols.size() == kBoxCols) {  // (the set still names this row's columns: nothing joins any more)
+            cols.resize(ncols);
+            pos.resize(nent);
+            return false;
+          }
           cs.stamp[at] = cs.now;
           cs.key[at] = ci[j];
-          cs.pos[at] = cs.count++;
+          cs.pos[at] = (int32_t)cols.size();
           cols.push_back(ci[j]);
         }
+        pos.push_back((uint16_t)cs.pos[at]);
+      }
       rows.push_back((int32_t)i);
       used[i - r0] = 1;
       return true;
@@ -147,86 +156,82 @@ void build_part(int64_t r0, int64_t r1, const int32_t *rp, const int32_t *ci, in
     }
     // Columns in ascending order: neighbouring rows of the box then read neighbouring X rows, staged from
     // whole lines of memory and read from shared memory without bank conflicts.
-    std::sort(cols.begin(), cols.end());
-    cs.clear();
-    for (int32_t c : cols) {
-      uint32_t at;
-      cs.find(c, at);
-      cs.stamp[at] = cs.now;
-      cs.key[at] = c;
-      cs.pos[at] = cs.count++;
-    }
+    const int32_t nc = (int32_t)cols.size();
+    order.resize(nc);
+    place.resize(nc);
+    for (int32_t k = 0; k < nc; ++k) order[k] = k;
+    std::sort(order.begin(), order.end(), [&](int32_t a, int32_t b) { return cols[a] < cols[b]; });
+    for (int32_t k = 0; k < nc; ++k) place[order[k]] = k;
     const size_t l0 = P.loc.size();
     P.loc.resize(l0 + (size_t)kBoxRows * K, (uint16_t)kBoxCols);  // missing entries: the row of zeros
-    for (size_t r = 0; r < rows.size(); ++r) {
-      const int64_t i = rows[r];
-      uint32_t at;
-      for (int32_t j = rp[i]; j < rp[i + 1]; ++j) P.loc[l0 + (size_t)(j - rp[i]) * kBoxRows + r] = (uint16_t)cs.find(ci[j], at);
-    }
-    P.cnt.push_back(make_int2((int32_t)rows.size(), (int32_t)cols.size()));
-    P.ucols += (int64_t)cols.size();
+    size_t e = 0;
+    for (size_t r = 0; r < rows.size(); ++r)
+      for (int32_t k = 0, len = rp[rows[r] + 1] - rp[rows[r]]; k < len; ++k) P.loc[l0 + (size_t)k * kBoxRows + r] = (uint16_t)place[pos[e++]];
+    const size_t c0 = P.cols.size();
+    P.cols.resize(c0 + kBoxCols, 0);
+    for (int32_t k = 0; k < nc; ++k) P.cols[c0 + k] = cols[order[k]];
+    P.cnt.push_back(make_int2((int32_t)rows.size(), nc));
+    P.ucols += nc;
     rows.resize(kBoxRows, -1);
-    cols.resize(kBoxCols, 0);
     P.rows.insert(P.rows.end(), rows.begin(), rows.end());
-    P.cols.insert(P.cols.end(), cols.begin(), cols.end());
   }
 }
 
 // Values of every box slot from the CSR arrays (0 in the padding): split pairs and float32.
 __global__ void k_box_values(int32_t boxes, int32_t K, const int32_t *__restrict__ brow, const int2 *__restrict__ bcnt,
-                             const int32_t *__restrict__ rp, const float2 *__restrict__ vs, const float *__restrict__ v32,
-                             float2 *__restrict__ bvs, float *__restrict__ bv32) {
+                             const int32_t *__restrict__ rp, const double *__restrict__ va, float2 *__restrict__ bvs,
+                             float *__restrict__ bv32) {
   const int64_t total = (int64_t)boxes * K * kBoxRows;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
     const int32_t r = (int32_t)(e % kBoxRows);
     const int64_t q = e / kBoxRows;
     const int32_t k = (int32_t)(q % K), b = (int32_t)(q / K);
-    float2 v = make_float2(0.f, 0.f);
-    float f = 0.f;
+    double v = 0.0;
     if (r < bcnt[b].x) {
       const int32_t i = brow[(int64_t)b * kBoxRows + r], j = rp[i] + k;
-      if (j < rp[i + 1]) {
-        v = vs[j];
-        f = v32[j];
-      }
+      if (j < rp[i + 1]) v = va[j];
     }
-    bvs[e] = v;
-    bv32[e] = f;
+    const float hi = (float)v;
+    bvs[e] = make_float2(hi, (float)(v - (double)hi));
+    bv32[e] = hi;
   }
 }
 
 }  // namespace
 
+struct HostBoxes {
+  std::vector<Part> part;
+  int64_t boxes = 0;
+};
+
+void free_plan(HostBoxes *h) { delete h; }
+
 void free_box(BoxPlan &B) {
-  cudaFree(B.row);
-  cudaFree(B.cnt);
-  cudaFree(B.col);
-  cudaFree(B.loc);
-  cudaFree(B.vs);
-  cudaFree(B.v32);
+  cudaFree(B.shape);
+  cudaFree(B.values);
   B = BoxPlan{};
 }
 
-static cudaError_t build(ens_matrix *A, const int32_t *rp, const int32_t *ci, cudaStream_t s) {
-  const int64_t n = A->n, nnz = A->nnz;
-  const int32_t K = A->max_row_len;
-  if (n < kBoxMinRows || K < 1 || K > kBoxMaxLen || (double)nnz < 0.75 * (double)K * (double)n) return cudaSuccess;
+namespace {
+
+HostBoxes *plan(int64_t n, int64_t nnz, int32_t K, const int32_t *rp, const int32_t *ci) {
+  if (n < kBoxMinRows || K < 1 || K > kBoxMaxLen || (double)nnz < 0.75 * (double)K * (double)n) return nullptr;
   int64_t s1 = 0, s2 = 0;
   common_steps(n, rp, ci, s1, s2);
   const int64_t per_min = 1 << 13;
   const int parts = (int)std::max<int64_t>(1, std::min<int64_t>({(int64_t)std::max(1u, std::thread::hardware_concurrency()), 16, n / per_min}));
-  std::vector<Part> part(parts);
+  std::unique_ptr<HostBoxes> h(new HostBoxes);
+  h->part.resize(parts);
   // ranges end on whole bricks of planes where the planes are known
   const int64_t unit = s2 ? s2 * kBoxLinesZ : kBoxRows;
   auto bound = [&](int p) { return p == parts ? n : std::min(n, (n * p / parts + unit / 2) / unit * unit); };
-  bool memory = true;
+  std::vector<uint8_t> failed(parts, 0);
   {
     std::vector<std::thread> th;
-    std::vector<uint8_t> failed(parts, 0);
     auto work = [&](int p) {
       try {
-        build_part(bound(p), bound(p + 1), rp, ci, K, s1, s2, part[p]);
-      } catch (const std::bad_alloc &) {
+        build_part(bound(p), bound(p + 1), rp, ci, K, s1, s2, h->part[p]);
+      } catch (...) {
         failed[p] = 1;
       }
     };
@@ -239,53 +244,74 @@ static cudaError_t build(ens_matrix *A, const int32_t *rp, const int32_t *ci, cu
     work(0);
     for (int p = started; p < parts; ++p) work(p);
     for (auto &t : th) t.join();
-    for (uint8_t f : failed) memory = memory && !f;
   }
-  if (!memory) return cudaSuccess;  // no plan
-  int64_t boxes = 0, ucols = 0;
-  for (auto &p : part) boxes += (int64_t)p.cnt.size(), ucols += p.ucols;
-  if (ucols > (int64_t)(0.45 * (double)nnz) || boxes * kBoxRows > n + n / 4 * 3 + 64 * kBoxRows) return cudaSuccess;
+  for (uint8_t f : failed)
+    if (f) return nullptr;
+  int64_t ucols = 0;
+  for (auto &p : h->part) h->boxes += (int64_t)p.cnt.size(), ucols += p.ucols;
+  if (ucols > (int64_t)(0.45 * (double)nnz) || h->boxes * kBoxRows > n + n / 4 * 3 + 64 * kBoxRows) return nullptr;
+  return h.release();
+}
+
+}  // namespace
+
+HostBoxes *plan_boxes(int64_t n, int64_t nnz, int32_t K, const int32_t *rp, const int32_t *ci) {
+  try {
+    return plan(n, nnz, K, rp, ci);
+  } catch (...) {  // no memory for it
+    return nullptr;
+  }
+}
+
+cudaError_t upload_boxes(ens_matrix *A, const HostBoxes *h, cudaStream_t s) {
   BoxPlan &B = A->box;
-  B.boxes = (int32_t)boxes;
-  B.K = K;
-  const size_t slots = (size_t)boxes * K * kBoxRows;
-  cudaError_t e = cudaMalloc((void **)&B.row, (size_t)boxes * kBoxRows * sizeof(int32_t));
-  if (e == cudaSuccess) e = cudaMalloc((void **)&B.col, (size_t)boxes * kBoxCols * sizeof(int32_t));
-  if (e == cudaSuccess) e = cudaMalloc((void **)&B.cnt, (size_t)boxes * sizeof(int2));
-  if (e == cudaSuccess) e = cudaMalloc((void **)&B.loc, slots * sizeof(uint16_t));
-  size_t at = 0;  // boxes of the parts before
-  for (auto &p : part) {
-    auto put = [&](auto *dst, const auto &src, size_t per_box) {
-      if (e == cudaSuccess && !src.empty())
-        e = cudaMemcpyAsync(dst + at * per_box, src.data(), src.size() * sizeof(src[0]), cudaMemcpyHostToDevice, s);
-    };
-    put(B.row, p.rows, kBoxRows);
-    put(B.col, p.cols, kBoxCols);
-    put(B.cnt, p.cnt, 1);
-    put(B.loc, p.loc, (size_t)kBoxRows * K);
-    at += p.cnt.size();
+  cudaError_t e = cudaSuccess;
+  {
+    B.boxes = (int32_t)h->boxes;
+    B.K = A->max_row_len;
+    const size_t boxes = (size_t)B.boxes, slots = boxes * B.K * kBoxRows;
+    const size_t row = boxes * kBoxRows * sizeof(int32_t), col = boxes * kBoxCols * sizeof(int32_t), loc = slots * sizeof(uint16_t);
+    char *p = nullptr;  // one block; every array's size is a multiple of 16 bytes
+    e = cudaMalloc((void **)&p, row + col + loc + boxes * sizeof(int2));
+    B.shape = p;
+    B.row = (int32_t *)p;
+    B.col = (int32_t *)(p + row);
+    B.loc = (uint16_t *)(p + row + col);
+    B.cnt = (int2 *)(p + row + col + loc);
+    size_t at = 0;  // boxes of the parts before
+    for (auto &part : h->part) {
+      auto put = [&](auto *dst, const auto &src, size_t per_box) {
+        if (e == cudaSuccess && !src.empty())
+          e = cudaMemcpyAsync(dst + at * per_box, src.data(), src.size() * sizeof(src[0]), cudaMemcpyHostToDevice, s);
+      };
+      put(B.row, part.rows, kBoxRows);
+      put(B.col, part.cols, kBoxCols);
+      put(B.cnt, part.cnt, 1);
+      put(B.loc, part.loc, (size_t)kBoxRows * B.K);
+      at += part.cnt.size();
+    }
   }
-  if (e == cudaSuccess) e = cudaMalloc((void **)&B.vs, slots * sizeof(float2));
-  if (e == cudaSuccess) e = cudaMalloc((void **)&B.v32, slots * sizeof(float));
   if (e == cudaSuccess) {
-    k_box_values<<<A->num_sms * 8, 256, 0, s>>>(B.boxes, K, B.row, B.cnt, A->row, A->valsplit, A->val32, B.vs, B.v32);
+    const size_t slots = (size_t)B.boxes * B.K * kBoxRows;
+    char *p = nullptr;
+    e = cudaMalloc((void **)&p, slots * (sizeof(float2) + sizeof(float)));
+    B.values = p;
+    B.vs = (float2 *)p;
+    B.v32 = (float *)(p + slots * sizeof(float2));
+  }
+  if (e == cudaSuccess) {
+    k_box_values<<<A->num_sms * 8, 256, 0, s>>>(B.boxes, B.K, B.row, B.cnt, A->row, A->val, B.vs, B.v32);
     e = cudaGetLastError();
   }
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess) free_box(B);
-  if (e == cudaErrorMemoryAllocation) {  // the matrix works without a plan
+  if (e != cudaSuccess) {
+    cudaStreamSynchronize(s);  // copies from the plan in flight
+    free_box(B);
+  }
+  if (e == cudaErrorMemoryAllocation) {  // the matrix works without boxes
     cudaGetLastError();
     e = cudaSuccess;
   }
   return e;
-}
-
-cudaError_t build_box(ens_matrix *A, const int32_t *rp, const int32_t *ci, cudaStream_t s) {
-  try {
-    return build(A, rp, ci, s);
-  } catch (const std::bad_alloc &) {  // no host memory for it: no plan
-    return cudaSuccess;
-  }
 }
 
 }  // namespace ens

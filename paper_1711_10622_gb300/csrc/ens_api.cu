@@ -10,8 +10,10 @@
 #include <cstring>
 #include <new>
 #include <string>
+#include <thread>
 #include <vector>
 
+#include "boxprod.cuh"
 #include "ens_internal.cuh"
 #include "rowprod.cuh"
 
@@ -217,41 +219,25 @@ static ens_status create_matrix_impl(int64_t n, int64_t ncols, int64_t nnz, cons
   A->nnz = nnz;
   A->max_row_len = max_len;
   A->flags = flags;
-  cudaError_t e = cudaGetDevice(&A->device);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&A->num_sms, cudaDevAttrMultiProcessorCount, A->device);
-  unsigned *dflags = nullptr;
-  // CSR arrays carry kCsrPad zeroed elements at the end: tiles stage 16-byte rounded segments.
-  if (e == cudaSuccess) e = dmalloc(&A->row, n + 1 + kCsrPad);
-  if (e == cudaSuccess) e = dmalloc(&A->col, nnz + kCsrPad);
-  if (e == cudaSuccess) e = dmalloc(&A->val, nnz + kCsrPad);
-  if (e == cudaSuccess) e = dmalloc(&A->val32, nnz + kCsrPad);
-  if (e == cudaSuccess) e = dmalloc(&A->valsplit, nnz + kCsrPad);
-  if (e == cudaSuccess) e = cudaMemsetAsync(A->row + n + 1, 0, kCsrPad * sizeof(int32_t), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(A->col + nnz, 0, kCsrPad * sizeof(int32_t), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(A->val + nnz, 0, kCsrPad * sizeof(double), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(A->val32 + nnz, 0, kCsrPad * sizeof(float), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(A->valsplit + nnz, 0, kCsrPad * sizeof(float2), s);
-  if (e == cudaSuccess) e = dmalloc(&A->dinv, n);
-  if (e == cudaSuccess) e = dmalloc(&A->dinv32, n);
-  if (e == cudaSuccess) e = dmalloc(&dflags, 1);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(A->row, row_ptr, (n + 1) * sizeof(int32_t), cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess && nnz) e = cudaMemcpyAsync(A->col, col_idx, nnz * sizeof(int32_t), cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess && nnz) e = cudaMemcpyAsync(A->val, val, nnz * sizeof(double), cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(dflags, 0, sizeof(unsigned), s);
-  if (e == cudaSuccess) {
-    const int grid = (int)std::min<int64_t>((n + 255) / 256, (int64_t)A->num_sms * 8);
-    k_matrix_aux<<<grid, 256, 0, s>>>((int32_t)n, A->row, A->col, A->val, A->val32, A->valsplit, A->dinv, A->dinv32, dflags);
-    e = cudaGetLastError();
+  // The row boxes are planned on threads of their own while the masks below are formed and the arrays go to the device:
+  // one after the other, operators of 65536 to 200000 rows took 1.8 to 1.9 times as long to create as without boxes.
+  struct Planner {
+    std::thread thread;
+    HostBoxes *plan = nullptr;
+    ~Planner() {
+      if (thread.joinable()) thread.join();
+      free_plan(plan);
+    }
+  } planner;
+  auto make_plan = [&] { planner.plan = plan_boxes(n, nnz, max_len, row_ptr, col_idx); };
+  bool planned = n < kBoxMinRows;
+  if (!planned) {
+    try {
+      planner.thread = std::thread(make_plan);
+      planned = true;
+    } catch (...) {  // no thread: planned below
+    }
   }
-  unsigned hflags = 0;
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&hflags, dflags, sizeof(unsigned), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  cudaFree(dflags);
-  if (e != cudaSuccess) return cuda_fail(e, "create_matrix");
-  A->split_ok = (hflags & 1u) == 0;
-  A->full_diag = (hflags & 2u) == 0;
-  e = build_box(A, row_ptr, col_idx, s);
-  if (e != cudaSuccess) return cuda_fail(e, "create_matrix: row boxes");
   // Row chunks of the pipelined host-buffer product: up to kPipeChunks chunks of whole tiles, each
   // with the set of X row blocks its column indices reach.
   {
@@ -274,6 +260,42 @@ static ens_status create_matrix_impl(int64_t n, int64_t ncols, int64_t nnz, cons
     });
     A->pipe_row.push_back(n);
   }
+  cudaError_t e = cudaGetDevice(&A->device);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&A->num_sms, cudaDevAttrMultiProcessorCount, A->device);
+  unsigned *dflags = nullptr;
+  // CSR arrays carry kCsrPad zeroed elements at the end: tiles stage 16-byte rounded segments.
+  if (e == cudaSuccess) e = dmalloc(&A->row, n + 1 + kCsrPad);
+  if (e == cudaSuccess) e = dmalloc(&A->col, nnz + kCsrPad);
+  if (e == cudaSuccess) e = dmalloc(&A->val, nnz + kCsrPad);
+  if (e == cudaSuccess) e = dmalloc(&A->val32, nnz + kCsrPad);
+  if (e == cudaSuccess) e = dmalloc(&A->valsplit, nnz + kCsrPad);
+  if (e == cudaSuccess) e = cudaMemsetAsync(A->row + n + 1, 0, kCsrPad * sizeof(int32_t), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(A->col + nnz, 0, kCsrPad * sizeof(int32_t), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(A->val + nnz, 0, kCsrPad * sizeof(double), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(A->val32 + nnz, 0, kCsrPad * sizeof(float), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(A->valsplit + nnz, 0, kCsrPad * sizeof(float2), s);
+  if (e == cudaSuccess) e = dmalloc(&A->dinv, n);
+  if (e == cudaSuccess) e = dmalloc(&A->dinv32, n);
+  if (e == cudaSuccess) e = dmalloc(&dflags, 1);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(A->row, row_ptr, (n + 1) * sizeof(int32_t), cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess && nnz) e = cudaMemcpyAsync(A->col, col_idx, nnz * sizeof(int32_t), cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess && nnz) e = cudaMemcpyAsync(A->val, val, nnz * sizeof(double), cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(dflags, 0, sizeof(unsigned), s);
+  if (planner.thread.joinable()) planner.thread.join();
+  if (!planned && e == cudaSuccess) make_plan();
+  if (e == cudaSuccess && planner.plan) e = upload_boxes(A, planner.plan, s);
+  if (e == cudaSuccess) {
+    const int grid = (int)std::min<int64_t>((n + 255) / 256, (int64_t)A->num_sms * 8);
+    k_matrix_aux<<<grid, 256, 0, s>>>((int32_t)n, A->row, A->col, A->val, A->val32, A->valsplit, A->dinv, A->dinv32, dflags);
+    e = cudaGetLastError();
+  }
+  unsigned hflags = 0;
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&hflags, dflags, sizeof(unsigned), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  cudaFree(dflags);
+  if (e != cudaSuccess) return cuda_fail(e, "create_matrix");
+  A->split_ok = (hflags & 1u) == 0;
+  A->full_diag = (hflags & 2u) == 0;
   return ENS_OK;
 }
 

@@ -132,8 +132,13 @@ ens_status fail(ens_status st, const char *fmt, ...);
 ens_status cuda_fail(cudaError_t e, const char *what);
 void clear_error();
 
-// Row boxes of A from its host CSR arrays (A->box stays empty where boxes do not pay or memory is short).
-cudaError_t build_box(ens_matrix *A, const int32_t *row_ptr, const int32_t *col_idx, cudaStream_t s);
+// Row boxes of a matrix, planned on the host from its CSR arrays (nullptr where boxes do not pay or memory is short).
+struct HostBoxes;
+HostBoxes *plan_boxes(int64_t n, int64_t nnz, int32_t max_row_len, const int32_t *row_ptr, const int32_t *col_idx);
+void free_plan(HostBoxes *h);
+// A->box from a plan; A->row and A->val are on the device by then. A->box stays empty where device memory is short. h may
+// be freed once stream s is through.
+cudaError_t upload_boxes(ens_matrix *A, const HostBoxes *h, cudaStream_t s);
 void free_box(BoxPlan &B);
 // Whether products of width m use A's row boxes: one exists, the width gains by it and no row-by-row
 // arithmetic or traversal was asked for.

@@ -32,6 +32,7 @@ struct BoxPlan {
   uint16_t *loc = nullptr;
   float2 *vs = nullptr;
   float *v32 = nullptr;
+  void *shape = nullptr, *values = nullptr;  // the blocks the arrays lie in: row, col, loc and cnt; vs and v32
 };
 
 template <typename T, int VEC>
