@@ -257,7 +257,7 @@ static ens_status amg_setup_impl(ens_matrix *A, const ens_amg_opts *opts, void *
           if (L.col[k] == i && L.val[k] != 0.0) dinv[i] = 1.0 / L.val[k];
       for (int64_t i = 0; i < L.n; ++i)
         for (int32_t k = L.row[i]; k < L.row[i + 1]; ++k) vs[k] = L.val[k] * dinv[L.col[k]];
-      st = ens_create_matrix(L.n, (int64_t)vs.size(), L.row.data(), L.col.data(), vs.data(), 0, stream, &f.As);
+      st = create_matrix(L.n, L.n, (int64_t)vs.size(), L.row.data(), L.col.data(), vs.data(), 0, stream, &f.As, f.A);
       if (st != ENS_OK) {
         free_amg(H);
         return st;

@@ -263,10 +263,13 @@ HostBoxes *plan_boxes(int64_t n, int64_t nnz, int32_t K, const int32_t *rp, cons
   }
 }
 
-cudaError_t upload_boxes(ens_matrix *A, const HostBoxes *h, cudaStream_t s) {
+cudaError_t upload_boxes(ens_matrix *A, const HostBoxes *h, const BoxPlan *shape, cudaStream_t s) {
   BoxPlan &B = A->box;
   cudaError_t e = cudaSuccess;
-  {
+  if (shape) {
+    B = *shape;
+    B.shape = B.values = nullptr;  // the shape stays with its owner
+  } else {
     B.boxes = (int32_t)h->boxes;
     B.K = A->max_row_len;
     const size_t boxes = (size_t)B.boxes, slots = boxes * B.K * kBoxRows;

@@ -158,16 +158,16 @@ ens_status ens_create_matrix(int64_t n, int64_t nnz, const int32_t *row_ptr, con
 }  // extern "C"
 
 static ens_status create_matrix_impl(int64_t n, int64_t ncols, int64_t nnz, const int32_t *row_ptr, const int32_t *col_idx,
-                                     const double *val, uint32_t flags, void *stream, ens_matrix *&A);
+                                     const double *val, uint32_t flags, void *stream, ens_matrix *&A, const ens_matrix *like);
 
 ens_status ens::create_matrix(int64_t n, int64_t ncols, int64_t nnz, const int32_t *row_ptr, const int32_t *col_idx,
-                              const double *val, uint32_t flags, void *stream, ens_matrix **out) {
+                              const double *val, uint32_t flags, void *stream, ens_matrix **out, const ens_matrix *like) {
   if (!out) return fail(ENS_ERR_INVALID, "create_matrix: out is NULL");
   *out = nullptr;
   ens_matrix *A = nullptr;
   ens_status st;
   try {  // nothing may leave a C entry
-    st = create_matrix_impl(n, ncols, nnz, row_ptr, col_idx, val, flags, stream, A);
+    st = create_matrix_impl(n, ncols, nnz, row_ptr, col_idx, val, flags, stream, A, like);
   } catch (const std::bad_alloc &) {
     st = fail(ENS_ERR_OOM, "create_matrix: host allocation failed");
   }
@@ -180,7 +180,7 @@ ens_status ens::create_matrix(int64_t n, int64_t ncols, int64_t nnz, const int32
 
 // A: the matrix as far as it was made, also when the call fails.
 static ens_status create_matrix_impl(int64_t n, int64_t ncols, int64_t nnz, const int32_t *row_ptr, const int32_t *col_idx,
-                                     const double *val, uint32_t flags, void *stream, ens_matrix *&A) {
+                                     const double *val, uint32_t flags, void *stream, ens_matrix *&A, const ens_matrix *like) {
   if (n < 1 || n > INT32_MAX) return fail(ENS_ERR_INVALID, "create_matrix: n = %lld outside [1, 2^31-1]", (long long)n);
   if (ncols < 1 || ncols > INT32_MAX)
     return fail(ENS_ERR_INVALID, "create_matrix: ncols = %lld outside [1, 2^31-1]", (long long)ncols);
@@ -230,7 +230,7 @@ static ens_status create_matrix_impl(int64_t n, int64_t ncols, int64_t nnz, cons
     }
   } planner;
   auto make_plan = [&] { planner.plan = plan_boxes(n, nnz, max_len, row_ptr, col_idx); };
-  bool planned = n < kBoxMinRows;
+  bool planned = n < kBoxMinRows || like;
   if (!planned) {
     try {
       planner.thread = std::thread(make_plan);
@@ -283,7 +283,8 @@ static ens_status create_matrix_impl(int64_t n, int64_t ncols, int64_t nnz, cons
   if (e == cudaSuccess) e = cudaMemsetAsync(dflags, 0, sizeof(unsigned), s);
   if (planner.thread.joinable()) planner.thread.join();
   if (!planned && e == cudaSuccess) make_plan();
-  if (e == cudaSuccess && planner.plan) e = upload_boxes(A, planner.plan, s);
+  if (e == cudaSuccess && (planner.plan || (like && like->box.boxes > 0)))
+    e = upload_boxes(A, planner.plan, like ? &like->box : nullptr, s);
   if (e == cudaSuccess) {
     const int grid = (int)std::min<int64_t>((n + 255) / 256, (int64_t)A->num_sms * 8);
     k_matrix_aux<<<grid, 256, 0, s>>>((int32_t)n, A->row, A->col, A->val, A->val32, A->valsplit, A->dinv, A->dinv32, dflags);

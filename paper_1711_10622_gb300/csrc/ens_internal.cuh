@@ -117,9 +117,10 @@ cudaMemPool_t scratch_pool(const ens_matrix *A);
 // Release a hierarchy (coarse matrices and maps; not the fine matrix).
 void free_amg(ens_amg *H);
 
-// Create a device matrix of n rows whose column indices lie in [0, ncols) (ncols = n: square).
+// Create a device matrix of n rows whose column indices lie in [0, ncols) (ncols = n: square). like: a matrix with the
+// same rows and columns that will live as long, whose row boxes are used (nullptr: they are planned).
 ens_status create_matrix(int64_t n, int64_t ncols, int64_t nnz, const int32_t *row_ptr, const int32_t *col_idx,
-                         const double *val, uint32_t flags, void *stream, ens_matrix **out);
+                         const double *val, uint32_t flags, void *stream, ens_matrix **out, const ens_matrix *like = nullptr);
 
 // Bytes of scratch the last solve call on this host thread took (or, if its caller-provided
 // workspace was too small, needed up to the failing request), and whether it ran out.
@@ -136,9 +137,10 @@ void clear_error();
 struct HostBoxes;
 HostBoxes *plan_boxes(int64_t n, int64_t nnz, int32_t max_row_len, const int32_t *row_ptr, const int32_t *col_idx);
 void free_plan(HostBoxes *h);
-// A->box from a plan; A->row and A->val are on the device by then. A->box stays empty where device memory is short. h may
-// be freed once stream s is through.
-cudaError_t upload_boxes(ens_matrix *A, const HostBoxes *h, cudaStream_t s);
+// A->box from a plan, or from the boxes `shape` of a matrix with the same rows and columns, which must live as long;
+// A->row and A->val are on the device by then. A->box stays empty where device memory is short. h may be freed once
+// stream s is through.
+cudaError_t upload_boxes(ens_matrix *A, const HostBoxes *h, const BoxPlan *shape, cudaStream_t s);
 void free_box(BoxPlan &B);
 // Whether products of width m use A's row boxes: one exists, the width gains by it and no row-by-row
 // arithmetic or traversal was asked for.

@@ -32,7 +32,9 @@ struct BoxPlan {
   uint16_t *loc = nullptr;
   float2 *vs = nullptr;
   float *v32 = nullptr;
-  void *shape = nullptr, *values = nullptr;  // the blocks the arrays lie in: row, col, loc and cnt; vs and v32
+  // The blocks the arrays lie in: row, col, loc and cnt; vs and v32. shape is nullptr where the boxes of another matrix
+  // with the same rows and columns are used (the column-scaled copy of a multigrid level).
+  void *shape = nullptr, *values = nullptr;
 };
 
 template <typename T, int VEC>

@@ -110,3 +110,33 @@ for k in range(1, 1000):
     seen.append(st)
 assert seen[-3:] == [N.ENS_OK] * 3 and seen.count(N.ENS_ERR_OOM) >= 10, seen
 """)
+
+
+def test_scaled_copy_uses_its_levels_boxes(fake):
+    """The column-scaled copy of a multigrid level takes the row boxes of the level (the same rows and columns) and holds
+    only values of its own."""
+    _run(fake, """
+import numpy as np
+op = gen.dirichlet_box(41)
+b0 = fake.fake_bytes()
+st, A = create(op)
+b1 = fake.fake_bytes()
+o = N.AmgOpts()
+L.ens_default_amg_opts(ctypes.byref(o))
+o.max_levels = 2
+assert L.ens_amg_setup(A, ctypes.byref(o), None) == N.ENS_OK
+b2 = fake.fake_bytes()
+rows, nnz = (ctypes.c_int64 * 16)(), (ctypes.c_int64 * 16)()
+assert L.ens_amg_info(A, None, rows, nnz) == N.ENS_OK and rows[1] > 512
+C = gen.Operator("level", (rows[1], 1, 1), ("x",) * 3, np.empty(rows[1] + 1, np.int32), np.empty(nnz[1], np.int32), np.empty(nnz[1]), False)
+assert L.ens_amg_level(A, 1, C.row_ptr.ctypes.data, C.col_idx.ctypes.data, C.val.ctypes.data, None) == N.ENS_OK
+b3 = fake.fake_bytes()
+st, B = create(C)
+maps = 4 * (op.n + op.n + rows[1] + 1)
+copy = (b2 - b1) - maps - (fake.fake_bytes() - b3)
+shape = op.n // 256 * (256 + 576) * 4  # at least this for rows and columns of the boxes
+assert copy <= (b1 - b0) - shape, (copy, b1 - b0, shape)
+destroy(B)
+destroy(A)
+assert fake.fake_live() == 0
+""")
