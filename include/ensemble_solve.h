@@ -109,7 +109,8 @@ ens_status ens_set_native_share(ens_matrix *A, int32_t share);
  * the matrix has them and m >= 3) and keep the fastest for later
  * ens_gspmv calls and for the solver's products of that width. Uses temporary device blocks of
  * n x m (stream-ordered, freed before return). Synchronous. Optional outputs: chosen lanes, chosen
- * share (32 = native, 64 = column hybrid), and the best time per launch in microseconds. A share
+ * share (32 = native, 64 = column hybrid, 0 = all split, row boxes among it: ens_tuned_variant tells
+ * them apart), and the best time per launch in microseconds. A share
  * set with ens_set_native_share, or ENS_F64_HYBRID / ENS_F64_SPLIT modes, still take priority.
  */
 ens_status ens_autotune(ens_matrix *A, int32_t m, int32_t dtype, void *stream, int32_t *lanes, int32_t *share,
@@ -126,7 +127,9 @@ ens_status ens_set_untiled(ens_matrix *A, int32_t mode);
 /*
  * The launch the autotuner chose for width m and dtype (-1 in every output where it has not run):
  * lanes per row, native share (as ens_autotune reports it) and untiled = 1 when the rows are read
- * straight from global memory instead of through shared-memory row tiles (both forms are timed).
+ * straight from global memory instead of through shared-memory row tiles (both forms are timed), 2 when
+ * the product runs by row boxes (all split, share 0; lanes are then those of the fastest row-by-row
+ * launch, which the row chunks of ens_gspmv_host take).
  */
 ens_status ens_tuned_variant(const ens_matrix *A, int32_t m, int32_t dtype, int32_t *lanes, int32_t *share,
                              int32_t *untiled);

@@ -100,7 +100,7 @@ class Matrix:
         ul = ctypes.c_int32()
         N.check(N.lib().ens_tuned_variant(self.handle, int(m), code, None, None, ctypes.byref(ul)))
         return {"m": int(m), "dtype": dtype, "lanes": lanes.value, "share": share.value, "untiled": bool(ul.value == 1),
-                "best_us": us.value}
+                "boxes": bool(ul.value == 2), "best_us": us.value}
 
     def amg_setup(self, stream=None, **opts):
         """Build the aggregation multigrid hierarchy (ens_amg_setup); keyword overrides of

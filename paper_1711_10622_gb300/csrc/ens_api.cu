@@ -360,9 +360,10 @@ ens_status ens_tuned_variant(const ens_matrix *A, int32_t m, int32_t dtype, int3
   if (m < 1 || m > kTuneMaxM) return fail(ENS_ERR_INVALID, "tuned_variant: m = %d outside [1, %d]", m, kTuneMaxM);
   if (dtype != ENS_F64 && dtype != ENS_F32) return fail(ENS_ERR_INVALID, "tuned_variant: unknown dtype %d", dtype);
   const int di = dtype == ENS_F32 ? 1 : 0;
+  const bool box = A->tuned_lanes[di][m] > 0 && use_box(A, m, dtype);
   if (lanes) *lanes = A->tuned_lanes[di][m];
-  if (share) *share = dtype == ENS_F32 ? 0 : A->tuned_share[m];
-  if (untiled) *untiled = A->tuned_direct[di][m];  // of the row-by-row launch (row boxes are neither)
+  if (share) *share = dtype == ENS_F32 || box ? 0 : A->tuned_share[m];
+  if (untiled) *untiled = box ? 2 : A->tuned_direct[di][m];
   return ENS_OK;
 }
 

@@ -229,3 +229,27 @@ def test_products_at_the_line_between_both_forms(ens, name, dt, m, off):
     with ens.Matrix.from_operator(op) as A:
         ens.gspmv(A, X, Y)
     _check(ref, X.cpu().numpy(), Y.cpu().numpy(), 1e-12 if dt == torch.float64 else 9 * 2.0**-24)
+
+
+@pytest.mark.parametrize("m,dtype", [(2, "f64"), (8, "f64"), (16, "f32"), (32, "f32")])
+def test_tuned_variant_is_the_launch_in_use(ens, m, dtype):
+    """ens_tuned_variant reports the share that ens_autotune returned and tells row boxes from the two traversals."""
+    import ctypes
+
+    from paper_1711_10622_gb300 import _native as N
+
+    with ens.Matrix.from_operator(gen.channel(128, 64, 64)) as A:
+        def variant():
+            v = [ctypes.c_int32() for _ in range(3)]
+            N.check(N.lib().ens_tuned_variant(A.handle, m, 1 if dtype == "f32" else 0, *(ctypes.byref(x) for x in v)))
+            return [x.value for x in v]
+
+        assert variant()[0] == -1 and variant()[2] == -1
+        t = A.autotune(m, dtype)
+        assert variant() == [t["lanes"], t["share"], 2 if t["boxes"] else int(t["untiled"])]
+        if m in (2, 32):
+            assert not t["boxes"]
+        if m == 8:  # 0.7 times the fastest row-by-row launch
+            assert t["boxes"] and t["share"] == 0
+        A.set_untiled(0)
+        assert variant()[2] in (0, 1)
