@@ -144,9 +144,13 @@ template <typename T, int CW>
 cudaError_t launch_box_cw(const ens_matrix *A, int m, const void *X, void *Y, cudaStream_t s) {
   const uint64_t p = (uint64_t)(uintptr_t)X | (uint64_t)(uintptr_t)Y | (uint64_t)m * sizeof(T);
   constexpr int kWide = CW * sizeof(T) >= 32 ? 32 / sizeof(T) : CW;
-  if (p % (kWide * sizeof(T)) == 0)
-    return m % CW == 0 ? launch_box_acc<T, CW, kWide, true>(A, m, X, Y, s) : launch_box_acc<T, CW, kWide, false>(A, m, X, Y, s);
-  if constexpr (kWide * sizeof(T) == 32)
+  if (p % (kWide * sizeof(T)) == 0) {
+    if constexpr (CW == 16)  // for m = 16 alone
+      return launch_box_acc<T, CW, kWide, true>(A, m, X, Y, s);
+    else
+      return m % CW == 0 ? launch_box_acc<T, CW, kWide, true>(A, m, X, Y, s) : launch_box_acc<T, CW, kWide, false>(A, m, X, Y, s);
+  }
+  if constexpr (kWide * sizeof(T) == 32 && CW != 16)  // (sixteen columns aligned to 8 or 16 bytes go row by row: box_pays)
     if (p % 16 == 0) return launch_box_acc<T, CW, kWide / 2, false>(A, m, X, Y, s);
   return launch_box_acc<T, CW, 1, false>(A, m, X, Y, s);
 }
