@@ -194,7 +194,8 @@ struct BoxShape {
 // aligned. FULL: m is a multiple of CW (checks of the last chunk cost 8-11 % where they are not needed). K0: slots
 // per row where it is known at compile time (0: B.K). ADD64: a float64 sum is widened with one FP64 addition; else
 // in integer arithmetic, which frees the FP64 pipe for an epilogue that needs it (the solver's Chebyshev step 235 ->
-// 212 us on cubes 192 x 128 x 96, m = 8) but costs the plain product 5 %. ahead(row, first column) runs before the
+// 212 us on cubes 192 x 128 x 96, m = 8) but costs the plain product 5 %. (The solver's other kernels take the integer form
+// too; it was not measured for each of them.) ahead(row, first column) runs before the
 // products: the epilogue's own reads can be asked for there.
 template <typename T, int CW, int ACC, bool FULL, int K0, bool INNER, bool ADD64, typename Pre, typename Epi>
 __device__ __forceinline__ void box_rows(const BoxPlan &B, const MatView &A, int32_t m, const T *__restrict__ X, Pre &&ahead, Epi &&epi) {

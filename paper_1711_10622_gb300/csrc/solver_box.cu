@@ -127,6 +127,7 @@ ENS_BOX_KERNEL(T, CW)
   box_reduce<T, 1, CW>(acc, m, partials, counter, [&](int l, const ColTotals<T, 1> &t) { step_alpha<T>(cs, l, t.v[0][l]); });
 }
 
+// (The two sums per column beside the product's own spill 84-96 bytes at eight float64 columns and 48-60 at four.)
 template <typename T, int CW, int K0>
 ENS_BOX_KERNEL(T, CW)
     kb_t(BoxPlan B, MatView A, int32_t m, const T *__restrict__ sh, T *__restrict__ t, const T *__restrict__ s, Cols<T> cs, T *partials,
@@ -166,8 +167,8 @@ ENS_BOX_KERNEL(T, CW)
   box_reduce<T, 1, CW>(acc, m, partials, counter, [&](int l, const ColTotals<T, 1> &t) { residual_norm<T>(cs, l, t.v[0][l], outer); });
 }
 
-// z1 = (1 + c1) z - c1 zp + c2 D^-1 (src - A z): five FP64 operations per element with the widening of A z, on a
-// pipe of two per clock and SM, where the form with the updates d and the running residual took six and moved
+// z1 = (1 + c1) z - c1 zp + c2 D^-1 (src - A z): four FP64 operations per element on a pipe of two per clock and SM (A z
+// is widened in integer arithmetic), where the form with the updates d and the running residual took five and moved
 // six streams instead of four.
 template <typename T, int CW, int K0, bool FIRST>
 ENS_BOX_KERNEL(T, CW)

@@ -82,6 +82,22 @@ def test_coupled_keeps_its_rounding(ens):
     assert np.all(np.linalg.norm(R, axis=0) <= 1.05e-8 * np.linalg.norm(B, axis=0))
 
 
+@pytest.mark.parametrize("m", [4, 8])
+@pytest.mark.parametrize("name", ["cubes97x43x37", "dirichlet48"])
+def test_coupled_with_vcycle_by_boxes(ens, name, m):
+    """The coupled solver with the V-cycle, whose fine level runs by row boxes: several blocks of right-hand sides
+    converge, and the true residuals are what the statuses say."""
+    op = _cubes() if name.startswith("cubes") else gen.dirichlet_box(48)
+    with ens.Matrix.from_operator(op) as A:
+        A.amg_setup()
+        for seed in range(1, 7):
+            B = gen.rhs_normal(op.n, m, seed, zero_mean=op.singular)
+            X, st = ens.solve_block_coupled(A, torch.from_numpy(B).cuda(), tol=1e-8, precond="amg", max_iter=100)
+            assert (st["status"] == 0).all(), (seed, st)
+            R = B - oracle.gspmv(op, X.cpu().numpy())
+            assert np.all(np.linalg.norm(R, axis=0) <= 1.05e-8 * np.linalg.norm(B, axis=0)), seed
+
+
 def test_columns_are_independent(ens):
     """A column's bits do not depend on the other columns, whether these converge, start at zero or are not finite."""
     op = _cubes()
