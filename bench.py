@@ -8,7 +8,8 @@ all inputs resident in HBM. `value` is the sweep's algorithmic HBM throughput:
 summed over the sweep, divided by the device time (CUDA events, max over ranks). Every launch
 moves >= 435 MB, more than the 129 MB L2, so no flush is needed between launches.
 
-Prints one JSON line (rank 0). `--impl reference` times the CPU oracle on the host instead.
+Prints one JSON line (rank 0), short enough to be read back from a log's last lines; `--detail FILE` also writes
+everything that was measured. `--impl reference` times the CPU oracle on the host instead.
 """
 
 from __future__ import annotations
@@ -43,6 +44,56 @@ def alg_bytes(n: int, nnz: int, m: int, sv: int = 8, sx: int = 8) -> int:
 def paper_traffic(n: int, nnz: int, m: int) -> float:
     """Sigma_m of Section 2.3 (X re-read for every nonzero)."""
     return 4.0 * n * (2 * m + 1) + 12.0 * nnz + 8.0 * m * nnz
+
+
+# What the printed line keeps of each measured entry, by section; sections not named here are printed whole.
+LINE_KEYS = {
+    "sweep": ("us", "gbs", "frac_of_measured_peak"),
+    "cusparse_spmm": ("ours_speedup",),
+    "cubes_gspmv": ("workload", "us"),
+    "projection": ("workload", "m", "us"),
+    "solves": ("solves_per_s", "max_rel_err_vs_oracle"),
+    "batch": ("precond", "precision", "tol", "rhs", "rhs_solves_per_s", "speedup_vs_one_rhs"),
+    "serving": ("p50_ms", "p99_ms", "wait_p99_ms", "capacity_requests_per_s", "converged_all"),
+    "oracle_references": (),
+    "cpu_baseline": ("value", "unit", "cores", "kind", "sample"),
+    "paper_estimate": (),
+}
+
+
+def short_line(record: dict) -> dict:
+    """The record as it is printed: of the sections in LINE_KEYS only these keys (at any depth), measured numbers beside
+    the contract's to four digits. Lines of 24 KB did not come through the logs that the bench is read from."""
+
+    def pick(x, keys):
+        if not isinstance(x, dict):
+            return None
+        out = {}
+        for k, v in x.items():
+            if k in keys and not isinstance(v, (dict, list)):
+                out[k] = v
+            elif isinstance(v, dict):
+                inner = pick(v, keys)
+                if inner:
+                    out[k] = inner
+        return out
+
+    def rounded(x):
+        if isinstance(x, float):
+            return float("%.4g" % x)
+        if isinstance(x, dict):
+            return {k: rounded(v) for k, v in x.items()}
+        return [rounded(v) for v in x] if isinstance(x, list) else x
+
+    line = {}
+    for k, v in record.items():
+        if k in LINE_KEYS:
+            v = pick(v, LINE_KEYS[k])
+            if v:
+                line[k] = rounded(v)
+        else:
+            line[k] = v
+    return line
 
 
 def hbm_peak():
@@ -1104,6 +1155,7 @@ def main():
     ap.add_argument("--warmup", type=int, default=5)
     ap.add_argument("--impl", default="ours", choices=["ours", "reference"])
     ap.add_argument("--f64-mode", default="auto", choices=["auto", "native", "split"])
+    ap.add_argument("--detail", default=None, metavar="FILE", help="write everything that was measured to this JSON file")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-solves", action="store_true", help="skip the solve-throughput section")
     ap.add_argument("--serving-requests", type=int, default=2000, help="requests of the serving stream (0: skip)")
@@ -1359,7 +1411,10 @@ def main():
             "clocks": clocks,
             "gpu_launches": K * len(M_SWEEP),
         }
-        print(json.dumps(line))
+        if args.detail:
+            with open(args.detail, "w") as f:
+                json.dump(line, f, indent=1)
+        print(json.dumps(short_line(line)))
     A.close()
     if dist is not None:
         dist.destroy_process_group()
