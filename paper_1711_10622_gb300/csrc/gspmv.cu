@@ -168,25 +168,30 @@ int pow2_at_least(int v, int cap) {
 //     12 0.91 and 20 0.90 times;
 //     float32, aligned to 16, m = 16 1.03, 24 1.12);
 //   * in float64 from m = 16 on where the rounds of boxes per resident block take 1.3 times the rows there are (bricks cut
-//     off by the grid, a last round that is nearly empty: 112640 rows in 440 boxes, m = 16 1.04 times, 32 1.10, 64 1.19;
-//     85000 rows in 630 boxes 1.06, 1.10, 1.15; 221184 rows at 1.4 times 1.00; 331776 rows at 1.06 times 0.8-0.9). Not
-//     asked where the autotuner has timed both.
-// float32 blocks of four columns below 2^17 rows take one latency either way, by boxes 17 us against 16.
+//     off by the grid, a last round that is nearly empty; back to back 112640 rows in 440 boxes m = 16 1.12 times, 32 1.13,
+//     64 1.14; 155648 rows in 1024 boxes 1.17, 1.21, 1.21; 221184 rows at 1.4 times 1.00; at 1.06 times 0.93-0.96). Below 400
+//     row tiles the row-by-row launch's last round is as empty (92160 rows in 360 boxes 0.93, 0.95, 0.98): there only where
+//     cut bricks alone make it 1.35 times (85140 rows in 495 boxes 1.15, 1.18, 1.21; 81807 in 400 0.92-0.96). Not asked where
+//     the autotuner has timed both.
+// float32, m = 14 on seven-point rows: 1.03 times on 2.1 million rows, 1.08 to 1.27 with cut bricks, else 0.9.
 bool box_pays(const ens_matrix *A, int m, int dtype, const void *X, const void *Y) {
   const bool f32 = dtype == ENS_F32;
   const uint64_t p = (uint64_t)(uintptr_t)X | (uint64_t)(uintptr_t)Y | (uint64_t)m * (f32 ? 4 : 8);
   const int tile = pow2_at_least(m, 32);  // columns of a row-by-row tile
-  const double full = (double)m / ((m + tile - 1) / tile * tile);
-  const bool timed = m <= kTuneMaxM && A->tuned_lanes[f32 ? 1 : 0][m] > 0;
+  const double full = (double)m / ((m + tile - 1) / tile * tile), rows = (double)A->n;
+  const int64_t boxes = A->box.boxes;
   if (f32) {
-    if (m == 4 && A->n < (1 << 17) && !timed) return false;
-    return p % 32 == 0 || p % 8 != 0 || m < (A->box.K == 7 ? 14 : 16) || full < 0.75;
+    if (p % 32 == 0 || p % 8 != 0 || m < 14 || full < 0.75) return true;
+    return m == 14 && (A->box.K != 7 || (A->n < (1 << 20) && boxes * kBoxRows <= 1.05 * rows));
   }
   if (m < 16 || m % 4 != 0 || full < 0.875) return true;
   if (p % 32 != 0 && p % 16 == 0) return false;
-  const int64_t round = A->num_sms * (int64_t)BoxShape<double, 8>::kBlocks, slots = (A->box.boxes + round - 1) / round * round;
-  return timed || p % 16 != 0 || 10 * slots * kBoxRows < 13 * A->n;
+  const bool timed = m <= kTuneMaxM && A->tuned_lanes[0][m] > 0;
+  if (timed || p % 16 != 0) return true;
+  const int64_t round = A->num_sms * (int64_t)BoxShape<double, 8>::kBlocks, slots = (boxes + round - 1) / round * round;
+  return slots * kBoxRows < 1.3 * rows || (A->n < 400 * kTileRows && boxes * kBoxRows < 1.35 * rows);
 }
+
 cudaError_t launch_box(const ens_matrix *A, int m, int dtype, const void *X, void *Y, cudaStream_t s) {
   if (dtype == ENS_F32) {
     if (m <= 4) return launch_box_cw<float, 4>(A, m, X, Y, s);
