@@ -36,12 +36,12 @@ MatView view_of(const ens_matrix *A) {
 }
 
 // Tiled GSpMV: CSR segments staged in shared memory (tile_rows), Y written with streaming stores.
-template <typename Arith, int VEC, int LANES>
+template <typename Arith, int VEC, int LANES, int R0 = 0>
 __device__ __forceinline__ void gspmv_body(const MatView &A, int32_t m, const typename Arith::T *__restrict__ X,
                                            typename Arith::T *__restrict__ Y, uint32_t native_mask) {
   using T = typename Arith::T;
-  tile_rows<Arith, VEC, LANES>(A, m, X, native_mask,
-                               [&](int64_t i, int32_t c, const T (&y)[VEC]) { store_vec_cs<T, VEC>(Y + i * m + c, y); });
+  tile_rows<Arith, VEC, LANES, R0>(A, m, X, native_mask,
+                                   [&](int64_t i, int32_t c, const T (&y)[VEC]) { store_vec_cs<T, VEC>(Y + i * m + c, y); });
 }
 
 template <typename Arith, int VEC, int LANES>
@@ -66,11 +66,14 @@ template <typename Arith, int VEC>
 struct MinBlocks {
   static constexpr int value = std::is_same<Arith, ArithF32>::value ? 8 : VEC == 4 ? 5 : 6;
 };
-template <typename Arith, int VEC, int LANES>
+// R0: rows of a tile where they are known at compile time (0: by the rows of the product, tile_rows_for). At 32 registers
+// the float32 kernels spill 40-72 bytes with a tile height of their own (two columns per lane, and four with two lanes
+// per row: m = 8 6.4 us against 5.5 on 127872 rows), so whole tiles have instances of theirs.
+template <typename Arith, int VEC, int LANES, int R0 = 0>
 __global__ void __launch_bounds__(kThreads, MinBlocks<Arith, VEC>::value)
     gspmv_kernel_capped(MatView A, int32_t m, const typename Arith::T *__restrict__ X,
                         typename Arith::T *__restrict__ Y, uint32_t native_mask) {
-  gspmv_body<Arith, VEC, LANES>(A, m, X, Y, native_mask);
+  gspmv_body<Arith, VEC, LANES, R0>(A, m, X, Y, native_mask);
 }
 
 // Untiled variant (direct_rows): an autotuner candidate beside the tiled kernels.
@@ -230,6 +233,13 @@ cudaError_t run(const ens_matrix *A, int m, const void *X, void *Y, uint32_t mas
       return cudaGetLastError();
     }
   }
+  if constexpr (std::is_same<Arith, ArithF32>::value && LANES > 1 && (VEC == 2 || (VEC == 4 && LANES == 2)))
+    if (tile_rows_for(v.n, LANES) == kTileRows) {
+      auto k = gspmv_kernel_capped<Arith, VEC, LANES, kTileRows>;
+      static std::atomic<int> known{0};
+      k<<<grid_for(A, v.n, resident(known, (const void *)k, kThreads, 0), kTileRows), kThreads, 0, s>>>(v, m, (const T *)X, y, mask);
+      return cudaGetLastError();
+    }
   if constexpr (capped) {
     auto k = gspmv_kernel_capped<Arith, VEC, LANES>;
     static std::atomic<int> known{0};

@@ -821,13 +821,13 @@ __device__ __forceinline__ void tile_order_rows(int64_t n, int32_t m, Fn &&fn) {
   }
 }
 
-template <typename Arith, int VEC, int LANES, typename Epi>
+template <typename Arith, int VEC, int LANES, int R0 = 0, typename Epi>
 __device__ __forceinline__ void tile_rows(const MatView &A, int32_t m, const typename Arith::T *__restrict__ X,
                                           uint32_t native_mask, Epi &&epi) {
   using T = typename Arith::T;
   constexpr int kThr = 256;
   constexpr int G = kThr / LANES;
-  const int R = tile_rows_for(A.n, LANES), RPG = R / G;
+  const int R = R0 ? R0 : tile_rows_for(A.n, LANES), RPG = R / G;
   // Row pointers of the current tile and of the next one: the next tile's are copied asynchronously
   // while the current tile is computed, so each tile waits for one memory round trip (its CSR
   // segment) instead of two (row pointers, then the segment they delimit). Measured on GB300:
