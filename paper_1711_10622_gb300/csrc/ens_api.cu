@@ -248,7 +248,8 @@ static ens_status create_matrix_impl(int64_t n, int64_t ncols, int64_t nnz, cons
     const int64_t count = (n + per - 1) / per;
     for (int64_t k = 0; k < count; ++k) A->pipe_row.push_back(k * per);
     A->pipe_mask.assign((size_t)count * kPipeMaskWords, 0);
-    host_parallel(count, nnz > (1 << 20) ? 1 : count, [&](int64_t k0, int64_t k1) {  // whole chunks: no two threads share a mask
+    // whole chunks: no two threads share a mask; four threads beside the planner's where one would take longer than it
+    host_parallel(count, nnz > (1 << 20) ? 1 : nnz > (1 << 18) ? 4 : count, [&](int64_t k0, int64_t k1) {
       for (int64_t k = k0; k < k1; ++k) {
         uint64_t *mask = A->pipe_mask.data() + k * kPipeMaskWords;
         const int64_t r1 = std::min<int64_t>(n, (k + 1) * per);
