@@ -150,6 +150,22 @@ def test_float32_cycle_error(ens, name):
     assert err[1] <= 1.15 * err[0], err
 
 
+def test_float32_small_level_error(ens):
+    """The float32 cycle with four threads per row (m = 8) is about as close to the float64 one as with two (m = 16): 1.04
+    times; 1.14 while each thread's first product was rounded on its own."""
+    op = gen.channel(32, 32, 32)
+    err = np.zeros(2)
+    with ens.Matrix.from_operator(op) as A:
+        A.amg_setup()
+        for seed in range(24):
+            R = torch.randn(op.n, 16, device="cuda", generator=torch.Generator(device="cuda").manual_seed(seed))
+            Z = ens.amg_apply(A, R.double())[:, :8]
+            for k, m in enumerate((16, 8)):
+                E = ens.amg_apply(A, R[:, :m].contiguous()).double()[:, :8] - Z
+                err[k] += float((E.norm(dim=0) / Z.norm(dim=0)).square().sum())
+    assert np.sqrt(err[1] / err[0]) <= 1.09, err
+
+
 @pytest.mark.parametrize("m", [1, 2, 5, 8, 33, 64])
 @pytest.mark.parametrize("nx,opts", [
     (45, dict(coarse_size=512, coarse_steps=16)),  # dense coarsest level
